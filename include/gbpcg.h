@@ -249,6 +249,12 @@ int gbpcg_workspace_size(const gbpcg_grid *grid, const gbpcg_opts *opts, size_t 
  * near 1 when it is far from 1: any scale of b that FP64 can hold converges
  * alike (a solve of 2^k b returns 2^k times the solution of b, bit for bit).
  *
+ * A constant-coefficient problem with nx >= 8 whose residual fits the GPU's
+ * registers and whose search direction fits its shared memory (up to about
+ * four million points) is solved in one cooperative launch that keeps both
+ * there; others, and calls with tile_cfg or GBPCG_FLAG_PROFILE, run the data
+ * passes from a device-driven CUDA graph.
+ *
  * Mixed precision (opts->storage BF16 or F16, FP64 b and x): iterative
  * refinement.  Each outer step computes r = b - A x in FP64 and stops when
  * ||r||/||b|| <= tol; otherwise it solves the scaled correction equation
@@ -260,7 +266,7 @@ int gbpcg_workspace_size(const gbpcg_grid *grid, const gbpcg_opts *opts, size_t 
  * guess in, solution out) hold nx*ny*nz elements of opts->io_dtype; they are
  * DEVICE pointers, or HOST pointers when opts->flags has GBPCG_FLAG_HOST_IO
  * (then they are copied through the workspace inside the call).  The whole
- * iteration runs on the device inside one CUDA graph (no per-iteration host
+ * iteration runs on the device (no per-iteration host
  * round trip; compare the paper's FP32 variant, which reads the norm back
  * every iteration).  Stops when ||r||/||b|| <= tol or after maxit
  * iterations; b = 0 gives x = 0.  Fills *result (host memory) and returns
@@ -277,7 +283,11 @@ int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_
  * (gbpcg_workspace_size_batched) holds every problem's scratch.  Returns
  * GBPCG_OK when all problems converged, else the first other status.
  *
- * Up to 4096 constant-coefficient grids with nx a multiple of 4 (and at most
+ * With tile_cfg 0, constant-coefficient grids that fit the chip are solved
+ * there (see gbpcg_pcg_solve) where that is estimated to be faster: those of
+ * up to 400,000 points side by side in one cooperative launch, larger ones
+ * one after another.  The rest streams: up to
+ * 4096 constant-coefficient grids with nx a multiple of 4 (and at most
  * 4096 tiles each) run as ONE persistent
  * kernel (a cooperative launch of as many CTAs as the GPU holds, inside a
  * cached one-node CUDA graph): every problem runs its own sequence of phases
@@ -287,14 +297,17 @@ int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_
  * completes a phase takes the problem's scalar step and opens its next
  * phase.  Setup and finalize are phases of all problems at once between
  * grid barriers.  Every wait is bounded: if one gives up, the unfinished
- * problems report GBPCG_TIMEOUT.  result.pass_launches = {1, phases run
+ * problems report GBPCG_TIMEOUT.  result.pass_launches = {launches
+ * of solver kernels (1 for a batch that runs one way), phases run
  * over all problems (2 per iteration and 2 per replacement)},
  * pass_ctas[0] = the tile configuration (0: 64x16, 1: 128x8, 2: 32x32):
  * opts->tile_cfg = c + 1 selects configuration c, else
  * GBPCG_FLAG_AUTOTUNE times the three and keeps the fastest per set of
  * shapes, else 64x16.  Otherwise (block coefficients, or GBPCG_FLAG_BATCH_GRAPH) each
  * problem's whole solve is a branch of one CUDA graph with its own
- * device-driven loop, tiles per shape from the autotuner.
+ * device-driven loop, tiles per shape from the autotuner (with
+ * GBPCG_FLAG_BATCH_GRAPH, grids that fit the chip are solved one after
+ * another as gbpcg_pcg_solve would, bit for bit).
  */
 int gbpcg_workspace_size_batched(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts *opts,
                                  size_t *bytes);

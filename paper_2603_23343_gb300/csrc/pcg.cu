@@ -18,6 +18,7 @@
 #include <tuple>
 #include <vector>
 
+#include "resident.cuh"
 #include "solver.cuh"
 
 namespace gb {
@@ -583,6 +584,62 @@ static int persistent_batch(int nprob, const gbpcg_grid *grids, const void *cons
     return worst;
 }
 
+// The problems of a batch that fit the chip, solved there (resident.cu): one launch for all that leave
+// room for others beside them (bitwise the same from run to run), and one launch each for the larger
+// ones and, with GBPCG_FLAG_BATCH_GRAPH, for all (bitwise the standalone solves).  `in_batch` and
+// `alone` hold their numbers; fills their results.
+static int resident_batch(const std::vector<int> &in_batch, const std::vector<int> &alone, const gbpcg_grid *grids,
+                          const void *const *b, void *const *x, const gbpcg_opts *opts, gbpcg_result *results, char *ws,
+                          size_t region, const std::vector<WsLayout> &L, const std::vector<size_t> &off,
+                          cudaStream_t s) {
+    const int nb = (int)in_batch.size(), n = nb + (int)alone.size();
+    auto which = [&](int i) { return i < nb ? in_batch[i] : alone[i - nb]; };
+    std::vector<SolveCall> calls(n);
+    for (int i = 0; i < n; ++i) {
+        const int p = which(i);
+        calls[i] = SolveCall{&grids[p], 0, 0, b[p], x[p], ws + off[p], L[p], opts->tol, opts->maxit, opts->io_dtype,
+                             1.0f, nullptr};
+    }
+    SolveState *states = reinterpret_cast<SolveState *>(ws);
+    const size_t state_bytes = round256((size_t)n * sizeof(SolveState));
+    if (state_bytes > region) return kResNoRoom;
+    cudaEvent_t e0, e1;
+    GB_CUDA(cudaEventCreate(&e0));
+    GB_CUDA(cudaEventCreate(&e1));
+    struct Ev { cudaEvent_t a, b; ~Ev() { cudaEventDestroy(a); cudaEventDestroy(b); } } guard{e0, e1};
+    GB_CUDA(cudaEventRecord(e0, s));
+    if (nb) {
+        if (int rc = resident_batch_launch(nb, calls.data(), states, ws + state_bytes, region - state_bytes,
+                                           opts->io_dtype, s))
+            return rc;
+    }
+    for (int i = nb; i < n; ++i) {
+        ResPlan plan;
+        resident_fits(*calls[i].g, &plan);
+        if (int rc = resident_launch(calls[i], plan, s, states + i)) return rc;
+    }
+    GB_CUDA(cudaEventRecord(e1, s));
+    std::vector<SolveState> hs(n);
+    GB_CUDA(cudaMemcpyAsync(hs.data(), states, (size_t)n * sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaStreamSynchronize(s));
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    for (int i = 0; i < n; ++i) {
+        gbpcg_result &r = results[which(i)];
+        memset(&r, 0, sizeof(r));
+        r.iters = hs[i].it;
+        r.status = hs[i].done ? hs[i].status : GBPCG_TIMEOUT;
+        r.rel_res_recursive = hs[i].bb > 0 ? sqrt(hs[i].rr / hs[i].bb) : 0.0;
+        r.rel_res_true = hs[i].bb_true > 0 ? sqrt(hs[i].rr_true / hs[i].bb_true) : 0.0;
+        r.time_ms = ms;
+        r.replacements = hs[i].n_replace;
+        r.pass_launches[0] = (nb ? 1 : 0) + (n - nb);
+        r.pass_launches[1] = 2 * (hs[i].it + hs[i].n_replace);
+        if (r.status == GBPCG_TIMEOUT) set_error("a bounded device wait timed out during a batched solve");
+    }
+    return GBPCG_OK;
+}
+
 static int check_batch(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts *opts) {
     if (nprob <= 0 || nprob > 4096) return fail_arg("nprob must be in 1..4096");
     if (!grids) return fail_arg("grids is NULL");
@@ -595,183 +652,11 @@ static int check_batch(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts 
     return GBPCG_OK;
 }
 
-}  // namespace gb
-
-using namespace gb;
-
-extern "C" {
-
-int gbpcg_tile_config(int32_t index, int32_t *tx, int32_t *ty, int32_t *stages) {
-    clear_error();
-    if (index < 0 || index >= NUM_CFG) return fail_arg("tile configuration index out of range");
-    const CfgDims d = cfg_dims(index);
-    if (tx) *tx = d.tx;
-    if (ty) *ty = d.ty;
-    if (stages) *stages = d.s;
-    return GBPCG_OK;
-}
-
-int gbpcg_workspace_size(const gbpcg_grid *grid, const gbpcg_opts *opts, size_t *bytes) {
-    clear_error();
-    if (int rc = check_grid(grid)) return rc;
-    if (int rc = check_opts(opts)) return rc;
-    if (!bytes) return fail_arg("bytes is NULL");
-    *bytes = workspace_total(*grid, *opts);
-    return GBPCG_OK;
-}
-
-int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_opts *opts, gbpcg_result *result,
-                    gbpcg_stream stream) {
-    NvtxRange range("gbpcg_pcg_solve");
-    clear_error();
-    if (int rc = check_grid(grid)) return rc;
-    if (int rc = check_opts(opts)) return rc;
-    if (!b || !x || !result) return fail_arg("b, x and result must be non-NULL");
-    memset(result, 0, sizeof(*result));
-    const size_t total = workspace_total(*grid, *opts);
-    if (!opts->workspace || opts->workspace_bytes < total) return fail_arg("workspace smaller than gbpcg_workspace_size()");
-    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    char *ws = static_cast<char *>(opts->workspace);
-    const gbpcg_grid g = *grid;
-    const int64_t n = (int64_t)g.nx * g.ny * g.nz;
-    const size_t esz = dtype_size(opts->io_dtype);
-    const size_t io_bytes = (size_t)n * esz;
-    if ((reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(x)) & (esz - 1))
-        return fail_arg("b and x must be aligned to their element size");
-    int cfg_a = 0, cfg_b = 0;
-    pick_cfgs(g, *opts, &cfg_a, &cfg_b);
-    if (!cfg_fits(cfg_a, g.nx) || !cfg_fits(cfg_b, g.nx))
-        return fail_arg("tile_cfg selects a whole-row configuration for a grid wider than 256");
-
-    // host buffers are staged through the end of the workspace
-    const bool host_io = opts->flags & GBPCG_FLAG_HOST_IO;
-    const bool b_host = host_io && !is_device_ptr(b);
-    const bool x_host = host_io && !is_device_ptr(x);
-    char *stage = ws + total - (host_io ? 2 * round256(io_bytes) : 0);
-    const void *bd = b_host ? static_cast<const void *>(stage) : b;
-    void *xd = x_host ? static_cast<void *>(stage + round256(io_bytes)) : x;
-    if (b_host) GB_CUDA(cudaMemcpyAsync(const_cast<void *>(bd), b, io_bytes, cudaMemcpyHostToDevice, s));
-    if (x_host) GB_CUDA(cudaMemcpyAsync(xd, x, io_bytes, cudaMemcpyHostToDevice, s));
-
-    if (refine_mode(*opts)) {
-        const RefineLayout R = refine_layout(g, *opts);
-        const bool tma = tma_ok(dtype_size(opts->storage), g.nx,
-                                {ws + R.inner + R.in.z, ws + R.inner + R.in.p0, ws + R.inner + R.in.p1,
-                                 ws + R.inner + R.in.d});
-        int rc = refine_solve(g, static_cast<const double *>(bd), static_cast<double *>(xd), opts, ws, R, cfg_a, cfg_b,
-                              tma, result, s);
-        if (x_host) {
-            GB_CUDA(cudaMemcpyAsync(x, xd, io_bytes, cudaMemcpyDeviceToHost, s));
-            GB_CUDA(cudaStreamSynchronize(s));
-        }
-        return rc;
-    }
-
-    if (opts->flags & GBPCG_FLAG_SPLIT) {
-        if (g.k_block) return fail_arg("SPLIT takes the constant-coefficient operator");
-        return split_solve(g, static_cast<const float *>(b), static_cast<float *>(x), *opts, result, s);
-    }
-
-    const WsLayout L = ws_layout_n((size_t)n, opts->storage, opts->io_dtype, false, block_count(g));
-    const bool tma = tma_ok(sizeof(float), g.nx, {ws + L.z, ws + L.p0, ws + L.p1, ws + L.d});
-    const SolveCall call{&g, cfg_a, cfg_b, bd, xd, ws, L, opts->tol, opts->maxit, opts->io_dtype, 1.0f, nullptr};
-    const SolveState *st = reinterpret_cast<const SolveState *>(ws + L.state);
-    cudaEvent_t e0, e1;
-    GB_CUDA(cudaEventCreate(&e0));
-    GB_CUDA(cudaEventCreate(&e1));
-    GB_CUDA(cudaEventRecord(e0, s));
-    const int rc = (opts->flags & GBPCG_FLAG_PROFILE)     ? solve_profiled<float>(call, tma, result, s)
-                   : (opts->flags & GBPCG_FLAG_HOST_LOOP) ? solve_host_loop<float>(call, tma, s)
-                                                          : solve_launch<float>(call, tma, s);
-    if (rc) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return rc;
-    }
-    GB_CUDA(cudaEventRecord(e1, s));
-    return finish_solve(st, x, xd, x_host, io_bytes, e0, e1, result, s);
-}
-
-int gbpcg_autotune(const gbpcg_grid *grid, const gbpcg_opts *opts, const void *b, int32_t *tile_cfg,
-                   double *us_per_iter, gbpcg_stream stream) {
-    NvtxRange range("gbpcg_autotune");
-    clear_error();
-    if (int rc = check_grid(grid)) return rc;
-    if (int rc = check_opts(opts)) return rc;
-    if (!b || !tile_cfg) return fail_arg("b and tile_cfg must be non-NULL");
-    if (opts->storage != GBPCG_F32) return fail_arg("the autotuner times F32 storage");
-    gbpcg_opts o = *opts;
-    o.flags |= GBPCG_FLAG_AUTOTUNE;
-    WsLayout L;
-    const size_t need = batch_piece(*grid, o, &L);
-    if (!opts->workspace || opts->workspace_bytes < need)
-        return fail_arg("workspace smaller than gbpcg_workspace_size() with GBPCG_FLAG_AUTOTUNE");
-    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
-    char *ws = static_cast<char *>(opts->workspace);
-    int code = 0;
-    if (int rc = autotune_one(*grid, o, b, ws + L.total, ws, L, reinterpret_cast<cudaStream_t>(stream), &code,
-                              us_per_iter))
-        return rc;
-    *tile_cfg = code;
-    return GBPCG_OK;
-}
-
-int gbpcg_autotune_record(const gbpcg_grid *grid, const gbpcg_opts *opts, int32_t tile_cfg) {
-    clear_error();
-    if (int rc = check_grid(grid)) return rc;
-    if (int rc = check_opts(opts)) return rc;
-    gbpcg_opts o = *opts;
-    o.tile_cfg = tile_cfg;
-    if (int rc = check_opts(&o)) return rc;
-    if (!tile_cfg) return fail_arg("tile_cfg 0 is not a configuration");
-    int ca = 0, cb = 0;
-    pick_cfgs(*grid, o, &ca, &cb);
-    if (!cfg_fits(ca, grid->nx) || !cfg_fits(cb, grid->nx)) return fail_arg("configuration does not fit the grid");
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[tune_key(*grid, *opts)] = tile_cfg;
-    return GBPCG_OK;
-}
-
-int gbpcg_workspace_size_batched(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts *opts, size_t *bytes) {
-    clear_error();
-    if (int rc = check_batch(nprob, grids, opts)) return rc;
-    if (!bytes) return fail_arg("bytes is NULL");
-    size_t total = round256(batch_persistent_bytes(nprob, grids));  // the persistent kernel's tables
-    for (int i = 0; i < nprob; ++i) {
-        WsLayout L;
-        total += batch_piece(grids[i], *opts, &L);
-    }
-    *bytes = total;
-    return GBPCG_OK;
-}
-
-int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *const *b, void *const *x,
-                            const gbpcg_opts *opts, gbpcg_result *results, gbpcg_stream stream) {
-    NvtxRange range("gbpcg_pcg_solve_batched");
-    clear_error();
-    if (int rc = check_batch(nprob, grids, opts)) return rc;
-    if (!b || !x || !results) return fail_arg("b, x and results must be non-NULL");
-    const size_t esz = dtype_size(opts->io_dtype);
-    for (int i = 0; i < nprob; ++i) {
-        if (!b[i] || !x[i]) return fail_arg("every b[i] and x[i] must be a device pointer");
-        if ((reinterpret_cast<uintptr_t>(b[i]) | reinterpret_cast<uintptr_t>(x[i])) & (esz - 1))
-            return fail_arg("b[i] and x[i] must be aligned to their element size");
-    }
-    const size_t region = round256(batch_persistent_bytes(nprob, grids));
-    size_t need = region;
-    std::vector<WsLayout> L(nprob);
-    std::vector<size_t> off(nprob);
-    for (int i = 0; i < nprob; ++i) {
-        off[i] = need;
-        need += batch_piece(grids[i], *opts, &L[i]);
-    }
-    if (!opts->workspace || opts->workspace_bytes < need)
-        return fail_arg("workspace smaller than gbpcg_workspace_size_batched()");
-    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    char *ws = static_cast<char *>(opts->workspace);
-
+// The problems in the streaming kernels: one persistent kernel where it takes them (batch.cu), else
+// (block coefficients, unaligned rows, GBPCG_FLAG_BATCH_GRAPH) one CUDA graph with a branch per problem.
+static int streamed_batch(int nprob, const gbpcg_grid *grids, const void *const *b, void *const *x,
+                          const gbpcg_opts *opts, gbpcg_result *results, char *ws, const std::vector<WsLayout> &L,
+                          const std::vector<size_t> &off, cudaStream_t s) {
     if (!(opts->flags & GBPCG_FLAG_BATCH_GRAPH) && batch_persistent_ok(nprob, grids))
         return persistent_batch(nprob, grids, b, x, opts, results, ws, L, off, s);
 
@@ -867,6 +752,251 @@ int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *
         if (r.status != GBPCG_OK && worst == GBPCG_OK) worst = r.status;
     }
     return worst;
+}
+
+}  // namespace gb
+
+using namespace gb;
+
+extern "C" {
+
+int gbpcg_tile_config(int32_t index, int32_t *tx, int32_t *ty, int32_t *stages) {
+    clear_error();
+    if (index < 0 || index >= NUM_CFG) return fail_arg("tile configuration index out of range");
+    const CfgDims d = cfg_dims(index);
+    if (tx) *tx = d.tx;
+    if (ty) *ty = d.ty;
+    if (stages) *stages = d.s;
+    return GBPCG_OK;
+}
+
+int gbpcg_workspace_size(const gbpcg_grid *grid, const gbpcg_opts *opts, size_t *bytes) {
+    clear_error();
+    if (int rc = check_grid(grid)) return rc;
+    if (int rc = check_opts(opts)) return rc;
+    if (!bytes) return fail_arg("bytes is NULL");
+    *bytes = workspace_total(*grid, *opts);
+    return GBPCG_OK;
+}
+
+int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_opts *opts, gbpcg_result *result,
+                    gbpcg_stream stream) {
+    NvtxRange range("gbpcg_pcg_solve");
+    clear_error();
+    if (int rc = check_grid(grid)) return rc;
+    if (int rc = check_opts(opts)) return rc;
+    if (!b || !x || !result) return fail_arg("b, x and result must be non-NULL");
+    memset(result, 0, sizeof(*result));
+    const size_t total = workspace_total(*grid, *opts);
+    if (!opts->workspace || opts->workspace_bytes < total) return fail_arg("workspace smaller than gbpcg_workspace_size()");
+    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    char *ws = static_cast<char *>(opts->workspace);
+    const gbpcg_grid g = *grid;
+    const int64_t n = (int64_t)g.nx * g.ny * g.nz;
+    const size_t esz = dtype_size(opts->io_dtype);
+    const size_t io_bytes = (size_t)n * esz;
+    if ((reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(x)) & (esz - 1))
+        return fail_arg("b and x must be aligned to their element size");
+    int cfg_a = 0, cfg_b = 0;
+    pick_cfgs(g, *opts, &cfg_a, &cfg_b);
+    if (!cfg_fits(cfg_a, g.nx) || !cfg_fits(cfg_b, g.nx))
+        return fail_arg("tile_cfg selects a whole-row configuration for a grid wider than 256");
+
+    // host buffers are staged through the end of the workspace
+    const bool host_io = opts->flags & GBPCG_FLAG_HOST_IO;
+    const bool b_host = host_io && !is_device_ptr(b);
+    const bool x_host = host_io && !is_device_ptr(x);
+    char *stage = ws + total - (host_io ? 2 * round256(io_bytes) : 0);
+    const void *bd = b_host ? static_cast<const void *>(stage) : b;
+    void *xd = x_host ? static_cast<void *>(stage + round256(io_bytes)) : x;
+    if (b_host) GB_CUDA(cudaMemcpyAsync(const_cast<void *>(bd), b, io_bytes, cudaMemcpyHostToDevice, s));
+    if (x_host) GB_CUDA(cudaMemcpyAsync(xd, x, io_bytes, cudaMemcpyHostToDevice, s));
+
+    if (refine_mode(*opts)) {
+        const RefineLayout R = refine_layout(g, *opts);
+        const bool tma = tma_ok(dtype_size(opts->storage), g.nx,
+                                {ws + R.inner + R.in.z, ws + R.inner + R.in.p0, ws + R.inner + R.in.p1,
+                                 ws + R.inner + R.in.d});
+        int rc = refine_solve(g, static_cast<const double *>(bd), static_cast<double *>(xd), opts, ws, R, cfg_a, cfg_b,
+                              tma, result, s);
+        if (x_host) {
+            GB_CUDA(cudaMemcpyAsync(x, xd, io_bytes, cudaMemcpyDeviceToHost, s));
+            GB_CUDA(cudaStreamSynchronize(s));
+        }
+        return rc;
+    }
+
+    if (opts->flags & GBPCG_FLAG_SPLIT) {
+        if (g.k_block) return fail_arg("SPLIT takes the constant-coefficient operator");
+        return split_solve(g, static_cast<const float *>(b), static_cast<float *>(x), *opts, result, s);
+    }
+
+    const WsLayout L = ws_layout_n((size_t)n, opts->storage, opts->io_dtype, false, block_count(g));
+    const bool tma = tma_ok(sizeof(float), g.nx, {ws + L.z, ws + L.p0, ws + L.p1, ws + L.d});
+    const SolveCall call{&g, cfg_a, cfg_b, bd, xd, ws, L, opts->tol, opts->maxit, opts->io_dtype, 1.0f, nullptr};
+    const SolveState *st = reinterpret_cast<const SolveState *>(ws + L.state);
+    cudaEvent_t e0, e1;
+    GB_CUDA(cudaEventCreate(&e0));
+    GB_CUDA(cudaEventCreate(&e1));
+    GB_CUDA(cudaEventRecord(e0, s));
+    // a problem that fits the chip is solved there (resident.cu) unless tiles or pass times were asked for
+    ResPlan plan;
+    const bool resident = !opts->tile_cfg && !(opts->flags & GBPCG_FLAG_PROFILE) && resident_fits(g, &plan);
+    const bool host_loop = opts->flags & GBPCG_FLAG_HOST_LOOP;
+    const int rc = (opts->flags & GBPCG_FLAG_PROFILE) ? solve_profiled<float>(call, tma, result, s)
+                   : resident && host_loop            ? resident_host_loop(call, plan, s)
+                   : resident                         ? resident_launch(call, plan, s)
+                   : host_loop                        ? solve_host_loop<float>(call, tma, s)
+                                                      : solve_launch<float>(call, tma, s);
+    if (rc) {
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return rc;
+    }
+    GB_CUDA(cudaEventRecord(e1, s));
+    return finish_solve(st, x, xd, x_host, io_bytes, e0, e1, result, s);
+}
+
+int gbpcg_autotune(const gbpcg_grid *grid, const gbpcg_opts *opts, const void *b, int32_t *tile_cfg,
+                   double *us_per_iter, gbpcg_stream stream) {
+    NvtxRange range("gbpcg_autotune");
+    clear_error();
+    if (int rc = check_grid(grid)) return rc;
+    if (int rc = check_opts(opts)) return rc;
+    if (!b || !tile_cfg) return fail_arg("b and tile_cfg must be non-NULL");
+    if (opts->storage != GBPCG_F32) return fail_arg("the autotuner times F32 storage");
+    gbpcg_opts o = *opts;
+    o.flags |= GBPCG_FLAG_AUTOTUNE;
+    WsLayout L;
+    const size_t need = batch_piece(*grid, o, &L);
+    if (!opts->workspace || opts->workspace_bytes < need)
+        return fail_arg("workspace smaller than gbpcg_workspace_size() with GBPCG_FLAG_AUTOTUNE");
+    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
+    char *ws = static_cast<char *>(opts->workspace);
+    int code = 0;
+    if (int rc = autotune_one(*grid, o, b, ws + L.total, ws, L, reinterpret_cast<cudaStream_t>(stream), &code,
+                              us_per_iter))
+        return rc;
+    *tile_cfg = code;
+    return GBPCG_OK;
+}
+
+int gbpcg_autotune_record(const gbpcg_grid *grid, const gbpcg_opts *opts, int32_t tile_cfg) {
+    clear_error();
+    if (int rc = check_grid(grid)) return rc;
+    if (int rc = check_opts(opts)) return rc;
+    gbpcg_opts o = *opts;
+    o.tile_cfg = tile_cfg;
+    if (int rc = check_opts(&o)) return rc;
+    if (!tile_cfg) return fail_arg("tile_cfg 0 is not a configuration");
+    int ca = 0, cb = 0;
+    pick_cfgs(*grid, o, &ca, &cb);
+    if (!cfg_fits(ca, grid->nx) || !cfg_fits(cb, grid->nx)) return fail_arg("configuration does not fit the grid");
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_tune[tune_key(*grid, *opts)] = tile_cfg;
+    return GBPCG_OK;
+}
+
+int gbpcg_workspace_size_batched(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts *opts, size_t *bytes) {
+    clear_error();
+    if (int rc = check_batch(nprob, grids, opts)) return rc;
+    if (!bytes) return fail_arg("bytes is NULL");
+    size_t total = round256(batch_persistent_bytes(nprob, grids));  // the persistent kernel's tables
+    for (int i = 0; i < nprob; ++i) {
+        WsLayout L;
+        total += batch_piece(grids[i], *opts, &L);
+    }
+    *bytes = total;
+    return GBPCG_OK;
+}
+
+int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *const *b, void *const *x,
+                            const gbpcg_opts *opts, gbpcg_result *results, gbpcg_stream stream) {
+    NvtxRange range("gbpcg_pcg_solve_batched");
+    clear_error();
+    if (int rc = check_batch(nprob, grids, opts)) return rc;
+    if (!b || !x || !results) return fail_arg("b, x and results must be non-NULL");
+    const size_t esz = dtype_size(opts->io_dtype);
+    for (int i = 0; i < nprob; ++i) {
+        if (!b[i] || !x[i]) return fail_arg("every b[i] and x[i] must be a device pointer");
+        if ((reinterpret_cast<uintptr_t>(b[i]) | reinterpret_cast<uintptr_t>(x[i])) & (esz - 1))
+            return fail_arg("b[i] and x[i] must be aligned to their element size");
+    }
+    const size_t region = round256(batch_persistent_bytes(nprob, grids));
+    size_t need = region;
+    std::vector<WsLayout> L(nprob);
+    std::vector<size_t> off(nprob);
+    for (int i = 0; i < nprob; ++i) {
+        off[i] = need;
+        need += batch_piece(grids[i], *opts, &L[i]);
+    }
+    if (!opts->workspace || opts->workspace_bytes < need)
+        return fail_arg("workspace smaller than gbpcg_workspace_size_batched()");
+    if (reinterpret_cast<uintptr_t>(opts->workspace) & 255u) return fail_arg("workspace must be 256-byte aligned");
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    char *ws = static_cast<char *>(opts->workspace);
+
+    // Problems that fit the chip are solved there unless tiles were asked for; what is left takes the
+    // streaming kernels as a batch of its own.
+    const bool graph = opts->flags & GBPCG_FLAG_BATCH_GRAPH;
+    ResidentChoice choice;
+    if (graph && !opts->tile_cfg && !(opts->flags & GBPCG_FLAG_AUTOTUNE)) {
+        ResPlan plan;  // bit for bit the standalone solves
+        for (int i = 0; i < nprob; ++i) (resident_fits(grids[i], &plan) ? choice.alone : choice.rest).push_back(i);
+    } else if (!graph && !opts->tile_cfg) {
+        choice = resident_choice(nprob, grids);
+    }
+    const std::vector<int> &in_batch = choice.in_batch, &alone = choice.alone, &rest = choice.rest;
+    if (!in_batch.empty() || !alone.empty()) {
+        int rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s);
+        if (rc == kResNoRoom) {  // (the tables outgrew the batch's region: one launch each)
+            std::vector<int> each = in_batch;
+            each.insert(each.end(), alone.begin(), alone.end());
+            rc = resident_batch({}, each, grids, b, x, opts, results, ws, region, L, off, s);
+        }
+        if (rc) return rc;
+        if (!rest.empty()) {
+            const int m = (int)rest.size();
+            std::vector<gbpcg_grid> g2(m);
+            std::vector<const void *> b2(m);
+            std::vector<void *> x2(m);
+            std::vector<gbpcg_result> r2(m);
+            std::vector<WsLayout> L2(m);
+            std::vector<size_t> off2(m);
+            for (int i = 0; i < m; ++i) {
+                g2[i] = grids[rest[i]];
+                b2[i] = b[rest[i]];
+                x2[i] = x[rest[i]];
+                L2[i] = L[rest[i]];
+                off2[i] = off[rest[i]];
+            }
+            rc = streamed_batch(m, g2.data(), b2.data(), x2.data(), opts, r2.data(), ws, L2, off2, s);
+            if (rc == GBPCG_ERR_ARG || rc == GBPCG_ERR_CUDA) return rc;
+            for (int i = 0; i < m; ++i) results[rest[i]] = r2[i];
+        }
+        // the batch's own figures: one time, and over all problems launches and phases
+        double ms = 0.0;
+        int launches = 0, phases = 0, worst = GBPCG_OK;
+        if (!rest.empty()) {
+            ms += results[rest[0]].time_ms;
+            launches += results[rest[0]].pass_launches[0];
+            phases += results[rest[0]].pass_launches[1];
+        }
+        const int first = in_batch.empty() ? alone[0] : in_batch[0];
+        ms += results[first].time_ms;
+        launches += results[first].pass_launches[0];
+        for (const std::vector<int> *v : {&in_batch, &alone})
+            for (int i : *v) phases += results[i].pass_launches[1];
+        for (int i = 0; i < nprob; ++i) {
+            results[i].time_ms = ms;
+            results[i].pass_launches[0] = graph ? 0 : launches;
+            results[i].pass_launches[1] = graph ? 0 : phases;
+            if (results[i].status != GBPCG_OK && worst == GBPCG_OK) worst = results[i].status;
+        }
+        return worst;
+    }
+    return streamed_batch(nprob, grids, b, x, opts, results, ws, L, off, s);
 }
 
 }  // extern "C"

@@ -1,0 +1,68 @@
+// On-chip Jacobi-PCG (resident.cu): what the solver entry points need of it.
+#pragma once
+
+#include <vector>
+
+#include "solver.cuh"
+
+namespace gb {
+
+constexpr int kResThreads = 512;
+constexpr int kResMaxCtas = 160;  // bricks of one problem (GB300 has 152 SMs)
+constexpr int kResSlotVals = 4;   // 16-byte slots per CTA and grid sum
+constexpr int kResFlagStride = 8;  // words between two CTAs' face flags
+// two buffers of slots, then the flags
+constexpr size_t kResSlotBytes = (size_t)2 * kResMaxCtas * kResSlotVals * 16 + (size_t)kResMaxCtas * kResFlagStride * 4;
+
+// How a grid is cut: sx x sy x sz bricks of 4 bx4 x by x bz points, each
+// thread of a CTA holding one four-point vector in x over `depth` planes
+// (cols = bx4 by vector columns, zseg runs of planes per column).
+struct ResPlan {
+    int build;  // which instance of the kernel (resident.cu)
+    int sx, sy, sz, bx4, by, bz, cols, zseg, depth, G;
+    int dplanes;  // planes of d held in shared memory
+    size_t smem;
+    double cycles;  // estimated SM cycles of one iteration
+};
+
+// Whether one solve of this grid runs on chip (constant coefficients), and its plan.
+bool resident_fits(const gbpcg_grid &g, ResPlan *plan);
+
+// The whole solve, enqueued on s; its scalars go to *st (DEVICE), or to the workspace's state block.
+int resident_launch(const SolveCall &c, const ResPlan &plan, cudaStream_t s, SolveState *st = nullptr);
+
+// The same solve driven from the host, which reads the device's stop flag after every iteration.
+int resident_host_loop(const SolveCall &c, const ResPlan &plan, cudaStream_t s);
+
+// Which problems of a batch run here, all in one launch or one by one, and which in the streaming
+// kernels (numbers into grids).
+struct ResidentChoice {
+    std::vector<int> in_batch, alone, rest;
+};
+ResidentChoice resident_choice(int n, const gbpcg_grid *grids);
+
+// One launch of calls[0 .. n) (ResidentChoice::in_batch) on s.  states: DEVICE, one per problem; tables:
+// DEVICE scratch (kResNoRoom, and nothing enqueued, if it is too small).
+constexpr int kResNoRoom = -1;
+int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes, int io,
+                          cudaStream_t s);
+
+struct ResProb {
+    int nx, ny, nz, nxp;  // nxp: row pitch of zg and pg, nx rounded up to a multiple of 4
+    int sx, sy, sz, bx4, by, bz, zseg, depth, cols, G, dplanes;
+    OpConst op;
+    int maxit, iters;           // iters: iterations this launch may take
+    int resume, save, final_x;  // host-driven loop: state from / to the workspace; final x update
+    double cx, cy, cz, tol;
+    const void *b;
+    void *x;
+    float *zg;  // r on brick faces, padded rows (all of r after a residual)
+    float *pg;     // p of a host-driven loop between launches
+    float4 *dlin;  // d, brick by brick, each thread's vectors a brick's thread count apart
+    SolveState *st;
+    ulonglong2 *slots;
+    unsigned *flags;      // per CTA: number of the sum its face values belong to
+    ulonglong2 *inbox;    // NULL, or every CTA's own slots of the loop's sums (grid_sum_pair)
+};
+
+}  // namespace gb
