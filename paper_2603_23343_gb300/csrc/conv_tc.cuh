@@ -873,4 +873,195 @@ __global__ void __launch_bounds__(128) wgrad_tc_kernel(const __grid_constant__ W
     if (!good && KT > 0 && threadIdx.x == 0) atomicExch(a.err, 1);
 }
 
+// ------------------------------------------------------------------------
+// Weight gradient marching in z, for 16 or 32 output channels and rows that
+// fill whole K steps (X a multiple of 16):
+//   gW[o, t, i] = sum_u gy[u - off(t), o] x[u, i]
+// Per plane a CTA takes R rows of x (R x XB voxels, NI of the input channels)
+// and R + 2 rows of gy with a voxel of halo at either end, each by one TMA
+// box, laid out [row][8-channel group][voxel][8 channels]: MN-major core
+// matrices as above, but with every tap of the three planes in reach of a
+// descriptor.  The three rows y - dy of a tap column are 3 Co consecutive
+// M rows (groups of 8 channels one row of voxels apart), dx is a shift of the
+// start address by one voxel's 16 bytes, dz another plane of the ring.  So a
+// 16-voxel K step is nine MMAs, (dz, dx), of M = 64 (Co = 16: 48 rows used)
+// or 128 (Co = 32: 96 used) and N = NI, each into its own TMEM columns; the
+// rows past 3 Co read the voxels that follow and are never looked at.
+//
+// What bounds it: wgrad_tc_kernel loads gy once per tap as boxes of 16-byte
+// pieces, 78 boxes of 128 pieces per 128 voxels (48 -> 16 channels), and the
+// TMA unit's rate for such pieces set its time.  Here a plane of gy is loaded
+// once for all 27 taps, 1,158 pieces per 128 voxels at R = 4, and the tensor
+// core's operand reads are next: 9 MMAs of 28 (M = 64, N = 48) shared-memory
+// wavefronts per 16 voxels.
+//
+// The steps (a plane of a column of rows) of the whole grid are split evenly
+// over the CTAs; each writes its sums to its own slot, added in a fixed order.
+
+struct __align__(128) WgzMaps {
+    CUtensorMap gy;  // (8, X, Co / 8, Y, Z) BF16, box (8, XB + 2, Co / 8, R + 2, 1)
+    CUtensorMap x;   // (8, X, Ci / 8, Y, Z) BF16, box (8, XB, NI / 8, R, 1)
+};
+
+struct WgzArgs {
+    int XB, R, ci, co, ni;  // ni: input channels of a CTA (slice blockIdx.y)
+    int nxb, nyb, Z;        // x blocks, y blocks, planes
+    int steps, steps_per_cta;
+    uint32_t gy_bytes, x_bytes, gy_slot, x_slot;  // box bytes and ring slot pitches
+    int ngy, nx;                                  // ring slots
+    float *partials;                              // [gridDim.x][co][27][ci]
+    int *err;
+};
+
+constexpr int kWgzMaxSlots = 8;
+
+__global__ void __launch_bounds__(128) wgrad_zmarch_kernel(const __grid_constant__ WgzMaps maps, const WgzArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t gfull[kWgzMaxSlots], gempty[kWgzMaxSlots], xfull[kWgzMaxSlots],
+        xempty[kWgzMaxSlots], done;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_err;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s0 = blockIdx.x * a.steps_per_cta, s1 = min(a.steps, s0 + a.steps_per_cta);
+    const uint32_t idesc = idesc_bf16_mn(a.co == 16 ? 64 : 128, a.ni);
+    const uint32_t ncol = tmem_cols(9 * a.ni);
+
+    if (threadIdx.x == 0) {
+        s_err = 0;
+        for (int s = 0; s < kWgzMaxSlots; ++s) {
+            mbar_init(&gfull[s], 1);
+            mbar_init(&gempty[s], 1);
+            mbar_init(&xfull[s], 1);
+            mbar_init(&xempty[s], 1);
+        }
+        mbar_init(&done, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(&tmem_base, ncol);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    const uint32_t xring = (uint32_t)a.ngy * a.gy_slot;
+
+    if (warp == 0 && lane == 0) {
+        // planes z - 1, z, z + 1 of gy for a column's first step, then one more per step
+        int kg = 0, kx = 0;  // boxes issued into either ring
+        bool ok = true;
+        auto load_gy = [&](int x0, int y0, int z) {
+            const int s = kg % a.ngy;
+            if (kg >= a.ngy && !mbar_wait_bounded(&gempty[s], ((kg / a.ngy) - 1) & 1)) return false;
+            mbar_arrive_expect_tx(&gfull[s], a.gy_bytes);
+            tma_load_5d(smem + (size_t)s * a.gy_slot, &maps.gy, &gfull[s], 0, x0 - 1, 0, y0 - 1, z);
+            ++kg;
+            return true;
+        };
+        for (int st = s0; st < s1 && ok; ++st) {
+            const int col = st / a.Z, z = st - col * a.Z;
+            const int x0 = col % a.nxb * a.XB, y0 = col / a.nxb * a.R;
+            if (st == s0 || z == 0) ok = load_gy(x0, y0, z - 1) && load_gy(x0, y0, z);
+            ok = ok && load_gy(x0, y0, z + 1);
+            if (!ok) break;
+            const int s = kx % a.nx;
+            if (kx >= a.nx && !mbar_wait_bounded(&xempty[s], ((kx / a.nx) - 1) & 1)) {
+                ok = false;
+                break;
+            }
+            mbar_arrive_expect_tx(&xfull[s], a.x_bytes);
+            tma_load_5d(smem + xring + (size_t)s * a.x_slot, &maps.x, &xfull[s], 0, x0, (int)blockIdx.y * (a.ni / 8), y0,
+                        z);
+            ++kx;
+        }
+        if (!ok) s_err = 1;
+        // every box issued has landed before the CTA can exit
+        for (int k = max(0, kg - a.ngy); k < kg; ++k)
+            if (!mbar_wait_bounded(&gfull[k % a.ngy], (k / a.ngy) & 1)) s_err = 1;
+        for (int k = max(0, kx - a.nx); k < kx; ++k)
+            if (!mbar_wait_bounded(&xfull[k % a.nx], (k / a.nx) & 1)) s_err = 1;
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t sbase = smem_u32(smem);
+        const uint32_t gv = (uint32_t)(a.XB + 2) * 16, gr = gv * (a.co / 8);  // bytes of a group, of a row
+        const uint32_t xv = (uint32_t)a.XB * 16, xr = xv * (a.ni / 8);
+        int kg = 0, kx = 0;  // boxes consumed (waited for)
+        int pl[3] = {0, 0, 0};
+        auto next_gy = [&](int &slot) {
+            slot = kg % a.ngy;
+            const bool ok = mbar_wait_bounded(&gfull[slot], (kg / a.ngy) & 1);
+            ++kg;
+            return ok;
+        };
+        bool ok = true;
+        for (int st = s0; st < s1; ++st, ++kx) {
+            const bool first = st == s0 || st % a.Z == 0;
+            if (first) {
+                if (st != s0) {  // the last column's planes, all used
+                    mma_commit(&gempty[pl[1]]);
+                    mma_commit(&gempty[pl[2]]);
+                }
+                ok = next_gy(pl[0]) && next_gy(pl[1]);
+            } else {
+                pl[0] = pl[1];
+                pl[1] = pl[2];
+            }
+            ok = ok && next_gy(pl[2]) && mbar_wait_bounded(&xfull[kx % a.nx], (kx / a.nx) & 1);
+            if (!ok) {
+                s_err = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t xs = sbase + xring + (uint32_t)(kx % a.nx) * a.x_slot;
+            for (int r = 0; r < a.R; ++r) {
+                for (int k = 0; k < a.XB / 16; ++k) {
+                    const uint64_t bd = umma_desc_mnmajor(xs + r * xr + k * 256, 128, xv);
+                    const uint32_t acc = (st != s0 || r || k) ? 1u : 0u;
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {  // plane z - 1 + p: dz = 1 - p
+                        const uint32_t ga = sbase + (uint32_t)pl[p] * a.gy_slot + r * gr + k * 256;
+#pragma unroll
+                        for (int q = 0; q < 3; ++q)  // voxel x + q of the halo row: dx = 1 - q
+                            mma_bf16(tmem + (uint32_t)((p * 3 + q) * a.ni), umma_desc_mnmajor(ga + q * 16, 128, gv), bd,
+                                     idesc, acc);
+                    }
+                }
+            }
+            mma_commit(&gempty[pl[0]]);
+            mma_commit(&xempty[kx % a.nx]);
+        }
+        mma_commit(&done);
+    }
+    __syncwarp();
+    const bool ok = mbar_wait_bounded(&done, 0);
+    __syncthreads();
+    const bool good = ok && !s_err && s1 > s0;
+    tc_fence_after();
+
+    // M row 16 or 32 j + o = tap dy = 1 - j, output channel o: warp j's lanes (an accumulator of 64 rows
+    // fills the first 16 lanes of each warp)
+    float *slot = a.partials + (int64_t)blockIdx.x * ((int64_t)a.co * 27 * a.ci);
+    for (int pq = 0; pq < 9; ++pq) {
+        const int t = (2 - pq / 3) * 9 + (2 - warp) * 3 + (2 - pq % 3);
+        for (int c0 = 0; c0 < a.ni; c0 += 16) {
+            float f[16];
+            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(pq * a.ni + c0), f);
+            if (warp < 3 && lane < a.co) {
+                float *dst = slot + ((int64_t)lane * 27 + t) * a.ci + blockIdx.y * a.ni + c0;
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    const float v[4] = {good ? f[i] : 0.f, good ? f[i + 1] : 0.f, good ? f[i + 2] : 0.f,
+                                        good ? f[i + 3] : 0.f};
+                    st4(dst + i, v);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, ncol);
+    if (!good && s1 > s0 && threadIdx.x == 0) atomicExch(a.err, 1);
+}
+
 }  // namespace gb

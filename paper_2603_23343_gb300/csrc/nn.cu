@@ -680,12 +680,28 @@ __global__ void __launch_bounds__(kWgThreads)
     }
 }
 
+// out[e] = sum of the slots' partials[k][e], in a fixed order: eight threads per element, each over every
+// eighth slot, then their sums in turn (one thread per element left the GPU waiting on 80 blocks' serial
+// loads: 35 us for 152 slots of 20,736 elements).
 __global__ void __launch_bounds__(256)
     sum_slots_kernel(int64_t n, int nslots, const float *__restrict__ partials, float *__restrict__ out) {
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (int64_t)gridDim.x * 256) {
+    __shared__ float part[8][33];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    for (int64_t e0 = (int64_t)blockIdx.x * 32; e0 < n; e0 += (int64_t)gridDim.x * 32) {
         float s = 0.0f;
-        for (int k = 0; k < nslots; ++k) s += partials[(int64_t)k * n + e];
-        out[e] = s;
+        if (e0 + lane < n) {
+#pragma unroll 4
+            for (int k = g; k < nslots; k += 8) s += partials[(int64_t)k * n + e0 + lane];
+        }
+        part[g][lane] = s;
+        __syncthreads();
+        if (g == 0 && e0 + lane < n) {
+            float t = part[0][lane];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) t += part[i][lane];
+            out[e0 + lane] = t;
+        }
+        __syncthreads();
     }
 }
 
@@ -751,11 +767,90 @@ inline WgTcPlan wgrad_tc_plan(int X, int Y, int Z, int ci, int co) {
     return p;
 }
 
+// The z-marching weight gradient (wgrad_zmarch_kernel): 16 or 32 output channels, rows of whole K steps.
+inline bool wgrad_zmarch_ok(int X, int Y, int Z, int ci, int co) {
+    return (co == 16 || co == 32) && ci % 16 == 0 && ci <= 128 && X % 16 == 0 && (X <= 128 || X % 128 == 0) &&
+           (int64_t)X * Y * Z <= INT32_MAX;
+}
+
+struct WgzPlan {
+    WgzArgs a;
+    int S;
+    size_t smem;
+};
+
+inline WgzPlan wgrad_zmarch_plan(int X, int Y, int Z, int ci, int co) {
+    WgzPlan p;
+    WgzArgs &a = p.a;
+    a.XB = std::min(X, 128);
+    a.ci = ci;
+    a.co = co;
+    a.ni = ci <= 48 ? ci : ci % 48 == 0 ? 48 : ci % 32 == 0 ? 32 : 16;  // nine accumulators in 512 TMEM columns
+    // rows per step: the most that leave room for a fourth plane of gy (three in use, one on its way), a
+    // divisor of Y so that no row of x lies outside the grid
+    const uint32_t room = 224 * 1024 - 2048;  // 2 KB spare: rows past 3 Co read on past the last plane
+    for (a.R = 4; a.R >= 1; --a.R) {
+        if (Y % a.R) continue;
+        a.gy_bytes = (uint32_t)(a.XB + 2) * 16 * (co / 8) * (a.R + 2);
+        a.x_bytes = (uint32_t)a.XB * 16 * (a.ni / 8) * a.R;
+        a.gy_slot = (a.gy_bytes + 127) / 128 * 128;
+        a.x_slot = (a.x_bytes + 127) / 128 * 128;
+        a.nx = 4 * a.gy_slot + 3 * a.x_slot <= room ? 3 : 2;
+        a.ngy = (int)std::min<uint32_t>(kWgzMaxSlots, (room - a.nx * a.x_slot) / a.gy_slot);
+        if (a.ngy >= 4 || a.R == 1) break;
+    }
+    a.nxb = X / a.XB;
+    a.nyb = Y / a.R;
+    a.Z = Z;
+    a.steps = a.nxb * a.nyb * Z;
+    // about two CTAs per SM of a 152-SM part, one after the other (a sum of half the length in the tensor
+    // core's accumulator, whose rounding grows with it), fixed so that workspace sizes do not depend on
+    // the device that asks
+    const int most = std::max(1, kWgTargetBlocks / 2 / (ci / a.ni));
+    a.steps_per_cta = (a.steps + most - 1) / most;
+    p.S = (a.steps + a.steps_per_cta - 1) / a.steps_per_cta;
+    p.smem = (size_t)a.ngy * a.gy_slot + (size_t)a.nx * a.x_slot + 2048;
+    a.partials = nullptr;
+    a.err = nullptr;
+    return p;
+}
+
 inline size_t wgrad_partial_bytes(int X, int Y, int Z, int ci, int co) {
     WgradPlan p = wgrad_plan(X, Y, Z, ci, co);
     size_t b = (size_t)p.S * 27 * ci * co * sizeof(float);
     if (wgrad_tc_ok(X, Y, Z, ci, co)) b = std::max(b, (size_t)wgrad_tc_plan(X, Y, Z, ci, co).S * 27 * ci * co * 4);
+    if (wgrad_zmarch_ok(X, Y, Z, ci, co))
+        b = std::max(b, (size_t)wgrad_zmarch_plan(X, Y, Z, ci, co).S * 27 * ci * co * 4);
     return b;
+}
+
+static int sum_slots(int64_t n, int slots, const float *partials, float *gw, cudaStream_t s) {
+    sum_slots_kernel<<<blocks_for(n, 32), 256, 0, s>>>(n, slots, partials, gw);
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "sum_slots launch");
+}
+
+static int wgrad_zmarch(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, const __nv_bfloat16 *gy,
+                        float *gw, float *partials, int *err, cudaStream_t s) {
+    const WgzPlan p = wgrad_zmarch_plan(X, Y, Z, ci, co);
+    WgzArgs a = p.a;
+    a.partials = partials;
+    a.err = err;
+    WgzMaps maps;
+    const uint64_t gd[5] = {8, (uint64_t)X, (uint64_t)co / 8, (uint64_t)Y, (uint64_t)Z};
+    const uint64_t gs[4] = {(uint64_t)co * 2, 16, (uint64_t)co * 2 * X, (uint64_t)co * 2 * X * Y};
+    const uint32_t gb[5] = {8, (uint32_t)a.XB + 2, (uint32_t)co / 8, (uint32_t)a.R + 2, 1};
+    int rc = make_map_nd(&maps.gy, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, gy, 5, gd, gs, gb);
+    if (rc) return rc;
+    const uint64_t xd[5] = {8, (uint64_t)X, (uint64_t)ci / 8, (uint64_t)Y, (uint64_t)Z};
+    const uint64_t xs[4] = {(uint64_t)ci * 2, 16, (uint64_t)ci * 2 * X, (uint64_t)ci * 2 * X * Y};
+    const uint32_t xb[5] = {8, (uint32_t)a.XB, (uint32_t)a.ni / 8, (uint32_t)a.R, 1};
+    rc = make_map_nd(&maps.x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, x, 5, xd, xs, xb);
+    if (rc) return rc;
+    GB_CUDA(cudaFuncSetAttribute(wgrad_zmarch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+    wgrad_zmarch_kernel<<<dim3(p.S, ci / a.ni), 128, p.smem, s>>>(maps, a);
+    GB_CUDA(cudaGetLastError());
+    return sum_slots((int64_t)27 * ci * co, p.S, partials, gw, s);
 }
 
 static int wgrad_tc(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, const __nv_bfloat16 *gy, float *gw,
@@ -793,10 +888,7 @@ static int wgrad_tc(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x,
     wgrad_tc_kernel<<<dim3(p.S, p.ngroups), 128, p.smem, s>>>(maps, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail_cuda(e, "wgrad_tc launch");
-    const int64_t n = (int64_t)27 * ci * co;
-    sum_slots_kernel<<<blocks_for(n, 256), 256, 0, s>>>(n, p.S, partials, gw);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "sum_slots launch");
+    return sum_slots((int64_t)27 * ci * co, p.S, partials, gw, s);
 }
 
 template <int BO, int BI>
@@ -810,6 +902,7 @@ static cudaError_t wgrad_launch(const WgradPlan &p, int X, int Y, int Z, int ci,
 
 static int wgrad(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, const __nv_bfloat16 *gy, float *gw,
                  float *partials, cudaStream_t s, int *err = nullptr) {
+    if (err && wgrad_zmarch_ok(X, Y, Z, ci, co)) return wgrad_zmarch(X, Y, Z, ci, co, x, gy, gw, partials, err, s);
     if (err && wgrad_tc_ok(X, Y, Z, ci, co)) return wgrad_tc(X, Y, Z, ci, co, x, gy, gw, partials, err, s);
     if (!wgrad_ok(X, ci, co)) return fail_arg("weight gradient: unsupported width or channel count");
     WgradPlan p = wgrad_plan(X, Y, Z, ci, co);
@@ -822,7 +915,7 @@ static int wgrad(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, co
     else e = wgrad_launch<1, 1>(p, X, Y, Z, ci, co, x, gy, partials, s);
     if (e != cudaSuccess) return fail_cuda(e, "wgrad launch");
     const int64_t n = (int64_t)27 * ci * co;
-    sum_slots_kernel<<<blocks_for(n, 256), 256, 0, s>>>(n, p.S, partials, gw);
+    sum_slots_kernel<<<blocks_for(n, 32), 256, 0, s>>>(n, p.S, partials, gw);
     e = cudaGetLastError();
     return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "sum_slots launch");
 }
