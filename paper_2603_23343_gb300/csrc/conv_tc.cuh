@@ -437,6 +437,175 @@ __global__ void __launch_bounds__(128) conv3_tc_halo_kernel(const __grid_constan
     if (!good && threadIdx.x == 0) atomicExch(a.err, 1);
 }
 
+// ------------------------------------------------------------------------
+// Halo-slab variant for rows shorter than 128 voxels (X = 64, 32 or 16): the
+// coarse levels of the network, and every level of grids below 128.  As above
+// a step is one 16-channel chunk of one source plane, loaded once for its nine
+// taps; what differs is the M tile:
+//   X = 64      M = 64, one row; the slab rows have their two halo voxels, and
+//               a tap is an offset into them as above
+//   X = 32, 16  M = 128, several rows, which must follow one another without a
+//               gap (one stride between 8-voxel groups): three copies of the
+//               slab, loaded at x - 1, x and x + 1 (TMA supplies the zeros
+//               past either end), one per dx
+// A CTA owns `tiles` M tiles, one accumulator each.  conv3_tc_kernel reloads a
+// tile for each tap: 18 16-byte pieces per voxel and plane chunk, whose rate
+// in the TMA unit set its time; here 2.6 (X = 64, 8 rows) or 7.5 (X = 32).
+
+template <int CO, bool WIDE>  // WIDE: X = 64
+struct RowsCfg {
+    static constexpr int M = WIDE ? 64 : 128;
+    static constexpr int MAXT = 256 / CO < 8 ? 256 / CO : 8;  // two CTAs per SM share its TMEM
+    static constexpr uint32_t B_HALF = 9u * CO * 16u;
+    __host__ __device__ static int rows(int X, int tiles) { return tiles * (M / X); }
+    // one half (8 channels) of a slab: all its copies
+    __host__ __device__ static uint32_t copy_bytes(int X, int tiles) {
+        return (uint32_t)((WIDE ? X + 2 : X) * (rows(X, tiles) + 2) * 16);
+    }
+    __host__ __device__ static uint32_t copy_pitch(int X, int tiles) { return (copy_bytes(X, tiles) + 127) & ~127u; }
+    __host__ __device__ static uint32_t a_half(int X, int tiles) { return (WIDE ? 1 : 3) * copy_pitch(X, tiles); }
+    __host__ __device__ static uint32_t stage(int X, int tiles) {
+        return (2 * a_half(X, tiles) + 2 * B_HALF + 1023) & ~1023u;
+    }
+};
+constexpr int kRowsMaxStages = 6;
+
+template <int CO, bool WIDE, typename OUT>
+__global__ void __launch_bounds__(128) conv3_tc_rows_kernel(const __grid_constant__ ConvMaps maps, const ConvArgs a,
+                                                            int tiles) {
+    using H = RowsCfg<CO, WIDE>;
+    constexpr uint32_t IDESC = idesc_bf16(H::M, CO);
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t full[kRowsMaxStages], empty[kRowsMaxStages], done;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_err;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int X = a.X, S = a.stages, tr = H::M / X;
+    const int y0 = blockIdx.x * tiles * tr, z0 = blockIdx.y;
+    const int kc = a.ci / 16;
+    const int KT = 3 * kc;  // (chunk, plane) steps
+    const uint32_t pitch = (uint32_t)(WIDE ? X + 2 : X) * 16;
+    const uint32_t cb = H::copy_bytes(X, tiles), cp = H::copy_pitch(X, tiles), ah = H::a_half(X, tiles);
+    const uint32_t sbytes = H::stage(X, tiles);
+    const uint32_t ncol = tmem_cols(tiles * CO);
+
+    if (threadIdx.x == 0) {
+        s_err = 0;
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&done, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(&tmem_base, ncol);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    const uint32_t sbase = smem_u32(smem);
+
+    if (warp == 0 && lane == 0) {
+        int kk = 0;
+        for (; kk < KT; ++kk) {
+            const int s = kk % S;
+            if (kk >= S && !mbar_wait_bounded(&empty[s], ((kk / S) - 1) & 1)) {
+                s_err = 1;
+                break;
+            }
+            const int cc = kk / 3, pz = kk - cc * 3;  // chunk, plane (dz = pz - 1)
+            unsigned char *st = smem + (size_t)s * sbytes;
+            mbar_arrive_expect_tx(&full[s], 2 * (WIDE ? 1 : 3) * cb + 2 * H::B_HALF);
+            for (int h = 0; h < 2; ++h) {
+                if (WIDE) {
+                    tma_load_4d(st + h * ah, &maps.act, &full[s], cc * 16 + h * 8, -1, y0 - 1, z0 + pz - 1);
+                } else {
+                    for (int dx = 0; dx < 3; ++dx)
+                        tma_load_4d(st + h * ah + dx * cp, &maps.act, &full[s], cc * 16 + h * 8, dx - 1, y0 - 1,
+                                    z0 + pz - 1);
+                }
+                tma_load_3d(st + 2 * ah + h * H::B_HALF, &maps.wgt, &full[s], cc * 16 + h * 8, 0, pz * 9);
+            }
+        }
+        for (int s = 0; s < S; ++s) {
+            const int last = kk - 1 - ((kk - 1 - s) % S + S) % S;
+            if (last >= 0 && last < kk && !mbar_wait_bounded(&full[s], (last / S) & 1)) s_err = 1;
+        }
+    } else if (warp == 1 && lane == 0) {
+        for (int kk = 0; kk < KT; ++kk) {
+            const int s = kk % S;
+            if (!mbar_wait_bounded(&full[s], (kk / S) & 1)) {
+                s_err = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t sa = sbase + (uint32_t)s * sbytes, sb = sa + 2 * ah;
+#pragma unroll 1
+            for (int j = 0; j < tiles; ++j)
+#pragma unroll
+                for (int tau = 0; tau < 9; ++tau) {
+                    const uint32_t row = (uint32_t)(j * tr + tau / 3) * pitch;  // dy = tau / 3 - 1
+                    const uint32_t aa = sa + row + (WIDE ? (uint32_t)(tau % 3) * 16 : (uint32_t)(tau % 3) * cp);
+                    mma_bf16(tmem + (uint32_t)(j * CO), umma_desc_kmajor(aa, ah, 128),
+                             umma_desc_kmajor(sb + (uint32_t)(tau * CO * 16), H::B_HALF, 128), IDESC,
+                             (kk > 0 || tau > 0) ? 1u : 0u);
+                }
+            mma_commit(&empty[s]);
+        }
+        mma_commit(&done);
+    }
+    __syncwarp();
+    const bool ok = mbar_wait_bounded(&done, 0);
+    __syncthreads();
+    const bool good = ok && !s_err;
+    tc_fence_after();
+
+    // epilogue: an accumulator of 64 rows fills the first 16 lanes of each warp, one of 128 all lanes
+    const int m = WIDE ? warp * 16 + lane : warp * 32 + lane;
+    const int x = WIDE ? m : m % X, yr = WIDE ? 0 : m / X;
+#pragma unroll 1
+    for (int j = 0; j < tiles; ++j) {
+        const int y = y0 + j * tr + yr;
+        const bool in = (!WIDE || lane < 16) && y < a.Y;
+        const int64_t v = ((int64_t)z0 * a.Y + y) * X + x;
+        OUT *out = static_cast<OUT *>(a.out) + v * a.cstride + a.coff;
+        const __nv_bfloat16 *mk = a.mask ? a.mask + v * a.mstride + a.moff : nullptr;
+#pragma unroll
+        for (int c0 = 0; c0 < CO; c0 += 16) {
+            float f[16];
+            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(j * CO + c0), f);
+            if (!in) continue;
+            float mv[16];
+            if (mk) {
+                ld8(mk + c0, mv);
+                ld8(mk + c0 + 8, mv + 8);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                f[i] = good ? f[i] : 0.0f;
+                if (a.relu) f[i] = f[i] < 0.0f ? 0.0f : f[i];
+                if (mk && !(mv[i] > 0.0f)) f[i] = 0.0f;
+            }
+            if constexpr (std::is_same<OUT, float>::value) {
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) st4(out + c0 + i, f + i);
+            } else {
+                st8(out + c0, f);
+                st8(out + c0 + 8, f + 8);
+            }
+        }
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, ncol);
+    if (!good && threadIdx.x == 0) atomicExch(a.err, 1);
+}
+
 }  // namespace gb
 
 namespace gb {

@@ -73,6 +73,39 @@ inline bool conv_tile(int X, int Y, int Z, ConvTile *t) {
 
 // ----------------------------------------------- tensor-core convolution --
 
+// Rows of 16, 32 or 64 voxels: the rows kernel, its tiles per CTA the most that still give every SM two CTAs.
+template <int CO, bool WIDE, typename OUT>
+static int conv_rows_launch(const ConvArgs &args, const __nv_bfloat16 *in, const __nv_bfloat16 *w, cudaStream_t s) {
+    using H = RowsCfg<CO, WIDE>;
+    ConvArgs a = args;
+    int tiles = H::MAXT;
+    auto ctas = [&](int t) { return (int64_t)((a.Y + H::rows(a.X, t) - 1) / H::rows(a.X, t)) * a.Z; };
+    while (tiles > 1 && ctas(tiles) < 2 * (int64_t)device_sm_count()) --tiles;
+    constexpr uint32_t kBudget = 110u * 1024u;  // two CTAs per SM
+    while (tiles > 1 && 2 * H::stage(a.X, tiles) > kBudget) --tiles;
+    const uint32_t stage = H::stage(a.X, tiles);
+    a.stages = (int)std::max<uint32_t>(2, std::min<uint32_t>(kRowsMaxStages, kBudget / stage));
+    const int rows = H::rows(a.X, tiles);
+    ConvMaps maps;
+    const uint64_t dims[4] = {(uint64_t)a.ci, (uint64_t)a.X, (uint64_t)a.Y, (uint64_t)a.Z};
+    const uint64_t strides[3] = {(uint64_t)a.ci * 2, (uint64_t)a.ci * 2 * a.X, (uint64_t)a.ci * 2 * a.X * a.Y};
+    const uint32_t box[4] = {8, (uint32_t)(WIDE ? a.X + 2 : a.X), (uint32_t)rows + 2, 1};
+    int rc = make_map_nd(&maps.act, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, in, 4, dims, strides, box);
+    if (rc) return rc;
+    const uint64_t wd[3] = {(uint64_t)a.ci, (uint64_t)CO, 27};
+    const uint64_t wst[2] = {(uint64_t)27 * a.ci * 2, (uint64_t)a.ci * 2};
+    const uint32_t wb[3] = {8, (uint32_t)CO, 9};
+    rc = make_map_nd(&maps.wgt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, w, 3, wd, wst, wb);
+    if (rc) return rc;
+    const size_t smem = (size_t)a.stages * stage;
+    GB_CUDA(cudaFuncSetAttribute(conv3_tc_rows_kernel<CO, WIDE, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    conv3_tc_rows_kernel<CO, WIDE, OUT>
+        <<<dim3((unsigned)((a.Y + rows - 1) / rows), (unsigned)a.Z), 128, smem, s>>>(maps, a, tiles);
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "conv3_tc_rows launch");
+}
+
 template <int CO, typename OUT>
 static int conv_tc_launch(int X, int Y, int Z, int ci, const __nv_bfloat16 *in, const __nv_bfloat16 *w, OUT *out,
                           int cstride, int coff, int relu, const __nv_bfloat16 *mask, int mstride, int moff, int *err,
@@ -92,6 +125,10 @@ static int conv_tc_launch(int X, int Y, int Z, int ci, const __nv_bfloat16 *in, 
     a.mstride = mstride;
     a.moff = moff;
     a.err = err;
+    if (Z <= 65535) {
+        if (X == 64) return conv_rows_launch<CO, true, OUT>(a, in, w, s);
+        if (X == 32 || X == 16) return conv_rows_launch<CO, false, OUT>(a, in, w, s);
+    }
     ConvMaps maps;
     const uint64_t dims[4] = {(uint64_t)ci, (uint64_t)X, (uint64_t)Y, (uint64_t)Z};
     const uint64_t strides[3] = {(uint64_t)ci * 2, (uint64_t)ci * 2 * X, (uint64_t)ci * 2 * X * Y};
