@@ -125,11 +125,106 @@ __global__ void stencil_f64_kernel(int nx, int ny, int nz, const double *__restr
     }
 }
 
+// Face weights of a thread's column (i, j) as it marches upwards in z from plane k0, the values of
+// OpBlock::weights: the x and y ones change with the z block only.
+struct ColumnWeights {
+    float w0, w1, w2, w3, kc, km, kp;  // km, kp: across the block's -z and +z face
+    int bz, iz;
+    __device__ __forceinline__ void block(const OpBlock &o, int i, int j) {
+        const int bx = i / o.kbx, by = j / o.kby, ix = i - bx * o.kbx, iy = j - by * o.kby;
+        kc = o.K(bx, by, bz);
+        w0 = o.cx * ((ix == 0 && i > 0) ? OpBlock::hm(kc, o.K(bx - 1, by, bz)) : kc);
+        w1 = o.cx * ((ix == o.kbx - 1 && i < o.nx - 1) ? OpBlock::hm(kc, o.K(bx + 1, by, bz)) : kc);
+        w2 = o.cy * ((iy == 0 && j > 0) ? OpBlock::hm(kc, o.K(bx, by - 1, bz)) : kc);
+        w3 = o.cy * ((iy == o.kby - 1 && j < o.ny - 1) ? OpBlock::hm(kc, o.K(bx, by + 1, bz)) : kc);
+        km = bz > 0 ? OpBlock::hm(kc, o.K(bx, by, bz - 1)) : kc;
+        kp = (bz + 1) * o.kbz < o.nz ? OpBlock::hm(kc, o.K(bx, by, bz + 1)) : kc;
+    }
+    __device__ __forceinline__ void start(const OpBlock &o, int i, int j, int k0) {
+        bz = k0 / o.kbz;
+        iz = k0 - bz * o.kbz;
+        block(o, i, j);
+    }
+    __device__ __forceinline__ void next(const OpBlock &o, int i, int j, int k) {  // to plane k < nz
+        if (++iz == o.kbz) {
+            iz = 0;
+            ++bz;
+            block(o, i, j);
+        }
+    }
+    // (A u)_c = sum of w_f (u_c - u_f)
+    __device__ __forceinline__ float apply(const OpBlock &o, float c, float xm, float xp, float ym, float yp, float zm,
+                                           float zp) const {
+        const float w4 = o.cz * (iz == 0 ? km : kc), w5 = o.cz * (iz == o.kbz - 1 ? kp : kc);
+        float q = fmaf(w0, c - xm, w1 * (c - xp));
+        q = fmaf(w2, c - ym, q);
+        q = fmaf(w3, c - yp, q);
+        q = fmaf(w4, c - zm, q);
+        return fmaf(w5, c - zp, q);
+    }
+};
+
+// q = A p with plain loads, one thread per (x, y) column of zc planes, its z neighbours in registers, the
+// others through L1: for arrays whose rows TMA cannot take, and for grids too small to fill the GPU with
+// marching tiles.  The engine's plain-load form copies each box element by element between two barriers
+// per plane (255 x 187 x 201, block coefficients: 119 us), and derives a point's six weights from the
+// block table each time; 32^3 in TMA boxes is a chain of eight planes in eight CTAs.
 template <typename T, typename Op>
-static int stencil_engine(const gbpcg_grid &gr, const void *p, void *q, const Op &op, cudaStream_t s) {
+__global__ void __launch_bounds__(256)
+    stencil_direct_kernel(int nx, int ny, int nz, int zc, const T *__restrict__ p, T *__restrict__ q, const Op op) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nx) return;
+    const int k0 = blockIdx.z * zc, k1 = min(nz, k0 + zc);
+    const int64_t plane = (int64_t)nx * ny;
+    for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < ny; j += gridDim.y * blockDim.y) {
+        const T *pc = p + (int64_t)k0 * plane + (int64_t)j * nx + i;
+        T *qc = q + (pc - p);
+        auto ld = [](const T *a) { return to_f(__ldg(a)); };
+        float zm = k0 > 0 ? ld(pc - plane) : 0.0f, c = ld(pc);
+        ColumnWeights cw;
+        if constexpr (!Op::kConst) cw.start(op, i, j, k0);
+        for (int k = k0; k < k1; ++k, pc += plane, qc += plane) {
+            const float zp = k + 1 < nz ? ld(pc + plane) : 0.0f;
+            const float xm = i > 0 ? ld(pc - 1) : 0.0f, xp = i + 1 < nx ? ld(pc + 1) : 0.0f;
+            const float ym = j > 0 ? ld(pc - nx) : 0.0f, yp = j + 1 < ny ? ld(pc + nx) : 0.0f;
+            float r, dg;
+            if constexpr (Op::kConst) {
+                op.apply(c, xm, xp, ym, yp, zm, zp, i, j, k, r, dg);
+            } else {
+                r = cw.apply(op, c, xm, xp, ym, yp, zm, zp);
+                if (k + 1 < k1) cw.next(op, i, j, k + 1);
+            }
+            *qc = from_f<T>(r);
+            zm = c;
+            c = zp;
+        }
+    }
+}
+
+// Where the engine could run, measured (us, engine and direct): constant coefficients FP32 32^3 9.4 / 1.3,
+// 64^3 5.1 / 2.2, 128^3 5.5 / 4.8, 192^3 10.3 / 9.7, 256^3 22.1 / 31.0, in 16 bits 128^3 5.3 / 5.3, 160^3
+// 7.0 / 8.3; block coefficients at every size direct (64^3 20.6 / 4.7, 256^3 112 / 63).
+template <typename T>
+constexpr int64_t direct_points() { return sizeof(T) == 4 ? 8000000 : 2200000; }
+
+template <typename T, typename Op>
+static int stencil_direct(const gbpcg_grid &g, const void *p, void *q, const Op &op, cudaStream_t s) {
+    const dim3 block = g.nx <= 32 ? dim3(32, 8) : dim3(64, 4);
+    const int64_t gx = (g.nx + block.x - 1) / block.x, gy = std::min<int64_t>(65535, (g.ny + block.y - 1) / block.y);
+    // planes per thread: up to 16, fewer where that leaves SMs without eight blocks each
+    const int64_t want = (int64_t)device_sm_count() * 8;
+    const int zc = (int)std::max<int64_t>({1, std::min<int64_t>(16, gx * gy * g.nz / want), (g.nz + 65534) / 65535});
+    stencil_direct_kernel<T, Op><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)((g.nz + zc - 1) / zc)), block, 0, s>>>(
+        g.nx, g.ny, g.nz, zc, static_cast<const T *>(p), static_cast<T *>(q), op);
+    GB_CUDA(cudaGetLastError());
+    return GBPCG_OK;
+}
+
+template <typename T>
+static int stencil_engine(const gbpcg_grid &gr, const void *p, void *q, const OpConst &op, cudaStream_t s) {
+    using Op = OpConst;
     const int nx = gr.nx, ny = gr.ny, nz = gr.nz;
     const int cfg = nx <= 32 ? CFG_32x16 : CFG_64x16;
-    const bool tma = tma_ok(sizeof(T), nx, {p, q});
     PassArgs a{};
     a.nx = nx; a.ny = ny; a.nz = nz;
     a.h0[0] = a.h0[1] = p;
@@ -140,30 +235,26 @@ static int stencil_engine(const gbpcg_grid &gr, const void *p, void *q, const Op
     a.scale = 1.0f;
     PassMaps maps;
     memset(&maps, 0, sizeof(maps));
-    int occ = tma ? GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::occupancy())
-                  : GB_CFG_DISPATCH(cfg, T, K_STENCIL, false, Op, K::occupancy());
-    size_t smem = tma ? GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::smem)
-                      : GB_CFG_DISPATCH(cfg, T, K_STENCIL, false, Op, K::smem);
-    PassGeom geo = make_geom(cfg, nx, ny, nz, occ, smem);
+    const int occ = GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::occupancy());
+    const PassGeom geo = make_geom(cfg, nx, ny, nz, occ, GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::smem));
     a.tiles_x = geo.tiles_x;
     a.zchunk = geo.zchunk;
-    if (tma) {
-        int rc = make_pass_map<T>(&maps.h0[0], cfg, true, p, nx, ny, nz);
-        if (rc) return rc;
-        maps.h0[1] = maps.h0[0];
-        maps.h1[0] = maps.h1[1] = maps.h0[0];
-        maps.c0 = maps.h0[0];
-    }
-    cudaError_t e = tma ? GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::launch(maps, a, op, geo.grid(), s))
-                        : GB_CFG_DISPATCH(cfg, T, K_STENCIL, false, Op, K::launch(maps, a, op, geo.grid(), s));
+    if (int rc = make_pass_map<T>(&maps.h0[0], cfg, true, p, nx, ny, nz)) return rc;
+    maps.h0[1] = maps.h0[0];
+    maps.h1[0] = maps.h1[1] = maps.h0[0];
+    maps.c0 = maps.h0[0];
+    const cudaError_t e = GB_CFG_DISPATCH(cfg, T, K_STENCIL, true, Op, K::launch(maps, a, op, geo.grid(), s));
     if (e != cudaSuccess) return fail_cuda(e, "stencil launch");
     return GBPCG_OK;
 }
 
 template <typename T>
 static int stencil_typed(const gbpcg_grid &g, const void *p, void *q, cudaStream_t s) {
-    if (g.k_block) return stencil_engine<T>(g, p, q, make_op_block(g), s);
-    return stencil_engine<T>(g, p, q, make_op_const(g.nx, g.ny, g.nz), s);
+    if (g.k_block) return stencil_direct<T>(g, p, q, make_op_block(g), s);
+    const OpConst op = make_op_const(g.nx, g.ny, g.nz);
+    const int64_t n = (int64_t)g.nx * g.ny * g.nz;
+    return tma_ok(sizeof(T), g.nx, {p, q}) && n > direct_points<T>() ? stencil_engine<T>(g, p, q, op, s)
+                                                                    : stencil_direct<T>(g, p, q, op, s);
 }
 
 int launch_stencil_f64(const gbpcg_grid &g, const double *p, double *q, cudaStream_t s) {

@@ -115,8 +115,6 @@ struct OpConst {
 // cell's own k inside a block and on the domain boundary.
 struct OpBlock {
     static constexpr bool kConst = false;
-    using Cache = NoCache;
-    float inv_d;  // unused
     const float *kb;
     int nx, ny, nz, nbx, nby, kbx, kby, kbz;
     float cx, cy, cz;
@@ -135,17 +133,6 @@ struct OpBlock {
         w[4] = cz * ((iz == 0 && k > 0) ? hm(kc, K(bx, by, bz - 1)) : kc);
         w[5] = cz * ((iz == kbz - 1 && k < nz - 1) ? hm(kc, K(bx, by, bz + 1)) : kc);
     }
-    __device__ __forceinline__ void apply(float c, float xm, float xp, float ym, float yp, float zm, float zp, int i,
-                                          int j, int k, float &q, float &dg) const {
-        float w[6];
-        weights(i, j, k, w);
-        q = w[0] * (c - xm) + w[1] * (c - xp) + w[2] * (c - ym) + w[3] * (c - yp) + w[4] * (c - zm) + w[5] * (c - zp);
-        dg = ((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]);
-    }
-    template <int V>
-    __device__ __forceinline__ void applyv(Cache &, const float c[V], float xl, float xr, const float ym[V],
-                                           const float yp[V], const float zm[V], const float zp[V], int gx, int gy,
-                                           int k, int nx_, int ny_, float q[V], float dg[V], float rdg[V]) const;
 };
 
 // 1/x by the hardware's approximate reciprocal (PTX rcp.approx.ftz.f32: at
@@ -185,13 +172,6 @@ __device__ __forceinline__ void OpConst::applyv(Cache &, const float c[V], float
                                                 int gy, int k, int nx, int ny, float q[V], float dg[V],
                                                 float rdg[V]) const {
     applyv_pointwise<V>(*this, c, xl, xr, ym, yp, zm, zp, gx, gy, k, nx, ny, q, dg, rdg);
-}
-template <int V>
-__device__ __forceinline__ void OpBlock::applyv(Cache &, const float c[V], float xl, float xr, const float ym[V],
-                                                const float yp[V], const float zm[V], const float zp[V], int gx,
-                                                int gy, int k, int nx_, int ny_, float q[V], float dg[V],
-                                                float rdg[V]) const {
-    applyv_pointwise<V>(*this, c, xl, xr, ym, yp, zm, zp, gx, gy, k, nx_, ny_, q, dg, rdg);
 }
 
 // Block-constant coefficient through a per-block face table built once per

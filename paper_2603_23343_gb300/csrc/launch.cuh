@@ -182,7 +182,6 @@ inline OpConst make_op_const(int nx, int ny, int nz, float scale = 1.0f) {
 inline OpBlock make_op_block(const gbpcg_grid &g, float scale = 1.0f) {
     auto c = [](int n) { double h = 1.0 / (n + 1); return 1.0 / (h * h); };
     OpBlock o;
-    o.inv_d = 0.0f;
     o.kb = g.k_block;
     o.nx = g.nx; o.ny = g.ny; o.nz = g.nz;
     o.kbx = g.kbx; o.kby = g.kby; o.kbz = g.kbz;
