@@ -40,7 +40,7 @@ constexpr int kMaxDirs = 32;
 struct FcgState {
     double bb, rz, rp, rr, rr64;
     double pq[kMaxDirs + 1];  // p.Ap of every ring slot
-    double c[kMaxDirs];       // projection coefficients of the current step
+    float cf[kMaxDirs];       // projection coefficients of the current step
     int bad;                  // 1: p.Ap <= 0 or not finite; 2: r.z <= 0 or not finite
     int pad;
     unsigned ticket[4];
@@ -96,37 +96,70 @@ __device__ __forceinline__ bool fcg_reduce(const double (&acc)[NV], double *part
 
 // r.z and z.Ap_i of every previous direction; the last block forms the
 // projection coefficients c_i = z.Ap_i / p_i.Ap_i and checks r.z > 0.
+// blockIdx.x: kMdotDirs of the vectors r, Ap_1, Ap_2, ...; blockIdx.y: a chunk
+// of the grid.  (One block row for all vectors left 32 blocks at 64^3, each
+// with 33 FP64 block sums to do: 106 us; the chunks' z is read again from L2.)
+constexpr int kMdotDirs = 4;
 __global__ void __launch_bounds__(kFcgThreads)
     fcg_mdot_kernel(int64_t n4, FcgState *st, double *partials, const float *__restrict__ r,
                     const float *__restrict__ z, const DirSet d) {
     // FP32 sums per thread (a handful of grid-stride steps), FP64 from the warp sums on:
     // GB300's FP64 pipe would otherwise bound this kernel, not its loads
-    float facc[kMaxDirs + 1];
+    const int v0 = blockIdx.x * kMdotDirs, nv = d.nd + 1;
+    const float4 *q[kMdotDirs];
+    float facc[kMdotDirs];
 #pragma unroll
-    for (int v = 0; v <= kMaxDirs; ++v) facc[v] = 0.0f;
-    for (int64_t i = (int64_t)blockIdx.x * kFcgThreads + threadIdx.x; i < n4; i += (int64_t)gridDim.x * kFcgThreads) {
-        const float4 zv = reinterpret_cast<const float4 *>(z)[i];
-        facc[0] += dot4f(reinterpret_cast<const float4 *>(r)[i], zv);
-#pragma unroll
-        for (int j = 0; j < kMaxDirs; ++j)
-            if (j < d.nd) facc[1 + j] += dot4f(reinterpret_cast<const float4 *>(d.q[j])[i], zv);
+    for (int v = 0; v < kMdotDirs; ++v) {
+        facc[v] = 0.0f;
+        q[v] = reinterpret_cast<const float4 *>(v0 + v == 0 ? r : d.q[min(max(v0 + v - 1, 0), kMaxDirs - 1)]);
     }
-    double acc[kMaxDirs + 1];
+    for (int64_t i = (int64_t)blockIdx.y * kFcgThreads + threadIdx.x; i < n4; i += (int64_t)gridDim.y * kFcgThreads) {
+        const float4 zv = reinterpret_cast<const float4 *>(z)[i];
 #pragma unroll
-    for (int v = 0; v <= kMaxDirs; ++v) acc[v] = (double)facc[v];
-    double tot[kMaxDirs + 1];
-    if (fcg_reduce<kMaxDirs + 1>(acc, partials, &st->ticket[0], tot) && threadIdx.x == 0) {
+        for (int v = 0; v < kMdotDirs; ++v)
+            if (v0 + v < nv) facc[v] += dot4f(q[v][i], zv);
+    }
+    __shared__ double red[kFcgThreads / 32][kMdotDirs];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int v = 0; v < kMdotDirs; ++v) {
+        const double s = warp_sum((double)facc[v]);
+        if (lane == 0) red[warp][v] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < kMdotDirs && v0 + threadIdx.x < nv) {
+        double s = 0.0;
+        for (int w = 0; w < kFcgThreads / 32; ++w) s += red[w][threadIdx.x];
+        partials[(size_t)(v0 + threadIdx.x) * gridDim.y + blockIdx.y] = s;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->ticket[0], 1u) == gridDim.x * gridDim.y - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the last block: one warp per vector adds its chunks in order
+    __shared__ double tot[kMaxDirs + 1];
+    for (int v = warp; v < nv; v += kFcgThreads / 32) {
+        double s = 0.0;
+        for (unsigned k = lane; k < gridDim.y; k += 32) s += __ldcg(partials + (size_t)v * gridDim.y + k);
+        s = warp_sum(s);
+        if (lane == 0) tot[v] = s;
+    }
+    __syncthreads();
+    bool bad = false;
+    if (threadIdx.x < d.nd) {
+        const double c = tot[1 + threadIdx.x] / st->pq[d.slot[threadIdx.x]];
+        bad = !isfinite(c);
+        st->cf[threadIdx.x] = (float)c;
+    }
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
         const double rz = tot[0];
-        bool ok = rz > 0.0 && isfinite(rz);
-#pragma unroll
-        for (int j = 0; j < kMaxDirs; ++j)  // static indices: no local copy of the parameter arrays
-            if (j < d.nd) {
-                const double c = tot[1 + j] / st->pq[d.slot[j]];
-                ok = ok && isfinite(c);
-                st->c[j] = c;
-            }
         st->rz = rz;
-        if (!ok) st->bad = 2;
+        st->ticket[0] = 0u;
+        if (bad || !(rz > 0.0) || !isfinite(rz)) st->bad = 2;
     }
 }
 
@@ -137,7 +170,7 @@ __global__ void __launch_bounds__(256)
     if (st->bad) return;
     float c[kMaxDirs];
 #pragma unroll
-    for (int j = 0; j < kMaxDirs; ++j) c[j] = j < d.nd ? (float)st->c[j] : 0.0f;
+    for (int j = 0; j < kMaxDirs; ++j) c[j] = j < d.nd ? st->cf[j] : 0.0f;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
         float4 v = reinterpret_cast<const float4 *>(z)[i];
 #pragma unroll
@@ -267,8 +300,10 @@ static int fcg_check(const gbpcg_grid *g, const gbpcg_opts *o) {
     return GBPCG_OK;
 }
 
+// Blocks of the reducing kernels: eight vectors of four per thread, fewer where that leaves SMs idle.
 static unsigned red_blocks(int64_t n4) {
-    const int64_t want = (n4 + kFcgThreads * 8 - 1) / (kFcgThreads * 8);
+    const int64_t per = std::max<int64_t>(1, std::min<int64_t>(8, n4 / ((int64_t)kFcgThreads * device_sm_count())));
+    const int64_t want = (n4 + kFcgThreads * per - 1) / (kFcgThreads * per);
     return (unsigned)std::max<int64_t>(
         1, std::min<int64_t>({want, (int64_t)device_sm_count() * 4, (int64_t)kFcgMaxBlocks}));
 }
@@ -418,7 +453,8 @@ extern "C" int gbpcg_fcg_solve(const gbpcg_grid *grid, const float *w, const voi
             float *p = ring_p(cur), *q = ring_q(cur);
             rc = precondition();
             if (rc) return rc;
-            fcg_mdot_kernel<<<rb, kFcgThreads, 0, s>>>(n4, st, partials, r, z, d);
+            const unsigned groups = (unsigned)(nd + kMdotDirs) / kMdotDirs;  // of nd + 1 vectors
+            fcg_mdot_kernel<<<dim3(groups, rb), kFcgThreads, 0, s>>>(n4, st, partials, r, z, d);
             GB_CUDA(cudaGetLastError());
             fcg_combine_kernel<<<eb, 256, 0, s>>>(n4, st, z, d, p);
             GB_CUDA(cudaGetLastError());

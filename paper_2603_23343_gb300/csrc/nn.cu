@@ -438,28 +438,30 @@ __global__ void __launch_bounds__(256)
 // the warp's 128 (x0 - 1, x0 + 128).  Input plane m feeds output planes m + 1, m and m - 1; plane
 // m - 1 is then complete and written.  Per output: 27 CI multiply-adds from CI / 8 x 3 sixteen-byte
 // loads per input plane.
+// NJ: voxels per lane, 4, or 2 and 1 for rows of up to 64 and 32; `chunk`: planes per block, 16, or fewer
+// where that leaves SMs idle (64^3: 108 us with 16 planes and NJ = 4).
 constexpr int kC1Rows = 8, kC1Chunk = 16;
 
-template <int CI, typename TO>
+template <int CI, int NJ, typename TO>
 __global__ void __launch_bounds__(32 * kC1Rows, 2)
     conv3_c1_march_kernel(int X, int Y, int Z, const __nv_bfloat16 *__restrict__ in,
                           const __nv_bfloat16 *__restrict__ w, TO *__restrict__ out, int relu,
                           const __nv_bfloat16 *__restrict__ mask, int mstride, int moff, const double *scale,
-                          const float *__restrict__ vscale) {
+                          const float *__restrict__ vscale, int chunk) {
     static_assert(CI % 8 == 0, "channels come in 16-byte groups");
     __shared__ __align__(16) float ws[27 * CI];  // ws[t * CI + i], t = 9 (dz+1) + 3 (dy+1) + (dx+1)
     for (int e = threadIdx.x; e < 27 * CI; e += blockDim.x) ws[e] = __bfloat162float(w[e]);
     __syncthreads();
     const float sc = scale ? (float)*scale : 1.0f;
     const int lane = threadIdx.x & 31;
-    const int x0 = blockIdx.x * 128;
+    const int x0 = blockIdx.x * 32 * NJ;
     const int y = blockIdx.y * kC1Rows + (threadIdx.x >> 5);
-    const int zb = blockIdx.z * kC1Chunk, ze = min(Z, zb + kC1Chunk);
+    const int zb = blockIdx.z * chunk, ze = min(Z, zb + chunk);
     // the edge voxel lane 0 (x0 - 1, tap dx = -1) or lane 31 (x0 + 128, tap dx = +1) also forms
-    const int ex = lane == 0 ? x0 - 1 : x0 + 128, edx = lane == 0 ? 0 : 2;
-    float ap[4], ac[4], an[4];  // partial sums of output planes m - 1, m, m + 1 at x0 + lane + 32 j
+    const int ex = lane == 0 ? x0 - 1 : x0 + 32 * NJ, edx = lane == 0 ? 0 : 2;
+    float ap[NJ], ac[NJ], an[NJ];  // partial sums of output planes m - 1, m, m + 1 at x0 + lane + 32 j
 #pragma unroll
-    for (int j = 0; j < 4; ++j) ap[j] = ac[j] = an[j] = 0.0f;
+    for (int j = 0; j < NJ; ++j) ap[j] = ac[j] = an[j] = 0.0f;
     for (int m = zb - 1; m <= ze; ++m) {
         // which of the three output planes this input plane still feeds (uniform over the block)
         const bool fn = m + 1 >= zb && m + 1 < ze, fc = m >= zb && m < ze, fp = m - 1 >= zb && m - 1 < ze;
@@ -469,10 +471,10 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
                 const int yy = y + r - 1;
                 if (yy < 0 || yy >= Y) continue;
                 const __nv_bfloat16 *row = in + ((int64_t)m * Y + yy) * X * CI;
-                float P[4][3][3];  // [voxel j][dz + 1][dx + 1]
+                float P[NJ][3][3];  // [voxel j][dz + 1][dx + 1]
                 float E[3];        // the edge voxel's product with tap dx = edx, per dz + 1
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < NJ; ++j)
 #pragma unroll
                     for (int a3 = 0; a3 < 3; ++a3)
 #pragma unroll
@@ -481,9 +483,9 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
                 for (int a3 = 0; a3 < 3; ++a3) E[a3] = 0.0f;
 #pragma unroll
                 for (int cb = 0; cb < CI; cb += 8) {
-                    float v[4][8], ve[8];
+                    float v[NJ][8], ve[8];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < NJ; ++j) {
                         const int xx = x0 + lane + 32 * j;
                         if (xx < X) {
                             ld8(row + (int64_t)xx * CI + cb, v[j]);
@@ -508,7 +510,7 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
                             for (int c = 0; c < 8; ++c) {
                                 const float wv = wt[c];
 #pragma unroll
-                                for (int j = 0; j < 4; ++j) P[j][a3][d3] = fmaf(wv, v[j][c], P[j][a3][d3]);
+                                for (int j = 0; j < NJ; ++j) P[j][a3][d3] = fmaf(wv, v[j][c], P[j][a3][d3]);
                             }
                         }
                         const float *we = ws + (a3 * 9 + r * 3 + edx) * CI + cb;
@@ -525,13 +527,13 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
                     const float e_lo = __shfl_sync(0xffffffffu, E[a3], 0);
                     const float e_hi = __shfl_sync(0xffffffffu, E[a3], 31);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < NJ; ++j) {
                         float lo = __shfl_up_sync(0xffffffffu, P[j][a3][0], 1);
                         float hi = __shfl_down_sync(0xffffffffu, P[j][a3][2], 1);
                         const float lo_w = __shfl_sync(0xffffffffu, P[j > 0 ? j - 1 : 0][a3][0], 31);
-                        const float hi_w = __shfl_sync(0xffffffffu, P[j < 3 ? j + 1 : 3][a3][2], 0);
+                        const float hi_w = __shfl_sync(0xffffffffu, P[j < NJ - 1 ? j + 1 : NJ - 1][a3][2], 0);
                         if (lane == 0) lo = j > 0 ? lo_w : e_lo;
-                        if (lane == 31) hi = j < 3 ? hi_w : e_hi;
+                        if (lane == 31) hi = j < NJ - 1 ? hi_w : e_hi;
                         const float sum = P[j][a3][1] + lo + hi;
                         if (a3 == 0) an[j] += sum;       // dz = -1: output plane m + 1 reads input plane m
                         else if (a3 == 1) ac[j] += sum;
@@ -542,7 +544,7 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
         }
         if (fp && y < Y) {  // output plane m - 1 has all three input planes
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < NJ; ++j) {
                 const int xx = x0 + lane + 32 * j;
                 if (xx >= X) continue;
                 const int64_t v = ((int64_t)(m - 1) * Y + y) * X + xx;
@@ -553,7 +555,7 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
             }
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < NJ; ++j) {
             ap[j] = ac[j];
             ac[j] = an[j];
             an[j] = 0.0f;
@@ -567,10 +569,16 @@ static int conv_simt_launch(int X, int Y, int Z, const __nv_bfloat16 *in, const 
                             const float *vscale, cudaStream_t s) {
     if constexpr (CO == 1 && CI % 8 == 0) {
         {
-            const dim3 grid((unsigned)((X + 127) / 128), (unsigned)((Y + kC1Rows - 1) / kC1Rows),
-                            (unsigned)((Z + kC1Chunk - 1) / kC1Chunk));
-            conv3_c1_march_kernel<CI, TO><<<grid, 32 * kC1Rows, 0, s>>>(X, Y, Z, in, w, out, relu, mask, mstride,
-                                                                        moff, scale, vscale);
+            const int nj = X <= 32 ? 1 : X <= 64 ? 2 : 4;
+            const int64_t cols = (int64_t)((X + 32 * nj - 1) / (32 * nj)) * ((Y + kC1Rows - 1) / kC1Rows);
+            int chunk = kC1Chunk;
+            while (chunk > 4 && cols * ((Z + chunk - 1) / chunk) < 2 * (int64_t)device_sm_count()) chunk /= 2;
+            const dim3 grid((unsigned)((X + 32 * nj - 1) / (32 * nj)), (unsigned)((Y + kC1Rows - 1) / kC1Rows),
+                            (unsigned)((Z + chunk - 1) / chunk));
+            auto *fn = nj == 1   ? &conv3_c1_march_kernel<CI, 1, TO>
+                       : nj == 2 ? &conv3_c1_march_kernel<CI, 2, TO>
+                                 : &conv3_c1_march_kernel<CI, 4, TO>;
+            fn<<<grid, 32 * kC1Rows, 0, s>>>(X, Y, Z, in, w, out, relu, mask, mstride, moff, scale, vscale, chunk);
             cudaError_t e = cudaGetLastError();
             return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "conv3_c1_march launch");
         }
@@ -1026,9 +1034,15 @@ __global__ void __launch_bounds__(256)
                     int kbx, int kby, int kbz, __nv_bfloat16 *__restrict__ xin, double *scale) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;  // z: blockIdx.z, striding
     const int64_t n = (int64_t)X * Y * Z;
-    const double rms = sqrt(*ss / (double)n);
-    const float inv = rms > 0.0 ? (float)(1.0 / rms) : 1.0f;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *scale = rms;
+    // one thread's FP64 square root and division per block (every thread's took 30 us at 64^3)
+    __shared__ float s_inv;
+    if (threadIdx.x == 0) {
+        const double rms = sqrt(*ss / (double)n);
+        s_inv = rms > 0.0 ? (float)(1.0 / rms) : 1.0f;
+        if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *scale = rms;
+    }
+    __syncthreads();
+    const float inv = s_inv;
     if (x >= X) return;
     const int nbx = (X + kbx - 1) / kbx, nby = (Y + kby - 1) / kby;
     const int bx = x / kbx, by = y / kby;
