@@ -9,25 +9,27 @@
 // four fine face weights across it and the coarse diagonal is the sum of the
 // eight fine diagonals minus twice the twelve face weights inside the
 // aggregate.  Level 0 is the solver's operator (weights computed per point,
-// nothing stored); coarser levels store (w+x, w+y, w+z, D) per cell.
+// nothing stored but omega / D of block coefficients); coarser levels store
+// w+x, w+y, w+z, D and omega / D per cell, an array each.
 // Levels are added while every size is even and stays >= 4 (at most 8
 // levels).
 //
 // V-cycle z = M r (level l, right-hand side f; the coarsest level takes
 // kMgCoarseSweeps damped Jacobi sweeps from zero in one CTA):
-//   u = omega D^-1 f;  f_{l+1} = P^T (f - A u)        (two kernels)
+//   f_{l+1} = P^T (f - A u),  u = omega D^-1 f              (one kernel)
 //   e = V-cycle(l + 1)
 //   out = u' + omega D^-1 (f - A u'),  u' = u + sigma P e   (one kernel)
-// Levels of at most kMgTailCells cells, the coarsest with them, run these
-// steps inside one CTA (mg_tail_kernel) instead of a launch per step.
+// (u is formed from f wherever it is used).  Levels of at most kMgTailCells
+// cells, the coarsest with them, run these steps inside one CTA
+// (mg_tail_kernel) instead of a launch per step.
 // Pre- and post-smoothing are adjoint, so M is symmetric (positive definite
 // for omega < 1, 0 < sigma < 2).  omega = 0.9 and sigma = 1.5 took the
 // fewest iterations in a sweep of the oracle at 32^3 and 64^3.
 //
 // PCG with M: pass A of the Jacobi solver (p_k = z_k + beta p_{k-1} on the
 // fly, the deferred x update, p.Ap -> alpha), pass R (r -= alpha A p_k, r.r,
-// the convergence test and the replacement trigger), the V-cycle, and r.z
-// (-> beta); residual replacements store r = b - A x (FP64) and go through
+// the convergence test and the replacement trigger), and the V-cycle, whose
+// last kernel also sums r.z (-> beta); residual replacements store r = b - A x (FP64) and go through
 // the V-cycle again.  One CUDA graph with a device-driven loop.
 #include <algorithm>
 #include <cstring>
@@ -46,16 +48,24 @@ constexpr float kMgSigma = 1.5f;
 constexpr int kMgCoarseSweeps = 24;
 constexpr int64_t kMgMaxCoarsest = 32768;
 constexpr int kMgThreads = 256;
-constexpr int kMgCoarseThreads = 1024;
+constexpr int kMgTailThreads = 1024;
 constexpr int64_t kMgTailCells = 4096;  // levels this small run inside the one-CTA tail kernel
-constexpr int kMgSmemCells = 4096;      // a coarsest level this small sweeps in shared memory
+constexpr int kMgTailCtas = 8;          // the cluster that sweeps a larger coarsest level
+static_assert(kMgTailCells / 8 <= kMgTailThreads, "a tail of several levels sweeps a cell a thread");
+// coarsest cells a thread keeps the weights of in registers
+constexpr int kMgSweepCells = (int)((kMgTailCells + kMgTailThreads - 1) / kMgTailThreads);
+// shared memory of the tail; the sweeps' two buffers of every coarsest level of kMgMinCoarse planes or more fit
+constexpr size_t kMgTailSmem = 216 * 1024;
+constexpr int kMgTailLevels = 3;  // 4096 cells, 512, 64: a coarsest level holds 4^3 cells or more
+static_assert(kMgTailSmem >= 2 * 3 * (kMgMaxCoarsest / kMgMinCoarse) * sizeof(float), "sweep buffers");
 
 struct MgLevel {
     int nx, ny, nz;
-    float *f;         // right-hand side (level 0: the solver's r)
-    float *u;         // pre-smoothed iterate (coarsest: its solution)
-    float *w;         // post-smoothed result (level 0: z; coarsest: sweep scratch)
-    const float4 *W;  // levels >= 1: (w+x, w+y, w+z, D) per cell
+    float *f;        // right-hand side (level 0: the solver's r)
+    float *od;       // omega / D per point (constant level 0 above the tail: unused; coarsest: unused)
+    float *w;        // post-smoothed result (level 0: z; coarsest: the sweeps' result)
+    const float *wx, *wy, *wz, *D;  // levels >= 1 and a level 0 inside the tail: w+x, w+y, w+z and D per cell
+    int64_t m;                      // cells
 };
 
 struct MgArgs {
@@ -74,18 +84,23 @@ struct MgArgs {
 // 2^-23 (n + 1/2) / d < 1/(2d), so truncation gives the exact quotient.
 __device__ __forceinline__ int mg_div(int n, float rd) { return (int)(((float)n + 0.5f) * rd); }
 
-// Weights of point (i, j, k) of level l: w[0..5] = faces x-, x+, y-, y+, z-,
+// Weights of point (i, j, k) of a level: w[0..5] = faces x-, x+, y-, y+, z-,
 // z+ towards interior neighbours (0 across the boundary), and D.
-// Which weights a kernel computes: W_ANY decides at run time (level and
-// coefficient kind); the level kernels are compiled for one case each, so
-// that a Poisson solve's kernels carry none of the table path's registers.
-enum MgWeights { W_ANY = 0, W_CONST0 = 1, W_TAB0 = 2, W_STORED = 3 };
+__device__ __forceinline__ void mg_weights_stored(const MgLevel &L, int i, int j, int k, float w[6], float &D) {
+    const int64_t c = ((int64_t)k * L.ny + j) * L.nx + i;
+    w[1] = L.wx[c];
+    w[3] = L.wy[c];
+    w[5] = L.wz[c];
+    D = L.D[c];
+    w[0] = i > 0 ? L.wx[c - 1] : 0.f;
+    w[2] = j > 0 ? L.wy[c - L.nx] : 0.f;
+    w[4] = k > 0 ? L.wz[c - (int64_t)L.nx * L.ny] : 0.f;
+}
 
-template <int WK = W_ANY>
 __device__ __forceinline__ void mg_weights(const MgArgs &a, int l, int i, int j, int k, float w[6], float &D) {
     const MgLevel &L = a.lv[l];
-    if (WK == W_CONST0 || WK == W_TAB0 || (WK == W_ANY && l == 0)) {
-        if (WK == W_TAB0 || (WK == W_ANY && a.block && a.tab)) {
+    if (l == 0) {
+        if (a.block) {
             // the face table holds the harmonic means (or the block's k on the domain boundary):
             // bitwise the weights of OpBlock::weights, without their divisions
             const OpBlock &o = a.ob;
@@ -100,58 +115,27 @@ __device__ __forceinline__ void mg_weights(const MgArgs &a, int l, int i, int j,
             w[3] = o.cy * (iy == o.kby - 1 ? t1.x : kc);
             w[4] = o.cz * (iz == 0 ? t1.y : kc);
             w[5] = o.cz * (iz == o.kbz - 1 ? t1.z : kc);
-        } else if (WK == W_ANY && a.block) {
-            a.ob.weights(i, j, k, w);
         } else {
             w[0] = w[1] = a.ob.cx;
             w[2] = w[3] = a.ob.cy;
             w[4] = w[5] = a.ob.cz;
         }
         D = ((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]);
-        // The level kernels (WK != W_ANY) load stencil inputs outside the grid as zero, so a
-        // boundary face's weight multiplies zero there and need not be cleared; the run-time
-        // form clears it (its callers index neighbours only where the weight is nonzero).
-        if (WK == W_ANY) {
-            if (i == 0) w[0] = 0.f;
-            if (i == L.nx - 1) w[1] = 0.f;
-            if (j == 0) w[2] = 0.f;
-            if (j == L.ny - 1) w[3] = 0.f;
-            if (k == 0) w[4] = 0.f;
-            if (k == L.nz - 1) w[5] = 0.f;
-        }
+        if (i == 0) w[0] = 0.f;
+        if (i == L.nx - 1) w[1] = 0.f;
+        if (j == 0) w[2] = 0.f;
+        if (j == L.ny - 1) w[3] = 0.f;
+        if (k == 0) w[4] = 0.f;
+        if (k == L.nz - 1) w[5] = 0.f;
         return;
     }
-    const int64_t c = ((int64_t)k * L.ny + j) * L.nx + i;
-    const float4 W = __ldg(L.W + c);
-    w[1] = W.x;
-    w[3] = W.y;
-    w[5] = W.z;
-    D = W.w;
-    w[0] = i > 0 ? __ldg(&L.W[c - 1].x) : 0.f;
-    w[2] = j > 0 ? __ldg(&L.W[c - L.nx].y) : 0.f;
-    w[4] = k > 0 ? __ldg(&L.W[c - (int64_t)L.nx * L.ny].z) : 0.f;
+    mg_weights_stored(L, i, j, k, w, D);
 }
 
-// sum over interior neighbours of w_f v(nb); v(flat index, i, j, k) of the neighbour
-template <typename V>
-__device__ __forceinline__ float mg_offdiag(const MgLevel &L, int i, int j, int k, int64_t c, const float w[6], V v) {
-    const int64_t sy = L.nx, sz = (int64_t)L.nx * L.ny;
-    float s = 0.f;
-    if (w[0] != 0.f) s = fmaf(w[0], v(c - 1, i - 1, j, k), s);
-    if (w[1] != 0.f) s = fmaf(w[1], v(c + 1, i + 1, j, k), s);
-    if (w[2] != 0.f) s = fmaf(w[2], v(c - sy, i, j - 1, k), s);
-    if (w[3] != 0.f) s = fmaf(w[3], v(c + sy, i, j + 1, k), s);
-    if (w[4] != 0.f) s = fmaf(w[4], v(c - sz, i, j, k - 1), s);
-    if (w[5] != 0.f) s = fmaf(w[5], v(c + sz, i, j, k + 1), s);
-    return s;
-}
+__device__ __forceinline__ bool mg_stand_down(const SolveState *st) { return st && st->done; }
 
-__device__ __forceinline__ bool mg_stand_down(const MgArgs &a) { return a.st && a.st->done; }
-
-// Launch geometry of the level kernels: a block is bx threads along x times
-// by rows along y and marches through zper planes; x, y and z come from the
-// block and thread indices (no integer division per point), and there are
-// about as many blocks as two waves of resident CTAs.
+// Launch geometry of the Galerkin kernel: a block is bx threads along x times
+// by rows along y and marches through zper planes.
 struct MgLaunch {
     dim3 grid, block;
     int zper;
@@ -167,380 +151,867 @@ inline MgLaunch mg_launch(int nx, int ny, int nz) {
                     dim3((unsigned)bx, (unsigned)by), zper};
 }
 
-// Four consecutive floats (16-byte aligned) <-> registers.
-__device__ __forceinline__ void ld4f(const float *p, float v[4]) {
-    const float4 t = *reinterpret_cast<const float4 *>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+// ------------------------------------------------- level kernels --
+//
+// A level above the tail takes two kernels: the restriction (with the
+// pre-smoothing u = (omega / D) f formed from f at every use, so u is neither
+// stored nor read back) and the post-smoothing.  Both are bound by memory if
+// the instructions per point stay near 30, so a thread keeps what it can:
+//   - V neighbouring points of a row (V = 4; 2 where nx % 4 == 2), marching
+//     along z with the planes before and after in registers;
+//   - lanes 0..15 of a warp hold 16 such segments of row 2J, lanes 16..31
+//     those of row 2J + 1: the x neighbours and the row inside the pair come
+//     by shuffle, only the one row outside the pair is loaded;
+//   - segments are numbered along the plane (row pair times segments of a
+//     row), so rows of any length fill the warps;
+//   - level-0 block weights are read from the face table once per block of
+//     planes, the stored weights of coarser levels are arrays per face
+//     direction read as vectors.
+// Loads of the plane after next are issued before the current plane is
+// computed.  Block coefficients at 256^3 (ncu): pre-smoothing and restriction
+// 30 + 68 us in two kernels -> 65 us, post-smoothing 115 us, and a pass of 20
+// us for r.z after it -> 81 us with r.z inside; the stored 128^3 level 64 ->
+// 39 us for both ways.
+
+// V consecutive floats (V * 4 byte aligned) -> registers
+template <int V>
+__device__ __forceinline__ void ldv(const float *p, float v[V]) {
+    if constexpr (V == 4) {
+        const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else {
+        const float2 t = __ldg(reinterpret_cast<const float2 *>(p));
+        v[0] = t.x; v[1] = t.y;
+    }
 }
 
-// u = omega D^-1 f at level l; V consecutive points per thread (V = 4 needs nx % 4 == 0)
+// What one launch of a level kernel reads of the hierarchy: a launch's
+// parameters are read through a cold constant cache, a line at a time.
+struct MgStep {
+    const SolveState *st;
+    MgLevel L;
+    float *c;  // the coarse level's f (restriction) or w (post-smoothing)
+    OpBlock ob;
+    const float4 *tab;
+    float rkbx, rkby, rkbz;
+};
+
+// Kind of weights a level kernel is compiled for.  W_TABV: block
+// coefficients whose block edge along x is a multiple of V, so that the V
+// points of a thread lie in one block.
+enum MgWeights { W_CONST0 = 1, W_TABV = 2, W_TAB0 = 3, W_STORED = 4 };
+
+// A thread's segment: V points from i0 of row j = 2J + hi.
+template <int V>
+struct MgSeg {
+    int i0, j;
+    bool hi, live, el, er, eo;  // eo: the row outside the pair exists; el / er: x neighbours to be loaded
+    bool xl0, xr0;              // the row starts / ends here
+    int64_t c;                  // flat index at plane 0
+    int dro;                    // offset of the row outside the pair
+    __device__ __forceinline__ MgSeg(const MgLevel &L, unsigned wseg) {  // the warp's 16 segments per row: 16 wseg ..
+        const int lane = threadIdx.x & 31, q = L.nx / V, np = q * (L.ny / 2);
+        int p = (int)wseg * 16 + (lane & 15);
+        live = p < np;
+        p = min(p, np - 1);
+        const int J = p / q;
+        hi = lane >= 16;
+        i0 = (p - J * q) * V;
+        j = 2 * J + (hi ? 1 : 0);
+        xl0 = i0 == 0;
+        xr0 = i0 + V >= L.nx;
+        el = (lane & 15) == 0 && !xl0;
+        er = (lane & 15) == 15 && !xr0;
+        eo = hi ? j + 1 < L.ny : j > 0;
+        dro = hi ? L.nx : -L.nx;
+        c = (int64_t)j * L.nx + i0;
+    }
+};
+
+// The weights of a segment's points at the current plane: w[m][0..5] = x-,
+// x+, the row inside the pair, the row outside it, z-, z+.  Values outside
+// the grid are read as 0, so boundary weights need not be cleared.
 template <int V, int WK>
-__global__ void __launch_bounds__(kMgThreads) mg_pre_kernel(const MgArgs a, int l, int zper) {
-    if (mg_stand_down(a)) return;
-    const MgLevel &L = a.lv[l];
-    const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V, j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i0 >= L.nx || j >= L.ny) return;
-    const int k0 = blockIdx.z * zper, k1 = min(L.nz, k0 + zper);
-    const float *__restrict__ f = L.f;
-    float *__restrict__ u = L.u;
-    for (int k = k0; k < k1; ++k) {
-        const int64_t c = ((int64_t)k * L.ny + j) * L.nx + i0;
-        float fv[V], out[V];
-        if constexpr (V == 4) ld4f(f + c, fv);
-        else fv[0] = f[c];
+struct MgCol {
+    float wc, wxl, wxr, win, wout, wz, wzl, wzh;      // W_TABV (wc, win, wout, wz also W_CONST0)
+    float px[WK == W_TAB0 ? V : 1][8];                // W_TAB0: the same per point
+    float sx[V], sxl, si[V], so[V], szm[V], sz[V], sD[V];  // W_STORED
+    int iz;
+
+    __device__ __forceinline__ void table(const MgStep &a, int i, int j, int k, bool hi, float t[8], bool last_of_seg) {
+        const OpBlock &o = a.ob;
+        const int bx = mg_div(i, a.rkbx), by = mg_div(j, a.rkby), bz = mg_div(k, a.rkbz);
+        const int ix = i - bx * o.kbx, iy = j - by * o.kby;
+        const float4 *tb = a.tab + 2 * (((int64_t)bz * o.nby + by) * o.nbx + bx);
+        const float4 t0 = __ldg(tb), t1 = __ldg(tb + 1);
+        const float kc = t0.x;
+        t[0] = o.cx * kc;
+        t[1] = o.cx * (ix == 0 ? t0.y : kc);
+        t[2] = o.cx * (ix + (last_of_seg ? V - 1 : 0) == o.kbx - 1 ? t0.z : kc);
+        const float ylo = o.cy * (iy == 0 ? t0.w : kc), yhi = o.cy * (iy == o.kby - 1 ? t1.x : kc);
+        t[3] = hi ? ylo : yhi;
+        t[4] = hi ? yhi : ylo;
+        t[5] = o.cz * kc;
+        t[6] = o.cz * t1.y;
+        t[7] = o.cz * t1.z;
+    }
+    __device__ __forceinline__ void block_at(const MgStep &a, const MgSeg<V> &s, int k) {
+        if constexpr (WK == W_TABV) {
+            float t[8];
+            table(a, s.i0, s.j, k, s.hi, t, true);
+            wc = t[0]; wxl = t[1]; wxr = t[2]; win = t[3]; wout = t[4]; wz = t[5]; wzl = t[6]; wzh = t[7];
+        } else if constexpr (WK == W_TAB0) {
+#pragma unroll
+            for (int m = 0; m < V; ++m) table(a, s.i0 + m, s.j, k, s.hi, px[m], false);
+        }
+    }
+    // the weights of the planes from k on
+    __device__ __forceinline__ void start(const MgStep &a, const MgLevel &L, const MgSeg<V> &s, int k) {
+        if constexpr (WK == W_CONST0) {
+            wc = a.ob.cx;
+            win = wout = a.ob.cy;
+            wz = a.ob.cz;
+        } else if constexpr (WK == W_STORED) {
+#pragma unroll
+            for (int m = 0; m < V; ++m) sz[m] = 0.f;
+            if (k > 0) ldv<V>(L.wz + s.c + (int64_t)(k - 1) * L.nx * L.ny, sz);
+        } else {
+            iz = k - mg_div(k, a.rkbz) * a.ob.kbz - 1;
+            block_at(a, s, k);
+        }
+    }
+    // plane k (called for consecutive k from start's)
+    __device__ __forceinline__ void plane(const MgStep &a, const MgLevel &L, const MgSeg<V> &s, int64_t c, int k) {
+        if constexpr (WK == W_TABV || WK == W_TAB0) {
+            if (++iz == a.ob.kbz) {
+                iz = 0;
+                block_at(a, s, k);
+            }
+        } else if constexpr (WK == W_STORED) {
+            float y[V], yo[V];
+#pragma unroll
+            for (int m = 0; m < V; ++m) {
+                szm[m] = sz[m];
+                yo[m] = 0.f;
+            }
+            ldv<V>(L.wx + c, sx);
+            ldv<V>(L.wy + c, y);
+            ldv<V>(L.wz + c, sz);
+            ldv<V>(L.D + c, sD);
+            if (!s.hi && s.eo) ldv<V>(L.wy + c - L.nx, yo);
+            const float xl = s.el ? __ldg(L.wx + c - 1) : 0.f;
+            const float xs = __shfl_up_sync(0xffffffffu, sx[V - 1], 1);
+            sxl = s.xl0 ? 0.f : s.el ? xl : xs;
+#pragma unroll
+            for (int m = 0; m < V; ++m) {
+                const float yp = __shfl_xor_sync(0xffffffffu, y[m], 16);
+                si[m] = s.hi ? yp : y[m];
+                so[m] = s.hi ? y[m] : yo[m];
+            }
+        }
+    }
+    __device__ __forceinline__ void get(const MgStep &a, int m, float w[6], float &D) const {
+        if constexpr (WK == W_CONST0) {
+            w[0] = w[1] = wc;
+            w[2] = win;
+            w[3] = wout;
+            w[4] = w[5] = wz;
+            D = ((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]);
+        } else if constexpr (WK == W_TABV) {
+            w[0] = m == 0 ? wxl : wc;
+            w[1] = m == V - 1 ? wxr : wc;
+            w[2] = win;
+            w[3] = wout;
+            w[4] = iz == 0 ? wzl : wz;
+            w[5] = iz == a.ob.kbz - 1 ? wzh : wz;
+            D = ((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]);
+        } else if constexpr (WK == W_TAB0) {
+            w[0] = px[m][1];
+            w[1] = px[m][2];
+            w[2] = px[m][3];
+            w[3] = px[m][4];
+            w[4] = iz == 0 ? px[m][6] : px[m][5];
+            w[5] = iz == a.ob.kbz - 1 ? px[m][7] : px[m][5];
+            D = ((w[0] + w[1]) + (w[2] + w[3])) + (w[4] + w[5]);
+        } else {
+            w[0] = m == 0 ? sxl : sx[m > 0 ? m - 1 : 0];
+            w[1] = sx[m];
+            w[2] = si[m];
+            w[3] = so[m];
+            w[4] = szm[m];
+            w[5] = sz[m];
+            D = sD[m];
+        }
+    }
+};
+
+// The march both level kernels make: for the planes [k0, k1) of a segment,
+// the iterate v (POST: u + sigma P e, else u = (omega / D) f) at the segment
+// and its neighbours (0 outside the grid), and body(k, c, A v, v, f,
+// omega / D) per plane.  What a plane reads is loaded one plane ahead (its
+// own row two ahead: the z neighbour).
+template <int V, int WK, bool POST, typename Body>
+__device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int k0, int k1, Body body) {
+    const MgLevel &L = a.L;
+    const float *e = a.c;
+    const float *f = L.f, *od = L.od;
+    const int64_t sz = (int64_t)L.nx * L.ny;
+    const int cnx = L.nx / 2;
+    const int64_t csz = (int64_t)cnx * (L.ny / 2);
+    const float wd = kMgOmega / (((a.ob.cx + a.ob.cx) + (a.ob.cy + a.ob.cy)) + (a.ob.cz + a.ob.cz));  // W_CONST0
+    struct Raw {
+        float f[V], o[V], e[V / 2];
+    };
+    // the V values at flat index c, whose parents start at flat index pc
+    auto fetch = [&](Raw &r, int64_t c, int64_t pc) {
+        ldv<V>(f + c, r.f);
+        if constexpr (WK == W_CONST0) {
+#pragma unroll
+            for (int m = 0; m < V; ++m) r.o[m] = wd;
+        } else {
+            ldv<V>(od + c, r.o);
+        }
+        if constexpr (POST) {
+            if constexpr (V == 4) {
+                const float2 t = __ldg(reinterpret_cast<const float2 *>(e + pc));
+                r.e[0] = t.x;
+                r.e[1] = t.y;
+            } else {
+                r.e[0] = __ldg(e + pc);
+            }
+        }
+    };
+    auto iterate = [&](const Raw &r, float v[V]) {
+#pragma unroll
+        for (int m = 0; m < V; ++m) {
+            v[m] = r.f[m] * r.o[m];
+            if constexpr (POST) v[m] = fmaf(kMgSigma, r.e[m >> 1], v[m]);
+        }
+    };
+    // flat index of the parents of this row at plane k, of the row outside the pair, of the edge point
+    auto par = [&](int k) { return (int64_t)(k >> 1) * csz; };
+    const int p0 = (s.j >> 1) * cnx + (s.i0 >> 1), po = p0 + (s.hi ? cnx : -cnx);
+    const bool ed = s.el || s.er;  // the point beside the segment that no lane of the half holds
+    const int de = s.el ? -1 : V, pe = (s.j >> 1) * cnx + ((s.i0 + de) >> 1);
+    struct Edge {
+        float f = 0.f, o = 0.f, e = 0.f;
+    };
+    auto edge = [&](Edge &g, int64_t c, int k) {
+        if (!ed) return;
+        g.f = __ldg(f + c + de);
+        g.o = WK == W_CONST0 ? wd : __ldg(od + c + de);
+        if constexpr (POST) g.e = __ldg(e + par(k) + pe);
+    };
+    MgCol<V, WK> col;
+    col.start(a, L, s, k0);
+    int64_t c = (int64_t)s.c + (int64_t)k0 * sz;
+    Raw rc, rn, ro;
+    Edge g;
+    float vm[V], vc[V];
+    const int klast = min(k1, L.nz - 1);  // the last plane read
+    fetch(rc, c, par(k0) + p0);
+    if (s.eo) fetch(ro, c + s.dro, par(k0) + po);
+    edge(g, c, k0);
+    if (k0 + 1 <= klast) fetch(rn, c + sz, par(k0 + 1) + p0);
+#pragma unroll
+    for (int m = 0; m < V; ++m) vm[m] = 0.f;
+    if (k0 > 0) {
+        Raw rm;
+        fetch(rm, c - sz, par(k0 - 1) + p0);
+        iterate(rm, vm);
+    }
+    iterate(rc, vc);
+    for (int k = k0; k < k1; ++k, c += sz) {
+        Raw r2, ron;
+        Edge gn;
+        if (k + 2 <= klast) fetch(r2, c + 2 * sz, par(k + 2) + p0);
+        if (k + 1 < k1) {
+            if (s.eo) fetch(ron, c + sz + s.dro, par(k + 1) + po);
+            edge(gn, c + sz, k + 1);
+        }
+        col.plane(a, L, s, c, k);
+        float vn[V], vo[V], vi[V];
+#pragma unroll
+        for (int m = 0; m < V; ++m) vn[m] = vo[m] = 0.f;
+        if (k + 1 < L.nz) iterate(rn, vn);
+        if (s.eo) iterate(ro, vo);
+        float ve = g.f * g.o;
+        if constexpr (POST) ve = fmaf(kMgSigma, g.e, ve);
+#pragma unroll
+        for (int m = 0; m < V; ++m) vi[m] = __shfl_xor_sync(0xffffffffu, vc[m], 16);
+        const float xls = __shfl_up_sync(0xffffffffu, vc[V - 1], 1), xrs = __shfl_down_sync(0xffffffffu, vc[0], 1);
+        const float xl = s.xl0 ? 0.f : s.el ? ve : xls, xr = s.xr0 ? 0.f : s.er ? ve : xrs;
+        float av[V];
 #pragma unroll
         for (int m = 0; m < V; ++m) {
             float w[6], D;
-            mg_weights<WK>(a, l, i0 + m, j, k, w, D);
-            out[m] = fv[m] * __fdividef(kMgOmega, D);
+            col.get(a, m, w, D);
+            float off = w[0] * (m == 0 ? xl : vc[m > 0 ? m - 1 : 0]);
+            off = fmaf(w[1], m == V - 1 ? xr : vc[m < V - 1 ? m + 1 : 0], off);
+            off = fmaf(w[2], vi[m], off);
+            off = fmaf(w[3], vo[m], off);
+            off = fmaf(w[4], vm[m], off);
+            off = fmaf(w[5], vn[m], off);
+            av[m] = fmaf(D, vc[m], -off);
         }
-        if constexpr (V == 4) *reinterpret_cast<float4 *>(u + c) = make_float4(out[0], out[1], out[2], out[3]);
-        else u[c] = out[0];
+        body(k, c, av, vc, rc.f, rc.o);
+#pragma unroll
+        for (int m = 0; m < V; ++m) {
+            vm[m] = vc[m];
+            vc[m] = vn[m];
+        }
+        rc = rn;
+        rn = r2;
+        ro = ron;
+        g = gn;
     }
 }
 
-// The stencil input of V consecutive points of a row and of their neighbours:
-// centre values c[V], the x neighbours left of point 0 and right of point
-// V-1, the rows above / below and the planes before / after.  Values outside
-// the grid read as 0 (their weights are 0 anyway).
-template <int V>
-struct Nbr {
-    float c[V], xl, xr, ym[V], yp[V], zm[V], zp[V];
+// One warp's restriction of the coarse planes [K0, K1) of its segments.
+template <int V, int WK>
+__device__ __forceinline__ void mg_restrict_warp(const MgStep &a, unsigned wseg, int K0, int K1) {
+    const int cnx = a.L.nx / 2;
+    const int64_t csz = (int64_t)cnx * (a.L.ny / 2);
+    const MgSeg<V> s(a.L, wseg);
+    float sum[V / 2];
+    float *fc = a.c + (int64_t)(s.j >> 1) * cnx + (s.i0 >> 1);
+    mg_march<V, WK, false>(a, s, 2 * K0, 2 * K1,
+                                 [&](int k, int64_t, const float *av, const float *, const float *f, const float *) {
+                                     float r[V / 2];
+#pragma unroll
+                                     for (int m = 0; m < V / 2; ++m) {
+                                         r[m] = (f[2 * m] - av[2 * m]) + (f[2 * m + 1] - av[2 * m + 1]);
+                                         r[m] += __shfl_xor_sync(0xffffffffu, r[m], 16);
+                                     }
+                                     if (!(k & 1)) {
+#pragma unroll
+                                         for (int m = 0; m < V / 2; ++m) sum[m] = r[m];
+                                         return;
+                                     }
+                                     if (!s.live || s.hi) return;
+                                     float *o = fc + (k >> 1) * csz;
+                                     if constexpr (V == 4)
+                                         *reinterpret_cast<float2 *>(o) = make_float2(sum[0] + r[0], sum[1] + r[1]);
+                                     else
+                                         o[0] = sum[0] + r[0];
+                                 });
+}
+
+// One warp's post-smoothing of the planes [k0, k1) of its segments; returns
+// its points' sum of f.out.
+template <int V, int WK>
+__device__ __forceinline__ float mg_post_warp(const MgStep &a, unsigned wseg, int k0, int k1) {
+    const MgSeg<V> s(a.L, wseg);
+    float *out = a.L.w;
+    float acc = 0.f;
+    mg_march<V, WK, true>(a, s, k0, k1,
+                                [&](int, int64_t c, const float *av, const float *v, const float *f, const float *o) {
+                                    float r[V];
+#pragma unroll
+                                    for (int m = 0; m < V; ++m) r[m] = fmaf(o[m], f[m] - av[m], v[m]);
+                                    if (!s.live) return;
+                                    if constexpr (V == 4) {
+                                        *reinterpret_cast<float4 *>(out + c) = make_float4(r[0], r[1], r[2], r[3]);
+                                    } else {
+                                        *reinterpret_cast<float2 *>(out + c) = make_float2(r[0], r[1]);
+                                    }
+#pragma unroll
+                                    for (int m = 0; m < V; ++m) acc = fmaf(f[m], r[m], acc);
+                                });
+    return acc;
+}
+
+// f_{l+1} = P^T (f - A u), u = (omega / D) f; a block marches kper coarse planes.
+template <int V, int WK>
+__global__ void __launch_bounds__(kMgThreads) mg_restrict_kernel(const MgStep a, unsigned nblk, int kper) {
+    if (mg_stand_down(a.st)) return;
+    const int K0 = blockIdx.y * kper, K1 = min(a.L.nz / 2, K0 + kper);
+    for (unsigned blk = blockIdx.x; blk < nblk; blk += gridDim.x)
+        mg_restrict_warp<V, WK>(a, blk * (kMgThreads / 32) + (threadIdx.x >> 5), K0, K1);
+}
+
+// The scalars a V-cycle inside a solve ends with: r.z -> beta (the first time
+// only r.z), breakdown, the loop condition.
+struct MgDot {
+    SolveState *st;
+    double *partials;
+    int init;
+    cudaGraphConditionalHandle cond;
+    int use_cond;
 };
-template <int V, typename GetV, typename Get1>
-__device__ __forceinline__ void load_nbr(const MgLevel &L, int i0, int j, int k, GetV getv, Get1 get1, Nbr<V> &n) {
-    getv(i0, j, k, n.c);
-    n.xl = i0 > 0 ? get1(i0 - 1, j, k) : 0.f;
-    n.xr = i0 + V < L.nx ? get1(i0 + V, j, k) : 0.f;
-#pragma unroll
-    for (int m = 0; m < V; ++m) n.ym[m] = n.yp[m] = n.zm[m] = n.zp[m] = 0.f;
-    if (j > 0) getv(i0, j - 1, k, n.ym);
-    if (j < L.ny - 1) getv(i0, j + 1, k, n.yp);
-    if (k > 0) getv(i0, j, k - 1, n.zm);
-    if (k < L.nz - 1) getv(i0, j, k + 1, n.zp);
-}
-
-// (A v)_m = D v_m - sum of the interior neighbours' w v for point m of a row segment
-template <int V>
-__device__ __forceinline__ float apply_m(const Nbr<V> &n, int m, const float w[6], float D) {
-    const float xm = m == 0 ? n.xl : n.c[m - 1];
-    const float xp = m == V - 1 ? n.xr : n.c[m + 1];
-    float off = w[0] * xm;
-    off = fmaf(w[1], xp, off);
-    off = fmaf(w[2], n.ym[m], off);
-    off = fmaf(w[3], n.yp[m], off);
-    off = fmaf(w[4], n.zm[m], off);
-    off = fmaf(w[5], n.zp[m], off);
-    return fmaf(D, n.c[m], -off);
-}
-
-// f_{l+1} = P^T (f - A u).  V = 1: one thread per coarse cell; V = 2: two
-// neighbouring coarse cells per thread, their four fine columns read as one
-// 16-byte vector per fine row (needs nx % 4 == 0).
-// FROM_F (level 0 with constant coefficients, where D is one number): the
-// pre-smoothed u = (omega / D) f is formed from f at every use instead of
-// being read, and the pre-smoothing kernel is not run (one multiply per
-// value; it rounds once more than omega f / D).
-template <int V, int WK, bool FROM_F = false>
-__global__ void __launch_bounds__(kMgThreads) mg_restrict_kernel(const MgArgs a, int l, int zper) {
-    if (mg_stand_down(a)) return;
-    const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
-    const int I0 = (blockIdx.x * blockDim.x + threadIdx.x) * V, J = blockIdx.y * blockDim.y + threadIdx.y;
-    if (I0 >= C.nx || J >= C.ny) return;
-    const int K0 = blockIdx.z * zper, K1 = min(C.nz, K0 + zper);
-    const float *__restrict__ u = FROM_F ? L.f : L.u;
-    const float *__restrict__ f = L.f;
-    float *__restrict__ fc = C.f;
-    constexpr int FV = 2 * V;  // fine points per fine row
-    const float wd = kMgOmega / (2.0f * ((a.ob.cx + a.ob.cy) + a.ob.cz));  // FROM_F: omega / D, D constant
-    auto toU = [&](float x) { return FROM_F ? x * wd : x; };
-    auto at = [&](int i, int j, int k) { return ((int64_t)k * L.ny + j) * L.nx + i; };
-    auto getv = [&](int i, int j, int k, float *v) {
-        const int64_t q = at(i, j, k);
-        if constexpr (FV == 4) ld4f(u + q, v);
-        else { v[0] = u[q]; v[1] = u[q + 1]; }
-#pragma unroll
-        for (int m = 0; m < FV; ++m) v[m] = toU(v[m]);
-    };
-    auto get1 = [&](int i, int j, int k) { return toU(u[at(i, j, k)]); };
-    for (int K = K0; K < K1; ++K) {
-        float sum[V];
-#pragma unroll
-        for (int m = 0; m < V; ++m) sum[m] = 0.f;
-#pragma unroll
-        for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-            for (int dy = 0; dy < 2; ++dy) {
-                const int i0 = 2 * I0, j = 2 * J + dy, k = 2 * K + dz;
-                const int64_t c0 = ((int64_t)k * L.ny + j) * L.nx + i0;
-                Nbr<FV> n;
-                load_nbr<FV>(L, i0, j, k, getv, get1, n);
-                float fv[FV];
-                if constexpr (FV == 4) ld4f(f + c0, fv);
-                else { fv[0] = f[c0]; fv[1] = f[c0 + 1]; }
-#pragma unroll
-                for (int m = 0; m < FV; ++m) {
-                    float w[6], D;
-                    mg_weights<WK>(a, l, i0 + m, j, k, w, D);
-                    sum[m >> 1] += fv[m] - apply_m<FV>(n, m, w, D);
-                }
-            }
-        const int64_t cc = ((int64_t)K * C.ny + J) * C.nx + I0;
-        if constexpr (V == 2) *reinterpret_cast<float2 *>(fc + cc) = make_float2(sum[0], sum[1]);
-        else fc[cc] = sum[0];
+__device__ __forceinline__ void mg_rz_finish(const MgDot &d, double rz) {
+    SolveState *st = d.st;
+    if (!isfinite(rz) || !(rz > 0.0)) {
+        st->done = 1;
+        st->status = GBPCG_BREAKDOWN;
+    } else {
+        if (!d.init) st->beta = rz / st->rzm;
+        st->rz = rz;
+        st->rzm = rz;
     }
+    if (d.use_cond) cudaGraphSetConditional(d.cond, st->done ? 0u : 1u);
 }
 
 // out = u' + omega D^-1 (f - A u'), u' = u + sigma P e with e the level-(l+1)
-// result, formed at every stencil input; V consecutive points per thread.
-template <int V, int WK, bool FROM_F = false>
+// result.  DOT (level 0 inside a solve): also f.out, r.z of the solver,
+// instead of a pass of its own over both vectors.
+template <int V, int WK, bool DOT>
 __global__ void __launch_bounds__(kMgThreads)
-    mg_post_kernel(const MgArgs a, int l, const float *__restrict__ e, int zper) {
-    if (mg_stand_down(a)) return;
-    const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
-    const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V, j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i0 >= L.nx || j >= L.ny) return;
-    const int k0 = blockIdx.z * zper, k1 = min(L.nz, k0 + zper);
-    const float *__restrict__ u = FROM_F ? L.f : L.u;  // FROM_F: u = omega f / D (see mg_restrict_kernel)
-    const float wd = kMgOmega / (2.0f * ((a.ob.cx + a.ob.cy) + a.ob.cz));
-    const float wd_const = kMgOmega / (((a.ob.cx + a.ob.cx) + (a.ob.cy + a.ob.cy)) + (a.ob.cz + a.ob.cz));
-    auto toU = [&](float x) { return FROM_F ? x * wd : x; };
-    const float *__restrict__ f = L.f;
-    float *__restrict__ out = L.w;
-    for (int k = k0; k < k1; ++k) {
-        const int64_t c0 = ((int64_t)k * L.ny + j) * L.nx + i0;
-        // u' = u + sigma e[parent] at fine points (i, j, k) (V of them from i, i a multiple of V)
-        auto fine = [&](int i, int jj, int kk) { return ((int64_t)kk * L.ny + jj) * L.nx + i; };
-        auto parent = [&](int i, int jj, int kk) {
-            return ((int64_t)(kk >> 1) * C.ny + (jj >> 1)) * C.nx + (i >> 1);
-        };
-        auto getv = [&](int i, int jj, int kk, float *v) {
-            const int64_t q = fine(i, jj, kk), pc = parent(i, jj, kk);
-            if constexpr (V == 4) {
-                float uv[4];
-                ld4f(u + q, uv);
-                const float2 ep = __ldg(reinterpret_cast<const float2 *>(e + pc));
-                v[0] = fmaf(kMgSigma, ep.x, toU(uv[0]));
-                v[1] = fmaf(kMgSigma, ep.x, toU(uv[1]));
-                v[2] = fmaf(kMgSigma, ep.y, toU(uv[2]));
-                v[3] = fmaf(kMgSigma, ep.y, toU(uv[3]));
-            } else {
-                v[0] = fmaf(kMgSigma, __ldg(e + pc), toU(u[q]));
-            }
-        };
-        auto get1 = [&](int i, int jj, int kk) {
-            return fmaf(kMgSigma, __ldg(e + parent(i, jj, kk)), toU(u[fine(i, jj, kk)]));
-        };
-        Nbr<V> n;
-        load_nbr<V>(L, i0, j, k, getv, get1, n);
-        float fv[V], res[V];
-        if constexpr (V == 4) ld4f(f + c0, fv);
-        else fv[0] = f[c0];
-#pragma unroll
-        for (int m = 0; m < V; ++m) {
-            float w[6], D;
-            mg_weights<WK>(a, l, i0 + m, j, k, w, D);
-            // omega / D: one number for constant coefficients (hoisted), else the fast division
-            const float od = WK == W_CONST0 ? wd_const : __fdividef(kMgOmega, D);
-            res[m] = fmaf(od, fv[m] - apply_m<V>(n, m, w, D), n.c[m]);
-        }
-        if constexpr (V == 4) *reinterpret_cast<float4 *>(out + c0) = make_float4(res[0], res[1], res[2], res[3]);
-        else out[c0] = res[0];
+    mg_post_kernel(const MgStep a, unsigned nblk, int kper, const MgDot d) {
+    if (mg_stand_down(a.st)) return;
+    const int k0 = blockIdx.y * kper, k1 = min(a.L.nz, k0 + kper);
+    float acc[1] = {0.f};
+    for (unsigned blk = blockIdx.x; blk < nblk; blk += gridDim.x)
+        acc[0] += mg_post_warp<V, WK>(a, blk * (kMgThreads / 32) + (threadIdx.x >> 5), k0, k1);
+    if constexpr (DOT) {
+        double part[1], tot[1];
+        block_sum<1, kMgThreads>(acc, part);
+        if (grid_sum_last<1, kMgThreads>(part, d.partials, &d.st->ticket[1], tot) && threadIdx.x == 0)
+            mg_rz_finish(d, tot[0]);
     }
 }
 
-// coarsest level: kMgCoarseSweeps damped Jacobi sweeps from zero by one CTA;
-// the result lands in lv[l].u (sweeps alternate between u and w)
-__device__ __forceinline__ void mg_coarse_sweeps(const MgArgs &a, int l) {
-    const MgLevel &L = a.lv[l];
-    const int64_t n = (int64_t)L.nx * L.ny * L.nz;
-    float *src = L.u, *dst = L.w;
-    // the final sweep must land in u: start in w when the sweep count is even
-    if (kMgCoarseSweeps % 2 == 0) {
-        src = L.w;
-        dst = L.u;
-    }
-    for (int64_t c = threadIdx.x; c < n; c += kMgCoarseThreads) {
-        const int i = (int)(c % L.nx);
-        const int64_t t = c / L.nx;
-        const int j = (int)(t % L.ny), k = (int)(t / L.ny);
-        float w[6], D;
-        mg_weights(a, l, i, j, k, w, D);
-        src[c] = kMgOmega * L.f[c] / D;
-    }
-    __syncthreads();
-    for (int sweep = 1; sweep < kMgCoarseSweeps; ++sweep) {
-        for (int64_t c = threadIdx.x; c < n; c += kMgCoarseThreads) {
-            const int i = (int)(c % L.nx);
-            const int64_t t = c / L.nx;
-            const int j = (int)(t % L.ny), k = (int)(t / L.ny);
-            float w[6], D;
-            mg_weights(a, l, i, j, k, w, D);
-            const float off = mg_offdiag(L, i, j, k, c, w, [&](int64_t q, int, int, int) { return src[q]; });
-            dst[c] = fmaf(kMgOmega / D, L.f[c] - fmaf(D, src[c], -off), src[c]);
-        }
-        __syncthreads();
-        float *tmp = src;
-        src = dst;
-        dst = tmp;
-    }
+// ------------------------------------------------------------ the tail --
+//
+// The levels of at most kMgTailCells cells in one launch of one CTA: on such
+// levels a launch costs more than its work.  Weights and omega / D of all of
+// them lie in one block of memory and are brought into shared memory by one
+// copy; the vectors stay there.  A pass over a level in one SM is bound by
+// its shared-memory reads, so the passes run over flat indices, two cells a
+// thread, without decoding (i, j, k): halo planes of zeros around u and the
+// zero weights of boundary faces make every neighbour read harmless.  Only
+// the transfers between levels decode, one coarse cell a thread.  The launch's
+// parameters are kept to a line or two of the constant cache, which is cold:
+// as an array of levels they took 11000 cycles to read, a miss after another.
+// 16^3 and below: 35 us with the levels in global memory -> 8 us (15700
+// cycles: copies 4000, 16^3 8300, 8^3 and transfers 2800, 24 sweeps 2970).
+
+struct MgTail {
+    const SolveState *st;
+    const float *wts;   // per level w+x, w+y, w+z, D, omega / D (m values each)
+    const float *f;     // the first level's right-hand side
+    float *w;           // and its result
+    int nl;             // levels before the coarsest
+    int nx, ny, nz;     // the first level's size
+    int nwts;           // floats of wts
+};
+
+// What sweeps a coarsest level that is the whole tail: one CTA, or above
+// kMgTailCells cells a cluster, its halo planes exchanged through distributed
+// shared memory (31^3 cells, the coarsest level of 248^3: about 700 us in one
+// CTA with the vectors in global memory -> about 30 us).
+struct MgSweep {
+    int ppc, na;  // planes per CTA, sweeping CTAs
+    unsigned ctas;
+    size_t smem;  // 0: in global memory
+};
+
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // (i, j, k) of flat cell c of a level (32-bit: the tail's levels are small)
-__device__ __forceinline__ void mg_cell(const MgLevel &L, int c, int &i, int &j, int &k) {
-    const int t = c / L.nx;
-    i = c - t * L.nx;
-    k = t / L.ny;
-    j = t - k * L.ny;
+__device__ __forceinline__ void mg_cell(int nx, int ny, int c, int &i, int &j, int &k) {
+    const int t = c / nx;
+    i = c - t * nx;
+    k = t / ny;
+    j = t - k * ny;
 }
 
-// The coarsest level's sweeps with src / dst in shared memory (n <= kMgSmemCells):
-// the same arithmetic as mg_coarse_sweeps; the result is written to lv[l].u
-__device__ __forceinline__ void mg_coarse_sweeps_smem(const MgArgs &a, int l, float *sa, float *sb) {
-    const MgLevel &L = a.lv[l];
-    const int n = L.nx * L.ny * L.nz;
-    for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) {
+// n floats into shared memory by the CTA (dst 16-byte aligned); wait with mg_copy_wait
+__device__ __forceinline__ void mg_copy(float *dst, const float *src, int n) {
+    const uint32_t d = smem_u32(dst);
+    const int n4 = (reinterpret_cast<uintptr_t>(src) & 15) == 0 ? n & ~3 : 0;
+    for (int i = threadIdx.x * 4; i < n4; i += kMgTailThreads * 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 4u * i), "l"(src + i) : "memory");
+    for (int i = n4 + threadIdx.x; i < n; i += kMgTailThreads)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4u * i), "l"(src + i) : "memory");
+}
+__device__ __forceinline__ void mg_copy_wait() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+}
+
+// A level of the tail in shared memory: offsets in floats.  u has a plane of
+// zeros on either side (so what a weight array's neighbour read finds before
+// its first element only has to be finite); g is the residual on the way down
+// and the result on the way up.
+struct MgSm {
+    int nx, ny, pl, m;
+    int u, wx, wy, wz, D, od, f, g;
+};
+__host__ __device__ inline int mg_round4(int n) { return (n + 3) & ~3; }
+// the coarsest level: wx, wy, wz, D, f, g and the sweeps' two buffers in u
+__host__ __device__ inline MgSm mg_sm_level(int nx, int ny, int nz, bool coarsest, int &wat, int &at) {
+    MgSm s;
+    s.nx = nx;
+    s.ny = ny;
+    s.pl = nx * ny;
+    s.m = s.pl * nz;
+    s.wx = wat;
+    s.wy = s.wx + s.m;
+    s.wz = s.wy + s.m;
+    s.D = s.wz + s.m;
+    s.od = s.D + s.m;
+    wat += 5 * s.m;
+    s.u = at + mg_round4(s.pl);
+    at = s.u + mg_round4(s.m) + (coarsest ? 2 * mg_round4(s.pl) + s.m + s.pl : s.pl);
+    at = mg_round4(at);
+    s.f = at;
+    s.g = at + mg_round4(s.m);
+    at = s.g + mg_round4(s.m);
+    return s;
+}
+
+// (f - A u) (UP: u + omega D^-1 (f - A u)) of a level into out
+template <bool UP>
+__device__ __forceinline__ void mg_sm_residual(const float *sm, const MgSm &s, float *out) {
+    auto ld2 = [&](int o) { return *reinterpret_cast<const float2 *>(sm + o); };
+    const int nx = s.nx, pl = s.pl;
+    for (int c = 2 * threadIdx.x; c < s.m; c += 2 * kMgTailThreads) {
+        const float2 u = ld2(s.u + c), ym = ld2(s.u + c - nx), yp = ld2(s.u + c + nx), zm = ld2(s.u + c - pl),
+                     zp = ld2(s.u + c + pl), x = ld2(s.wx + c), y0 = ld2(s.wy + c - nx), y1 = ld2(s.wy + c),
+                     z0 = ld2(s.wz + c - pl), z1 = ld2(s.wz + c), D = ld2(s.D + c), f = ld2(s.f + c);
+        const float ul = sm[s.u + c - 1], ur = sm[s.u + c + 2], xl = sm[s.wx + c - 1];
+        float a = fmaf(x.x, u.y, xl * ul), b = fmaf(x.y, ur, x.x * u.x);
+        a = fmaf(y0.x, ym.x, a);
+        b = fmaf(y0.y, ym.y, b);
+        a = fmaf(y1.x, yp.x, a);
+        b = fmaf(y1.y, yp.y, b);
+        a = fmaf(z0.x, zm.x, a);
+        b = fmaf(z0.y, zm.y, b);
+        a = fmaf(z1.x, zp.x, a);
+        b = fmaf(z1.y, zp.y, b);
+        a = f.x - fmaf(D.x, u.x, -a);
+        b = f.y - fmaf(D.y, u.y, -b);
+        if (UP) {
+            const float2 o = ld2(s.od + c);
+            a = fmaf(o.x, a, u.x);
+            b = fmaf(o.y, b, u.y);
+        }
+        out[c] = a;
+        out[c + 1] = b;
+    }
+}
+
+// fn(coarse cell, flat index of its first fine cell) for every coarse cell of a level
+template <typename F>
+__device__ __forceinline__ void mg_sm_coarse(const MgSm &s, F fn) {
+    const int cnx = s.nx / 2, cny = s.ny / 2, cm = s.m / 8;
+    for (int cc = threadIdx.x; cc < cm; cc += kMgTailThreads) {
+        int I, J, K;
+        mg_cell(cnx, cny, cc, I, J, K);
+        fn(cc, (2 * K * s.ny + 2 * J) * s.nx + 2 * I);
+    }
+}
+
+// The coarsest level of a tail of several levels (at most a cell a thread):
+// kMgCoarseSweeps damped Jacobi sweeps from zero, into g.  Only the warps with
+// cells take part; the buffers' halo planes are zero.
+__device__ __forceinline__ void mg_sm_sweeps(float *sm, const MgSm &s) {
+    const int c = threadIdx.x, nthr = (s.m + 31) / 32 * 32, nx = s.nx, pl = s.pl;
+    if (c >= nthr) return;  // the caller's barrier follows
+    const int stride = mg_round4(s.m) + 2 * mg_round4(pl) - (mg_round4(pl) - pl);
+    const bool on = c < s.m;
+    const int q = on ? c : 0;
+    const float w0 = sm[s.wx + q - 1], w1 = sm[s.wx + q], w2 = sm[s.wy + q - nx], w3 = sm[s.wy + q],
+                w4 = sm[s.wz + q - pl], w5 = sm[s.wz + q], D = sm[s.D + q], f = sm[s.f + q], o = kMgOmega / D;
+    float *b0 = sm + s.u + q, *b1 = b0 + stride;
+    auto sync = [&] {
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+    };
+    float v = o * f;
+    if (on) *b0 = v;
+    sync();
+    auto sweep = [&](const float *p) {
+        const float a = fmaf(w2, p[-nx], w0 * p[-1]), b = fmaf(w3, p[nx], w1 * p[1]), d = fmaf(w5, p[pl], w4 * p[-pl]);
+        v = fmaf(o, f - fmaf(D, v, -((a + b) + d)), v);
+    };
+    for (int t = 1; t + 1 < kMgCoarseSweeps; t += 2) {
+        sweep(b0);
+        if (on) *b1 = v;
+        sync();
+        sweep(b1);
+        if (on) *b0 = v;
+        sync();
+    }
+    if (kMgCoarseSweeps % 2 == 0) sweep(b0);
+    if (on) sm[s.g + c] = v;
+}
+
+// coarsest level: kMgCoarseSweeps damped Jacobi sweeps from zero; the result
+// lands in L.w.  CTA `rank` of t.na sweeps t.ppc planes, kept twice in
+// shared memory with a halo plane on either side; a CTA writes its first and
+// last plane into the neighbours' halos as it computes them.  Weights of up
+// to NC cells a thread stay in registers (NC = 0: they are read each sweep).
+template <int NC>
+__device__ __forceinline__ void mg_sweeps(const MgArgs &a, const MgSweep &t, int rank, float *sm) {
+    const MgLevel L = a.lv[a.L - 1];
+    const bool lvl0 = a.L == 1;
+    const int nx = L.nx, pl = L.nx * L.ny, ppc = t.ppc, na = t.na;
+    const int k0 = rank * ppc, planes = max(0, min(L.nz - k0, ppc)), n = planes * pl;
+    const int stride = (ppc + 2) * pl;
+    const uint32_t sbase = smem_u32(sm);
+    // one CTA: only the warps with cells take part
+    const int nthr = min((n + 31) / 32 * 32, kMgTailThreads);
+    auto sync = [&] {
+        __syncwarp();
+        if (na > 1) cluster_barrier();
+        else asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+    };
+    auto remote = [&](int r, int which, int idx) {
+        uint32_t ra;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(sbase + 4u * (uint32_t)(which * stride + idx)), "r"(r));
+        return ra;
+    };
+    auto put = [&](int which, int c, float v) {
+        sm[which * stride + pl + c] = v;
+        if (na == 1) return;
+        if (c < pl && rank > 0)  // the halo after the previous CTA's (full) planes
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(rank - 1, which, (ppc + 1) * pl + c)), "f"(v) : "memory");
+        if (c >= n - pl && rank + 1 < na)
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote(rank + 1, which, c - (n - pl))), "f"(v) : "memory");
+    };
+    for (int q = threadIdx.x; q < 2 * stride; q += kMgTailThreads) sm[q] = 0.f;
+    if (na > 1) cluster_barrier();
+    else __syncthreads();
+    if (na == 1 && (int)threadIdx.x >= nthr) return;  // the caller's barrier follows
+    constexpr int NR = NC > 0 ? NC : 1;
+    float w[NR][6], D[NR], o[NR], f[NR];
+    auto load = [&](int c, float (&ww)[6], float &DD, float &oo, float &ff) {
         int i, j, k;
-        mg_cell(L, c, i, j, k);
+        mg_cell(nx, L.ny, c, i, j, k);
+        if (lvl0) mg_weights(a, 0, i, j, k + k0, ww, DD);
+        else mg_weights_stored(L, i, j, k + k0, ww, DD);
+        ff = L.f[k0 * pl + c];
+        oo = kMgOmega / DD;
+    };
+    auto point = [&](const float *s, int c, const float (&ww)[6], float DD, float oo, float ff) {
+        const float *p = s + pl + c;
+        float off = ww[0] * p[-1];
+        off = fmaf(ww[1], p[1], off);
+        off = fmaf(ww[2], p[-nx], off);
+        off = fmaf(ww[3], p[nx], off);
+        off = fmaf(ww[4], p[-pl], off);
+        off = fmaf(ww[5], p[pl], off);
+        return fmaf(oo, ff - fmaf(DD, p[0], -off), p[0]);
+    };
+    float *res = L.w + k0 * pl;
+    auto cells = [&](auto fn) {
+        if constexpr (NC > 0) {
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+                const int c = threadIdx.x + m * kMgTailThreads;
+                if (c < n) fn(m, c);
+            }
+        } else {
+            for (int c = threadIdx.x; c < n; c += kMgTailThreads) fn(0, c);
+        }
+    };
+    cells([&](int m, int c) {
+        load(c, w[m], D[m], o[m], f[m]);
+        put(0, c, o[m] * f[m]);
+    });
+    sync();
+    for (int sweep = 1; sweep < kMgCoarseSweeps - 1; ++sweep) {
+        const float *src = sm + ((sweep - 1) & 1) * stride;
+        cells([&](int m, int c) {
+            if constexpr (NC == 0) load(c, w[0], D[0], o[0], f[0]);
+            put(sweep & 1, c, point(src, c, w[m], D[m], o[m], f[m]));
+        });
+        sync();
+    }
+    cells([&](int m, int c) {
+        if constexpr (NC == 0) load(c, w[0], D[0], o[0], f[0]);
+        res[c] = point(sm + (kMgCoarseSweeps & 1) * stride, c, w[m], D[m], o[m], f[m]);
+    });
+}
+static_assert(kMgCoarseSweeps >= 2, "first and last sweep");
+
+// The same sweeps by one CTA in global memory (od and w of the coarsest level
+// in turn): a grid of one level whose planes are too large for the shared
+// memory (nz < 4).
+__device__ __forceinline__ void mg_sweeps_flat(const MgArgs &a) {
+    const int l = a.L - 1;
+    const MgLevel &L = a.lv[l];
+    const int n = (int)L.m, sy = L.nx, sz = L.nx * L.ny;
+    float *src = kMgCoarseSweeps % 2 ? L.w : L.od, *dst = kMgCoarseSweeps % 2 ? L.od : L.w;
+    for (int sweep = 0; sweep < kMgCoarseSweeps; ++sweep) {
+        float *out = sweep == 0 ? src : dst;
+        for (int c = threadIdx.x; c < n; c += kMgTailThreads) {
+            int i, j, k;
+            mg_cell(L.nx, L.ny, c, i, j, k);
+            float w[6], D;
+            mg_weights(a, l, i, j, k, w, D);
+            const float o = kMgOmega / D;
+            if (sweep == 0) {
+                out[c] = o * L.f[c];
+                continue;
+            }
+            float off = 0.f;
+            if (i > 0) off = fmaf(w[0], src[c - 1], off);
+            if (i + 1 < L.nx) off = fmaf(w[1], src[c + 1], off);
+            if (j > 0) off = fmaf(w[2], src[c - sy], off);
+            if (j + 1 < L.ny) off = fmaf(w[3], src[c + sy], off);
+            if (k > 0) off = fmaf(w[4], src[c - sz], off);
+            if (k + 1 < L.nz) off = fmaf(w[5], src[c + sz], off);
+            out[c] = fmaf(o, L.f[c] - fmaf(D, src[c], -off), src[c]);
+        }
+        __syncthreads();
+        if (sweep > 0) {
+            float *tmp = src;
+            src = dst;
+            dst = tmp;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kMgTailThreads) mg_sweep_kernel(const MgArgs a, const MgSweep t) {
+    extern __shared__ __align__(16) float mg_sm[];
+    if (mg_stand_down(a.st)) return;  // the same for the whole cluster
+    if (t.smem == 0) {                // one CTA
+        mg_sweeps_flat(a);
+        return;
+    }
+    const int n = t.ppc * a.lv[a.L - 1].nx * a.lv[a.L - 1].ny, rank = (int)blockIdx.x;
+    if (n <= kMgTailThreads) mg_sweeps<1>(a, t, rank, mg_sm);
+    else if (n <= kMgSweepCells * kMgTailThreads) mg_sweeps<kMgSweepCells>(a, t, rank, mg_sm);
+    else mg_sweeps<0>(a, t, rank, mg_sm);
+    if (t.na > 1) cluster_barrier();  // no CTA leaves while its halos can still be written
+}
+
+__global__ void __launch_bounds__(kMgTailThreads) mg_tail_kernel(const MgTail t) {
+    extern __shared__ __align__(16) float mg_sm[];
+    if (mg_stand_down(t.st)) return;
+    const int tid = threadIdx.x;
+    if (tid < 4) mg_sm[tid] = 0.f;  // before the weights: finite
+    mg_copy(mg_sm + 4, t.wts, t.nwts);
+    MgSm lv[kMgTailLevels];
+    int wat = 4, at = 4 + mg_round4(t.nwts);
+#pragma unroll
+    for (int q = 0; q < kMgTailLevels; ++q)
+        if (q <= t.nl) {
+            lv[q] = mg_sm_level(t.nx >> q, t.ny >> q, t.nz >> q, q == t.nl, wat, at);
+            const MgSm &s = lv[q];
+            // zeros around u (the coarsest: its two buffers)
+            if (q < t.nl) {
+                for (int i = tid; i < s.pl; i += kMgTailThreads) mg_sm[s.u - s.pl + i] = mg_sm[s.u + s.m + i] = 0.f;
+            } else {
+                for (int i = s.u - s.pl + tid; i < s.f; i += kMgTailThreads) mg_sm[i] = 0.f;
+            }
+        }
+    mg_copy(mg_sm + lv[0].f, t.f, lv[0].m);
+    mg_copy_wait();
+    for (int c = tid; c < lv[0].m; c += kMgTailThreads) mg_sm[lv[0].u + c] = mg_sm[lv[0].f + c] * mg_sm[lv[0].od + c];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q + 1 < kMgTailLevels; ++q)
+        if (q < t.nl) {
+            const MgSm &s = lv[q], &C = lv[q + 1];
+            const bool next = q + 1 < t.nl;
+            mg_sm_residual<false>(mg_sm, s, mg_sm + s.g);
+            __syncthreads();
+            mg_sm_coarse(s, [&](int cc, int c) {
+                const float *g = mg_sm + s.g + c;
+                const float a0 = g[0] + g[1], a1 = g[s.nx] + g[s.nx + 1];
+                const float b0 = g[s.pl] + g[s.pl + 1], b1 = g[s.pl + s.nx] + g[s.pl + s.nx + 1];
+                const float r = (a0 + a1) + (b0 + b1);
+                mg_sm[C.f + cc] = r;
+                if (next) mg_sm[C.u + cc] = r * mg_sm[C.od + cc];
+            });
+            __syncthreads();
+        }
+#pragma unroll
+    for (int q = 1; q < kMgTailLevels; ++q)
+        if (q == t.nl) mg_sm_sweeps(mg_sm, lv[q]);
+    __syncthreads();
+#pragma unroll
+    for (int q = kMgTailLevels - 2; q >= 0; --q)
+        if (q < t.nl) {
+            const MgSm &s = lv[q];
+            const int e = lv[q + 1].g;
+            mg_sm_coarse(s, [&](int cc, int c) {
+                float *u = mg_sm + s.u + c;
+                const float v = mg_sm[e + cc];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float *p = u + (r & 1) * s.nx + (r >> 1) * s.pl;
+                    p[0] = fmaf(kMgSigma, v, p[0]);
+                    p[1] = fmaf(kMgSigma, v, p[1]);
+                }
+            });
+            __syncthreads();
+            if (q > 0) {
+                mg_sm_residual<true>(mg_sm, s, mg_sm + s.g);
+                __syncthreads();
+            } else {
+                mg_sm_residual<true>(mg_sm, s, t.w);
+            }
+        }
+}
+
+// Level 0 inside the tail: its weights in the coarse levels' stored form
+__global__ void __launch_bounds__(kMgThreads) mg_store0_kernel(const MgArgs a, float *W) {
+    const MgLevel &L = a.lv[0];
+    for (int c = blockIdx.x * kMgThreads + threadIdx.x; c < (int)L.m; c += gridDim.x * kMgThreads) {
+        int i, j, k;
+        mg_cell(L.nx, L.ny, c, i, j, k);
         float w[6], D;
-        mg_weights(a, l, i, j, k, w, D);
-        sa[c] = kMgOmega * L.f[c] / D;
-    }
-    __syncthreads();
-    float *src = sa, *dst = sb;
-    for (int sweep = 1; sweep < kMgCoarseSweeps; ++sweep) {
-        for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) {
-            int i, j, k;
-            mg_cell(L, c, i, j, k);
-            float w[6], D;
-            mg_weights(a, l, i, j, k, w, D);
-            const float off = mg_offdiag(L, i, j, k, c, w, [&](int64_t q, int, int, int) { return src[q]; });
-            dst[c] = fmaf(kMgOmega / D, L.f[c] - fmaf(D, src[c], -off), src[c]);
-        }
-        __syncthreads();
-        float *tmp = src;
-        src = dst;
-        dst = tmp;
-    }
-    for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) L.u[c] = src[c];
-    __syncthreads();
-}
-
-// The small levels l0 .. L-1 of the V-cycle in one CTA (every level but
-// possibly the coarsest holds at most kMgTailCells cells; the coarsest at most
-// kMgMaxCoarsest, in 32-bit range): pre-smoothing and
-// restriction down to the coarsest level, its sweeps, post-smoothing back up
-// to l0 (the same steps as the level kernels, with a CTA barrier between
-// them instead of a kernel launch: on levels of a few thousand cells the
-// launches cost more than the work).  Level l0's result lands in lv[l0].w,
-// or in lv[l0].u when l0 is the coarsest level; a one-level hierarchy copies
-// it into lv[0].w, the V-cycle's output.
-__global__ void __launch_bounds__(kMgCoarseThreads) mg_tail_kernel(const MgArgs a, int l0) {
-    if (mg_stand_down(a)) return;
-    const int lc = a.L - 1;
-    for (int l = l0; l < lc; ++l) {
-        const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
-        const int n = L.nx * L.ny * L.nz, nc = C.nx * C.ny * C.nz;
-        for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) {
-            int i, j, k;
-            mg_cell(L, c, i, j, k);
-            float w[6], D;
-            mg_weights(a, l, i, j, k, w, D);
-            L.u[c] = kMgOmega * L.f[c] / D;
-        }
-        __syncthreads();
-        for (int cc = threadIdx.x; cc < nc; cc += kMgCoarseThreads) {
-            int I, J, K;
-            mg_cell(C, cc, I, J, K);
-            float sum = 0.f;
-            for (int dz = 0; dz < 2; ++dz)
-                for (int dy = 0; dy < 2; ++dy)
-                    for (int dx = 0; dx < 2; ++dx) {
-                        const int i = 2 * I + dx, j = 2 * J + dy, k = 2 * K + dz;
-                        const int c = (k * L.ny + j) * L.nx + i;
-                        float w[6], D;
-                        mg_weights(a, l, i, j, k, w, D);
-                        const float off = mg_offdiag(L, i, j, k, c, w, [&](int64_t q, int, int, int) { return L.u[q]; });
-                        sum += L.f[c] - fmaf(D, L.u[c], -off);
-                    }
-            C.f[cc] = sum;
-        }
-        __syncthreads();
-    }
-    __shared__ float s_sweep[2][kMgSmemCells];
-    if ((int64_t)a.lv[lc].nx * a.lv[lc].ny * a.lv[lc].nz <= kMgSmemCells)
-        mg_coarse_sweeps_smem(a, lc, s_sweep[0], s_sweep[1]);
-    else
-        mg_coarse_sweeps(a, lc);
-    for (int l = lc - 1; l >= l0; --l) {
-        const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
-        const float *e = (l + 1 == lc) ? C.u : C.w;
-        const int n = L.nx * L.ny * L.nz;
-        // u' = u + sigma P e at a fine cell
-        auto up = [&](int64_t q, int i, int j, int k) {
-            return fmaf(kMgSigma, e[((int64_t)(k >> 1) * C.ny + (j >> 1)) * C.nx + (i >> 1)], L.u[q]);
-        };
-        for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) {
-            int i, j, k;
-            mg_cell(L, c, i, j, k);
-            float w[6], D;
-            mg_weights(a, l, i, j, k, w, D);
-            const float uc = up(c, i, j, k);
-            const float off = mg_offdiag(L, i, j, k, c, w, up);
-            L.w[c] = fmaf(kMgOmega / D, L.f[c] - fmaf(D, uc, -off), uc);
-        }
-        __syncthreads();
-    }
-    if (lc == 0) {
-        const MgLevel &L = a.lv[0];
-        const int n = L.nx * L.ny * L.nz;
-        for (int c = threadIdx.x; c < n; c += kMgCoarseThreads) L.w[c] = L.u[c];
+        mg_weights(a, 0, i, j, k, w, D);
+        W[c] = w[1];
+        W[c + L.m] = w[3];
+        W[c + 2 * L.m] = w[5];
+        W[c + 3 * L.m] = D;
     }
 }
 
-// Galerkin coarsening of level l into level l + 1 (one thread per coarse cell)
-__global__ void __launch_bounds__(kMgThreads) mg_galerkin_kernel(const MgArgs a, int l, float4 *Wc, int zper) {
-    const MgLevel &C = a.lv[l + 1];
+// Galerkin coarsening of level l into level l + 1 (one thread per coarse
+// cell), and omega / D of level l's points into its od (NULL: not used)
+__global__ void __launch_bounds__(kMgThreads) mg_galerkin_kernel(const MgArgs a, int l, float *Wc, float *od, int zper) {
+    const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
     const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
     if (I >= C.nx || J >= C.ny) return;
     const int K0 = blockIdx.z * zper, K1 = min(C.nz, K0 + zper);
     for (int K = K0; K < K1; ++K) {
         float sx = 0.f, sy = 0.f, sz = 0.f, sD = 0.f, inner = 0.f;
         for (int dz = 0; dz < 2; ++dz)
-            for (int dy = 0; dy < 2; ++dy)
+            for (int dy = 0; dy < 2; ++dy) {
+                float o[2];
+#pragma unroll
                 for (int dx = 0; dx < 2; ++dx) {
                     float w[6], D;
                     mg_weights(a, l, 2 * I + dx, 2 * J + dy, 2 * K + dz, w, D);
+                    o[dx] = kMgOmega / D;
                     sD += D;
                     if (dx == 1) sx += w[1]; else inner += w[1];
                     if (dy == 1) sy += w[3]; else inner += w[3];
                     if (dz == 1) sz += w[5]; else inner += w[5];
                 }
-        Wc[((int64_t)K * C.ny + J) * C.nx + I] = make_float4(sx, sy, sz, sD - 2.0f * inner);
+                if (od)
+                    *reinterpret_cast<float2 *>(od + ((int64_t)(2 * K + dz) * L.ny + 2 * J + dy) * L.nx + 2 * I) =
+                        make_float2(o[0], o[1]);
+            }
+        const int64_t c = ((int64_t)K * C.ny + J) * C.nx + I;
+        Wc[c] = sx;
+        Wc[c + C.m] = sy;
+        Wc[c + 2 * C.m] = sz;
+        Wc[c + 3 * C.m] = sD - 2.0f * inner;
     }
 }
 
-// r.z; last CTA: beta (the first time, only r.z), breakdown, the loop condition
+// r.z in a pass of its own, where the tail holds the whole hierarchy
 __global__ void __launch_bounds__(kMgThreads)
-    mg_rz_kernel(int64_t n, const float *__restrict__ r, const float *__restrict__ z, SolveState *st, double *partials,
-                 int init, cudaGraphConditionalHandle cond, int use_cond) {
-    if (st->done) return;
+    mg_rz_kernel(int64_t n, const float *__restrict__ r, const float *__restrict__ z, const MgDot d) {
+    if (d.st->done) return;
     float acc[1] = {0.f};
     for (int64_t i = (int64_t)blockIdx.x * kMgThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kMgThreads)
         acc[0] = fmaf(r[i], z[i], acc[0]);
     double part[1], tot[1];
     block_sum<1, kMgThreads>(acc, part);
-    if (!grid_sum_last<1, kMgThreads>(part, partials, &st->ticket[1], tot) || threadIdx.x != 0) return;
-    const double rz = tot[0];
-    if (!isfinite(rz) || !(rz > 0.0)) {
-        st->done = 1;
-        st->status = GBPCG_BREAKDOWN;
-    } else {
-        if (!init) st->beta = rz / st->rzm;
-        st->rz = rz;
-        st->rzm = rz;
-    }
-    if (use_cond) cudaGraphSetConditional(cond, st->done ? 0u : 1u);
+    if (!grid_sum_last<1, kMgThreads>(part, d.partials, &d.st->ticket[1], tot) || threadIdx.x != 0) return;
+    mg_rz_finish(d, tot[0]);
 }
 
 // ---------------------------------------------------------- host side --
@@ -564,11 +1035,13 @@ MgGeom mg_geom(const gbpcg_grid &g) {
     return m;
 }
 
-// workspace pieces beyond the Jacobi solver's: r, level 0's u, and per coarse
-// level f, u, w and the weights
+// workspace pieces beyond the Jacobi solver's: r, per coarse level f and w, the
+// block of all levels' weights and omega / D (level by level, w+x, w+y, w+z, D,
+// omega / D; level 0 only where it is inside the tail), and omega / D of a
+// level 0 above the tail
 struct MgLayout {
     WsLayout base;
-    size_t r, u0, lev[kMgMaxLevels][4];
+    size_t r, od0, f[kMgMaxLevels], w[kMgMaxLevels], wts[kMgMaxLevels];
     size_t total;
 };
 
@@ -578,18 +1051,19 @@ MgLayout mg_layout(const gbpcg_grid &g, int io) {
     M.base = ws_layout_n(n, GBPCG_F32, io, false, block_count(g));
     size_t o = M.base.total;
     M.r = o; o += round256(n * 4);
-    M.u0 = o; o += round256(n * 4);
+    M.od0 = o;
+    if ((int64_t)n > kMgTailCells) o += round256(n * 4);
     const MgGeom G = mg_geom(g);
+    auto cells = [&](int l) { return (size_t)G.nx[l] * G.ny[l] * G.nz[l]; };
     for (int l = 1; l < G.L; ++l) {
-        const size_t m = (size_t)G.nx[l] * G.ny[l] * G.nz[l];
-        for (int v = 0; v < 3; ++v) {
-            M.lev[l][v] = o;
-            o += round256(m * 4);
-        }
-        M.lev[l][3] = o;
-        o += round256(m * 16);
+        M.f[l] = o; o += round256(cells(l) * 4);
+        M.w[l] = o; o += round256(cells(l) * 4);
     }
-    M.total = o;
+    for (int l = (int64_t)n > kMgTailCells ? 1 : 0; l < G.L; ++l) {
+        M.wts[l] = o;
+        o += cells(l) * 20;  // every level but the coarsest holds a multiple of 8 cells: 16-byte arrays
+    }
+    M.total = round256(o);
     return M;
 }
 
@@ -601,16 +1075,17 @@ MgArgs mg_args(const gbpcg_grid &g, char *ws, const MgLayout &M, float *f0, floa
     for (int l = 0; l < G.L; ++l) {
         MgLevel &L = a.lv[l];
         L.nx = G.nx[l]; L.ny = G.ny[l]; L.nz = G.nz[l];
-        if (l == 0) {
-            L.f = f0;
-            L.u = reinterpret_cast<float *>(ws + M.u0);
-            L.w = z;
-            L.W = nullptr;
+        L.m = (int64_t)L.nx * L.ny * L.nz;
+        L.f = l == 0 ? f0 : reinterpret_cast<float *>(ws + M.f[l]);
+        L.w = l == 0 ? z : reinterpret_cast<float *>(ws + M.w[l]);
+        if (l > 0 || L.m <= kMgTailCells) {
+            L.wx = reinterpret_cast<const float *>(ws + M.wts[l]);
+            L.wy = L.wx + L.m;
+            L.wz = L.wy + L.m;
+            L.D = L.wz + L.m;
+            L.od = const_cast<float *>(L.D + L.m);
         } else {
-            L.f = reinterpret_cast<float *>(ws + M.lev[l][0]);
-            L.u = reinterpret_cast<float *>(ws + M.lev[l][1]);
-            L.w = reinterpret_cast<float *>(ws + M.lev[l][2]);
-            L.W = reinterpret_cast<const float4 *>(ws + M.lev[l][3]);
+            L.od = reinterpret_cast<float *>(ws + M.od0);
         }
     }
     a.block = g.k_block ? 1 : 0;
@@ -636,71 +1111,125 @@ unsigned mg_grid(int64_t n) {
         1, std::min<int64_t>((n + kMgThreads - 1) / kMgThreads, (int64_t)device_sm_count() * 8));
 }
 
+// the first level of the tail
+int mg_l0(const MgArgs &a) {
+    int l0 = a.L - 1;
+    while (l0 > 0 && a.lv[l0 - 1].m <= kMgTailCells) --l0;
+    return l0;
+}
+
+// whether level 0's omega / D is kept per point (constant coefficients above the tail: one number)
+bool mg_od0(const MgArgs &a) { return a.block || mg_l0(a) == 0; }
+
 // the coarse operators (once per solve)
 cudaError_t mg_setup(const MgArgs &a, cudaStream_t s) {
+    if (a.L > 1 && mg_l0(a) == 0)
+        mg_store0_kernel<<<mg_grid(a.lv[0].m), kMgThreads, 0, s>>>(a, const_cast<float *>(a.lv[0].wx));
     for (int l = 0; l + 1 < a.L; ++l) {
         const MgLevel &C = a.lv[l + 1];
         const MgLaunch g = mg_launch(C.nx, C.ny, C.nz);
-        mg_galerkin_kernel<<<g.grid, g.block, 0, s>>>(a, l, const_cast<float4 *>(C.W), g.zper);
+        mg_galerkin_kernel<<<g.grid, g.block, 0, s>>>(a, l, const_cast<float *>(C.wx),
+                                                      l > 0 || mg_od0(a) ? a.lv[l].od : nullptr, g.zper);
     }
     return cudaGetLastError();
 }
 
-// z = M f0 (a.lv[0].f -> a.lv[0].w)
-cudaError_t mg_vcycle(const MgArgs &a, cudaStream_t s) {
-    // levels whose rows split into 16-byte vectors take four points per thread (and their
-    // restriction two coarse cells per thread)
-    auto vec = [&](int l) { return a.lv[l].nx % 4 == 0; };
-    // levels from l0 down (at most kMgTailCells cells each) run in one CTA
-    int l0 = a.L - 1;
-    while (l0 > 0 && (int64_t)a.lv[l0 - 1].nx * a.lv[l0 - 1].ny * a.lv[l0 - 1].nz <= kMgTailCells) --l0;
-    // the kernels of one level, compiled for its kind of weights
-    auto down = [&](auto wk_tag, int l) {
-        constexpr int WK = decltype(wk_tag)::value;
-        const MgLevel &L = a.lv[l], &C = a.lv[l + 1];
-        if (vec(l) && WK == W_CONST0) {
-            // constant coefficients: u = omega f / D is formed inside restriction and post-smoothing
-            const MgLaunch gc = mg_launch(C.nx / 2, C.ny, C.nz);
-            mg_restrict_kernel<2, WK, true><<<gc.grid, gc.block, 0, s>>>(a, l, gc.zper);
-        } else if (vec(l)) {
-            const MgLaunch gf = mg_launch(L.nx / 4, L.ny, L.nz), gc = mg_launch(C.nx / 2, C.ny, C.nz);
-            mg_pre_kernel<4, WK><<<gf.grid, gf.block, 0, s>>>(a, l, gf.zper);
-            mg_restrict_kernel<2, WK><<<gc.grid, gc.block, 0, s>>>(a, l, gc.zper);
+// The level kernels' grid: blocks of 128 segments of row pairs times runs of
+// planes (`planes` of them, fine or coarse), kMgBlocks blocks per SM in all.
+constexpr int kMgBlocks = 3;
+struct MgGrid {
+    dim3 grid;
+    unsigned nblk;
+    int kper;
+};
+MgGrid mg_level_grid(const MgLevel &L, int V, int planes) {
+    const int64_t np = (int64_t)(L.nx / V) * (L.ny / 2);
+    const int64_t nblk = (np + kMgThreads / 2 - 1) / (kMgThreads / 2);
+    const int64_t want = std::max<int64_t>(1, (int64_t)device_sm_count() * kMgBlocks / nblk);
+    const int kper = (int)((planes + std::min<int64_t>(want, planes) - 1) / std::min<int64_t>(want, planes));
+    // at most kMaxPassBlocks blocks leave a partial sum
+    const unsigned gz = (unsigned)((planes + kper - 1) / kper);
+    const unsigned gx = (unsigned)std::min<int64_t>(nblk, std::max<unsigned>(1u, kMaxPassBlocks / gz));
+    return MgGrid{dim3(gx, gz), (unsigned)nblk, kper};
+}
+
+// z = M f0 (a.lv[0].f -> a.lv[0].w); dot: also r.z and what follows from it
+cudaError_t mg_vcycle(const MgArgs &a, cudaStream_t s, const MgDot *dot) {
+    const int l0 = mg_l0(a), lc = a.L - 1;
+    auto step = [&](int l, float *c) { return MgStep{a.st, a.lv[l], c, a.ob, a.tab, a.rkbx, a.rkby, a.rkbz}; };
+    // f(V, WK) for the level's row length and kind of weights
+    auto dispatch = [&](int l, auto f) {
+        using V4 = std::integral_constant<int, 4>;
+        using V2 = std::integral_constant<int, 2>;
+        if (l > 0) {
+            using Stored = std::integral_constant<int, W_STORED>;
+            if (a.lv[l].nx % 4 == 0) f(V4{}, Stored{});
+            else f(V2{}, Stored{});
+        } else if (!a.block) {
+            f(V4{}, std::integral_constant<int, W_CONST0>{});
+        } else if (a.ob.kbx % 4 == 0) {
+            f(V4{}, std::integral_constant<int, W_TABV>{});
         } else {
-            const MgLaunch gf = mg_launch(L.nx, L.ny, L.nz), gc = mg_launch(C.nx, C.ny, C.nz);
-            mg_pre_kernel<1, WK><<<gf.grid, gf.block, 0, s>>>(a, l, gf.zper);
-            mg_restrict_kernel<1, WK><<<gc.grid, gc.block, 0, s>>>(a, l, gc.zper);
+            f(V4{}, std::integral_constant<int, W_TAB0>{});
         }
     };
-    auto up = [&](auto wk_tag, int l) {
-        constexpr int WK = decltype(wk_tag)::value;
-        const MgLevel &L = a.lv[l];
-        const float *e = (l + 1 == a.L - 1) ? a.lv[l + 1].u : a.lv[l + 1].w;
-        if (vec(l) && WK == W_CONST0) {
-            const MgLaunch gf = mg_launch(L.nx / 4, L.ny, L.nz);
-            mg_post_kernel<4, WK, true><<<gf.grid, gf.block, 0, s>>>(a, l, e, gf.zper);
-        } else if (vec(l)) {
-            const MgLaunch gf = mg_launch(L.nx / 4, L.ny, L.nz);
-            mg_post_kernel<4, WK><<<gf.grid, gf.block, 0, s>>>(a, l, e, gf.zper);
-        } else {
-            const MgLaunch gf = mg_launch(L.nx, L.ny, L.nz);
-            mg_post_kernel<1, WK><<<gf.grid, gf.block, 0, s>>>(a, l, e, gf.zper);
+    for (int l = 0; l < l0; ++l)
+        dispatch(l, [&](auto v, auto wk) {
+            const MgGrid g = mg_level_grid(a.lv[l], v(), a.lv[l + 1].nz);
+            mg_restrict_kernel<v(), wk()><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].f), g.nblk, g.kper);
+        });
+    if (l0 < lc) {
+        const MgLevel &L = a.lv[l0];
+        MgTail t{a.st, L.wx, L.f, L.w, lc - l0, L.nx, L.ny, L.nz, 0};
+        int wat = 4, at = 0;
+        for (int q = 0; q <= t.nl; ++q) t.nwts += 5 * (int)a.lv[l0 + q].m;
+        at = 4 + mg_round4(t.nwts);
+        for (int q = 0; q <= t.nl; ++q) (void)mg_sm_level(L.nx >> q, L.ny >> q, L.nz >> q, q == t.nl, wat, at);
+        const size_t smem = (size_t)at * sizeof(float);
+        if (cudaError_t e = cudaFuncSetAttribute(mg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMgTailSmem))
+            return e;
+        mg_tail_kernel<<<1, kMgTailThreads, smem, s>>>(t);
+    } else {
+        const MgLevel &C = a.lv[lc];
+        const bool large = C.m > kMgTailCells;
+        MgSweep t;
+        t.ppc = large ? (C.nz + kMgTailCtas - 1) / kMgTailCtas : C.nz;
+        t.na = (C.nz + t.ppc - 1) / t.ppc;
+        t.ctas = large ? kMgTailCtas : 1;
+        t.smem = (size_t)2 * (t.ppc + 2) * C.nx * C.ny * sizeof(float);
+        if (t.smem > kMgTailSmem) {  // only a single level with nz < 4
+            t.smem = 0;
+            t.ctas = 1;
         }
-    };
-    using Const0 = std::integral_constant<int, W_CONST0>;
-    using Tab0 = std::integral_constant<int, W_TAB0>;
-    using Stored = std::integral_constant<int, W_STORED>;
-    for (int l = 0; l < l0; ++l) {
-        if (l > 0) down(Stored{}, l);
-        else if (a.block) down(Tab0{}, 0);
-        else down(Const0{}, 0);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(t.ctas);
+        cfg.blockDim = dim3(kMgTailThreads);
+        cfg.dynamicSmemBytes = t.smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = t.ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t e = cudaFuncSetAttribute(mg_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMgTailSmem);
+        if (!e) e = cudaLaunchKernelEx(&cfg, mg_sweep_kernel, a, t);
+        if (e) return e;
     }
-    mg_tail_kernel<<<1, kMgCoarseThreads, 0, s>>>(a, l0);
-    for (int l = l0 - 1; l >= 0; --l) {
-        if (l > 0) up(Stored{}, l);
-        else if (a.block) up(Tab0{}, 0);
-        else up(Const0{}, 0);
-    }
+    MgDot none;
+    memset(&none, 0, sizeof(none));
+    for (int l = l0 - 1; l >= 0; --l)
+        dispatch(l, [&](auto v, auto wk) {
+            const MgGrid g = mg_level_grid(a.lv[l], v(), a.lv[l].nz);
+            if constexpr (wk() != W_STORED) {
+                if (dot) {
+                    mg_post_kernel<v(), wk(), true><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].w), g.nblk, g.kper, *dot);
+                    return;
+                }
+            }
+            mg_post_kernel<v(), wk(), false><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].w), g.nblk, g.kper, none);
+        });
+    if (dot && l0 == 0) mg_rz_kernel<<<mg_grid(a.lv[0].m), kMgThreads, 0, s>>>(a.lv[0].m, a.lv[0].f, a.lv[0].w, *dot);
     return cudaGetLastError();
 }
 
@@ -725,13 +1254,14 @@ struct MgSolve {
     PassArgs ar;
     MgArgs mg;
     float *r, *z;
-    int64_t n;
 
     cudaError_t launch_r(cudaStream_t s) {
         return GB_CFG_DISPATCH(sp.cfg_b, float, K_PASSR, true, Op, K::launch(mr, ar, sp.op, sp.gb.grid(), s));
     }
-    void launch_rz(cudaStream_t s, int init) {
-        mg_rz_kernel<<<mg_grid(n), kMgThreads, 0, s>>>(n, r, z, sp.st, sp.partials, init, sp.cond_loop, sp.use_cond);
+    // the V-cycle and r.z
+    cudaError_t launch_m(cudaStream_t s, int init) {
+        const MgDot d{sp.st, sp.partials, init, sp.cond_loop, sp.use_cond};
+        return mg_vcycle(mg, s, &d);
     }
 
     int capture(cudaGraph_t *out) {
@@ -778,9 +1308,8 @@ struct MgSolve {
             if (e) break;
             e = mg_setup(mg, cs);
             if (e) break;
-            e = mg_vcycle(mg, cs);
+            e = launch_m(cs, 1);
             if (e) break;
-            launch_rz(cs, 1);
             cudaGraph_t body = nullptr;
             e = add_cond(cs, cond, cudaGraphCondTypeWhile, &body);
             if (e) break;
@@ -808,9 +1337,8 @@ struct MgSolve {
             e = cudaStreamEndCapture(rs, &tmp);
             cap_r = false;
             if (e) break;
-            e = mg_vcycle(mg, bs);
+            e = launch_m(bs, 0);
             if (e) break;
-            launch_rz(bs, 0);
             e = cudaStreamEndCapture(bs, &tmp);
             cap_b = false;
             if (e) break;
@@ -850,7 +1378,6 @@ int mg_solve_op(const gbpcg_grid &g, const Op &op, const double *b, double *x, c
         cb = narrow >= 0 ? narrow : CFG_128x8;
     }
     if (int rc = P.sp.init(g, op, ca, cb, b, x, ws, M.base, o.tol, o.maxit, 1.0, nullptr)) return rc;
-    P.n = (int64_t)g.nx * g.ny * g.nz;
     P.r = reinterpret_cast<float *>(ws + M.r);
     P.z = P.sp.z;
     // the FP64 residuals store r itself, in the r vector
@@ -932,7 +1459,7 @@ int gbpcg_mg_vcycle(const gbpcg_grid *grid, const float *r, float *z, void *work
         build_face_table<<<blocks, 256, 0, s>>>(grid->k_block, nbx, nby, nbz, const_cast<float4 *>(a.tab));
     }
     GB_CUDA(mg_setup(a, s));
-    GB_CUDA(mg_vcycle(a, s));
+    GB_CUDA(mg_vcycle(a, s, nullptr));
     if (levels) *levels = a.L;
     return GBPCG_OK;
 }
