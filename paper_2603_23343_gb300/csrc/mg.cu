@@ -47,7 +47,14 @@ constexpr float kMgOmega = 0.9f;
 constexpr float kMgSigma = 1.5f;
 constexpr int kMgCoarseSweeps = 24;
 constexpr int64_t kMgMaxCoarsest = 32768;
+// Grids up to this size (and ny even, for the row pairs) take the solver's passes A and R on the
+// march of the level kernels instead of through the TMA ring.  us per MG-PCG iteration, ring ->
+// march, Poisson / block coefficients: 32^3 67 -> 53 / 70 -> 50; 64^3 66 -> 59 / 70 -> 61; 128^3
+// 92 -> 91 / 102 -> 98; 160^3 132 -> 132 / 165 -> 153; 192^3 179 -> 187 / 219 -> 224; 256^3 308 ->
+// 334 / 410 -> 433.
+constexpr int64_t kMgDirectPoints = 5000000;
 constexpr int kMgThreads = 256;
+constexpr int64_t kMgRunPoints = 1 << 27;  // a run of planes: its offsets fit 32 bits
 constexpr int kMgTailThreads = 1024;
 constexpr int64_t kMgTailCells = 4096;  // levels this small run inside the one-CTA tail kernel
 constexpr int kMgTailCtas = 8;          // the cluster that sweeps a larger coarsest level
@@ -168,10 +175,11 @@ inline MgLaunch mg_launch(int nx, int ny, int nz) {
 //     planes, the stored weights of coarser levels are arrays per face
 //     direction read as vectors.
 // Loads of the plane after next are issued before the current plane is
-// computed.  Block coefficients at 256^3 (ncu): pre-smoothing and restriction
-// 30 + 68 us in two kernels -> 65 us, post-smoothing 115 us, and a pass of 20
-// us for r.z after it -> 81 us with r.z inside; the stored 128^3 level 64 ->
-// 39 us for both ways.
+// computed, at two or three CTAs per SM: the registers hold what is in flight.
+// The work is split evenly over the CTAs the device holds (mg_runs).  Block
+// coefficients at 256^3 (ncu): pre-smoothing and restriction 30 + 68 us in two
+// kernels -> 44 us, post-smoothing 115 -> 51 us (and no pass of 20 us for r.z
+// after it); the stored 128^3 level 64 -> 27 us both ways.
 
 // V consecutive floats (V * 4 byte aligned) -> registers
 template <int V>
@@ -201,13 +209,16 @@ struct MgStep {
 // points of a thread lie in one block.
 enum MgWeights { W_CONST0 = 1, W_TABV = 2, W_TAB0 = 3, W_STORED = 4 };
 
+// CTAs per SM the register count is held to: the constant weights leave room for three.
+constexpr int mg_min_blocks(int wk) { return wk == W_CONST0 ? 3 : 2; }
+
 // A thread's segment: V points from i0 of row j = 2J + hi.
 template <int V>
 struct MgSeg {
     int i0, j;
     bool hi, live, el, er, eo;  // eo: the row outside the pair exists; el / er: x neighbours to be loaded
     bool xl0, xr0;              // the row starts / ends here
-    int64_t c;                  // flat index at plane 0
+    unsigned c;                 // flat index at plane 0
     int dro;                    // offset of the row outside the pair
     __device__ __forceinline__ MgSeg(const MgLevel &L, unsigned wseg) {  // the warp's 16 segments per row: 16 wseg ..
         const int lane = threadIdx.x & 31, q = L.nx / V, np = q * (L.ny / 2);
@@ -224,7 +235,7 @@ struct MgSeg {
         er = (lane & 15) == 15 && !xr0;
         eo = hi ? j + 1 < L.ny : j > 0;
         dro = hi ? L.nx : -L.nx;
-        c = (int64_t)j * L.nx + i0;
+        c = (unsigned)j * L.nx + i0;
     }
 };
 
@@ -281,7 +292,7 @@ struct MgCol {
         }
     }
     // plane k (called for consecutive k from start's)
-    __device__ __forceinline__ void plane(const MgStep &a, const MgLevel &L, const MgSeg<V> &s, int64_t c, int k) {
+    __device__ __forceinline__ void plane(const MgStep &a, const MgLevel &L, const MgSeg<V> &s, int64_t cb, unsigned c, int k) {
         if constexpr (WK == W_TABV || WK == W_TAB0) {
             if (++iz == a.ob.kbz) {
                 iz = 0;
@@ -294,12 +305,12 @@ struct MgCol {
                 szm[m] = sz[m];
                 yo[m] = 0.f;
             }
-            ldv<V>(L.wx + c, sx);
-            ldv<V>(L.wy + c, y);
-            ldv<V>(L.wz + c, sz);
-            ldv<V>(L.D + c, sD);
-            if (!s.hi && s.eo) ldv<V>(L.wy + c - L.nx, yo);
-            const float xl = s.el ? __ldg(L.wx + c - 1) : 0.f;
+            ldv<V>(L.wx + cb + c, sx);
+            ldv<V>(L.wy + cb + c, y);
+            ldv<V>(L.wz + cb + c, sz);
+            ldv<V>(L.D + cb + c, sD);
+            if (!s.hi && s.eo) ldv<V>(L.wy + cb + (c - L.nx), yo);
+            const float xl = s.el ? __ldg(L.wx + cb + (c - 1)) : 0.f;
             const float xs = __shfl_up_sync(0xffffffffu, sx[V - 1], 1);
             sxl = s.xl0 ? 0.f : s.el ? xl : xs;
 #pragma unroll
@@ -345,31 +356,43 @@ struct MgCol {
     }
 };
 
-// The march both level kernels make: for the planes [k0, k1) of a segment,
-// the iterate v (POST: u + sigma P e, else u = (omega / D) f) at the segment
-// and its neighbours (0 outside the grid), and body(k, c, A v, v, f,
-// omega / D) per plane.  What a plane reads is loaded one plane ahead (its
-// own row two ahead: the z neighbour).
-template <int V, int WK, bool POST, typename Body>
-__device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int k0, int k1, Body body) {
+// The march all these kernels make: for the planes [k0, k1) of a segment, the
+// iterate v at the segment and its neighbours (0 outside the grid), and
+// body(k, c, A v, v, f, o) per plane.  What a plane reads is loaded one plane
+// ahead (its own row two ahead: the z neighbour).
+//   I_U     v = (omega / D) f, o = omega / D     (restriction)
+//   I_POST  v = (omega / D) f + sigma P e        (post-smoothing)
+//   I_P     v = f + beta o, o = p_{k-1}          (pass A)
+//   I_V     v = f                                (pass R)
+// The solver's passes form A v from the differences w (v - v_nb), whose
+// rounding is relative to A v's terms, the V-cycle as D v - sum w v_nb.
+enum MgIter { I_U, I_POST, I_P, I_V };
+template <int V, int WK, int IT, typename Body>
+__device__ __forceinline__ void mg_march(const MgStep &a, const float *f, const float *od, float beta, bool first,
+                                         const MgSeg<V> &s, int k0, int k1, Body body) {
+    constexpr bool POST = IT == I_POST, HAS_O = IT == I_P || (IT != I_V && WK != W_CONST0);
     const MgLevel &L = a.L;
     const float *e = a.c;
-    const float *f = L.f, *od = L.od;
-    const int64_t sz = (int64_t)L.nx * L.ny;
+    // offsets from plane kb on: 32 bits (a run of planes is kept below 2^29 points), shared by all arrays
+    const int kb = max(k0 - 1, 0) & ~1;
+    const unsigned sz = (unsigned)L.nx * L.ny;
     const int cnx = L.nx / 2;
-    const int64_t csz = (int64_t)cnx * (L.ny / 2);
+    const unsigned csz = (unsigned)cnx * (L.ny / 2);
+    f += (int64_t)kb * sz;
+    if (HAS_O) od += (int64_t)kb * sz;
+    if (POST) e += (int64_t)(kb / 2) * csz;
     const float wd = kMgOmega / (((a.ob.cx + a.ob.cx) + (a.ob.cy + a.ob.cy)) + (a.ob.cz + a.ob.cz));  // W_CONST0
     struct Raw {
         float f[V], o[V], e[V / 2];
     };
     // the V values at flat index c, whose parents start at flat index pc
-    auto fetch = [&](Raw &r, int64_t c, int64_t pc) {
+    auto fetch = [&](Raw &r, unsigned c, unsigned pc) {
         ldv<V>(f + c, r.f);
-        if constexpr (WK == W_CONST0) {
+        if constexpr (HAS_O) {
+            ldv<V>(od + c, r.o);
+        } else {
 #pragma unroll
             for (int m = 0; m < V; ++m) r.o[m] = wd;
-        } else {
-            ldv<V>(od + c, r.o);
         }
         if constexpr (POST) {
             if constexpr (V == 4) {
@@ -381,30 +404,32 @@ __device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int
             }
         }
     };
+    auto form = [&](float fv, float o, float ev) {
+        if constexpr (IT == I_V) return fv;
+        else if constexpr (IT == I_P) return first ? fv : fmaf(beta, o, fv);  // no p_{k-1} to read in the first iteration
+        else return POST ? fmaf(kMgSigma, ev, fv * o) : fv * o;
+    };
     auto iterate = [&](const Raw &r, float v[V]) {
 #pragma unroll
-        for (int m = 0; m < V; ++m) {
-            v[m] = r.f[m] * r.o[m];
-            if constexpr (POST) v[m] = fmaf(kMgSigma, r.e[m >> 1], v[m]);
-        }
+        for (int m = 0; m < V; ++m) v[m] = form(r.f[m], r.o[m], r.e[m >> 1]);
     };
     // flat index of the parents of this row at plane k, of the row outside the pair, of the edge point
-    auto par = [&](int k) { return (int64_t)(k >> 1) * csz; };
+    auto par = [&](int k) { return (unsigned)((k - kb) >> 1) * csz; };
     const int p0 = (s.j >> 1) * cnx + (s.i0 >> 1), po = p0 + (s.hi ? cnx : -cnx);
     const bool ed = s.el || s.er;  // the point beside the segment that no lane of the half holds
     const int de = s.el ? -1 : V, pe = (s.j >> 1) * cnx + ((s.i0 + de) >> 1);
     struct Edge {
         float f = 0.f, o = 0.f, e = 0.f;
     };
-    auto edge = [&](Edge &g, int64_t c, int k) {
+    auto edge = [&](Edge &g, unsigned c, int k) {
         if (!ed) return;
         g.f = __ldg(f + c + de);
-        g.o = WK == W_CONST0 ? wd : __ldg(od + c + de);
+        g.o = HAS_O ? __ldg(od + c + de) : wd;
         if constexpr (POST) g.e = __ldg(e + par(k) + pe);
     };
     MgCol<V, WK> col;
     col.start(a, L, s, k0);
-    int64_t c = (int64_t)s.c + (int64_t)k0 * sz;
+    unsigned c = s.c + (unsigned)(k0 - kb) * sz;
     Raw rc, rn, ro;
     Edge g;
     float vm[V], vc[V];
@@ -421,6 +446,8 @@ __device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int
         iterate(rm, vm);
     }
     iterate(rc, vc);
+    const int64_t cb = (int64_t)kb * sz;
+#pragma unroll 1
     for (int k = k0; k < k1; ++k, c += sz) {
         Raw r2, ron;
         Edge gn;
@@ -429,14 +456,13 @@ __device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int
             if (s.eo) fetch(ron, c + sz + s.dro, par(k + 1) + po);
             edge(gn, c + sz, k + 1);
         }
-        col.plane(a, L, s, c, k);
+        col.plane(a, L, s, cb, c, k);
         float vn[V], vo[V], vi[V];
 #pragma unroll
         for (int m = 0; m < V; ++m) vn[m] = vo[m] = 0.f;
         if (k + 1 < L.nz) iterate(rn, vn);
         if (s.eo) iterate(ro, vo);
-        float ve = g.f * g.o;
-        if constexpr (POST) ve = fmaf(kMgSigma, g.e, ve);
+        const float ve = form(g.f, g.o, g.e);
 #pragma unroll
         for (int m = 0; m < V; ++m) vi[m] = __shfl_xor_sync(0xffffffffu, vc[m], 16);
         const float xls = __shfl_up_sync(0xffffffffu, vc[V - 1], 1), xrs = __shfl_down_sync(0xffffffffu, vc[0], 1);
@@ -446,15 +472,25 @@ __device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int
         for (int m = 0; m < V; ++m) {
             float w[6], D;
             col.get(a, m, w, D);
-            float off = w[0] * (m == 0 ? xl : vc[m > 0 ? m - 1 : 0]);
-            off = fmaf(w[1], m == V - 1 ? xr : vc[m < V - 1 ? m + 1 : 0], off);
-            off = fmaf(w[2], vi[m], off);
-            off = fmaf(w[3], vo[m], off);
-            off = fmaf(w[4], vm[m], off);
-            off = fmaf(w[5], vn[m], off);
-            av[m] = fmaf(D, vc[m], -off);
+            const float xm = m == 0 ? xl : vc[m > 0 ? m - 1 : 0], xp = m == V - 1 ? xr : vc[m < V - 1 ? m + 1 : 0];
+            if constexpr (IT == I_P || IT == I_V) {
+                float q = w[0] * (vc[m] - xm);
+                q = fmaf(w[1], vc[m] - xp, q);
+                q = fmaf(w[2], vc[m] - vi[m], q);
+                q = fmaf(w[3], vc[m] - vo[m], q);
+                q = fmaf(w[4], vc[m] - vm[m], q);
+                av[m] = fmaf(w[5], vc[m] - vn[m], q);
+            } else {
+                float off = w[0] * xm;
+                off = fmaf(w[1], xp, off);
+                off = fmaf(w[2], vi[m], off);
+                off = fmaf(w[3], vo[m], off);
+                off = fmaf(w[4], vm[m], off);
+                off = fmaf(w[5], vn[m], off);
+                av[m] = fmaf(D, vc[m], -off);
+            }
         }
-        body(k, c, av, vc, rc.f, rc.o);
+        body(k, cb, c, av, vc, rc.f, rc.o);
 #pragma unroll
         for (int m = 0; m < V; ++m) {
             vm[m] = vc[m];
@@ -467,6 +503,29 @@ __device__ __forceinline__ void mg_march(const MgStep &a, const MgSeg<V> &s, int
     }
 }
 
+// The level kernels' work: blocks of kMgThreads / 2 segments times planes
+// (coarse ones for the restriction), `planes` per block of segments, split
+// evenly over the grid's CTAs as runs of planes; fn(block of segments, planes
+// [k0, k1)) per run.
+template <typename F>
+__device__ __forceinline__ void mg_runs(const MgLevel &L, int seg, int planes, F fn) {
+    const int64_t np = (int64_t)(L.nx / seg) * (L.ny / 2), units = (np + kMgThreads / 2 - 1) / (kMgThreads / 2) * planes;
+    int64_t u = units * blockIdx.x / gridDim.x;
+    const int64_t u1 = units * (blockIdx.x + 1) / gridDim.x;
+    unsigned blk = (unsigned)(u / planes);
+    int k = (int)(u - (int64_t)blk * planes);
+    while (u < u1) {
+        const int n = (int)min(min((int64_t)(planes - k), u1 - u), kMgRunPoints / ((int64_t)L.nx * L.ny) + 1);
+        fn(blk * (kMgThreads / 32) + (threadIdx.x >> 5), k, k + n);
+        u += n;
+        k += n;
+        if (k == planes) {
+            k = 0;
+            ++blk;
+        }
+    }
+}
+
 // One warp's restriction of the coarse planes [K0, K1) of its segments.
 template <int V, int WK>
 __device__ __forceinline__ void mg_restrict_warp(const MgStep &a, unsigned wseg, int K0, int K1) {
@@ -475,8 +534,8 @@ __device__ __forceinline__ void mg_restrict_warp(const MgStep &a, unsigned wseg,
     const MgSeg<V> s(a.L, wseg);
     float sum[V / 2];
     float *fc = a.c + (int64_t)(s.j >> 1) * cnx + (s.i0 >> 1);
-    mg_march<V, WK, false>(a, s, 2 * K0, 2 * K1,
-                                 [&](int k, int64_t, const float *av, const float *, const float *f, const float *) {
+    mg_march<V, WK, I_U>(a, a.L.f, a.L.od, 0.f, false, s, 2 * K0, 2 * K1,
+                                 [&](int k, int64_t, unsigned, const float *av, const float *, const float *f, const float *) {
                                      float r[V / 2];
 #pragma unroll
                                      for (int m = 0; m < V / 2; ++m) {
@@ -504,16 +563,16 @@ __device__ __forceinline__ float mg_post_warp(const MgStep &a, unsigned wseg, in
     const MgSeg<V> s(a.L, wseg);
     float *out = a.L.w;
     float acc = 0.f;
-    mg_march<V, WK, true>(a, s, k0, k1,
-                                [&](int, int64_t c, const float *av, const float *v, const float *f, const float *o) {
+    mg_march<V, WK, I_POST>(a, a.L.f, a.L.od, 0.f, false, s, k0, k1,
+                                [&](int, int64_t cb, unsigned c, const float *av, const float *v, const float *f, const float *o) {
                                     float r[V];
 #pragma unroll
                                     for (int m = 0; m < V; ++m) r[m] = fmaf(o[m], f[m] - av[m], v[m]);
                                     if (!s.live) return;
                                     if constexpr (V == 4) {
-                                        *reinterpret_cast<float4 *>(out + c) = make_float4(r[0], r[1], r[2], r[3]);
+                                        *reinterpret_cast<float4 *>(out + cb + c) = make_float4(r[0], r[1], r[2], r[3]);
                                     } else {
-                                        *reinterpret_cast<float2 *>(out + c) = make_float2(r[0], r[1]);
+                                        *reinterpret_cast<float2 *>(out + cb + c) = make_float2(r[0], r[1]);
                                     }
 #pragma unroll
                                     for (int m = 0; m < V; ++m) acc = fmaf(f[m], r[m], acc);
@@ -521,13 +580,11 @@ __device__ __forceinline__ float mg_post_warp(const MgStep &a, unsigned wseg, in
     return acc;
 }
 
-// f_{l+1} = P^T (f - A u), u = (omega / D) f; a block marches kper coarse planes.
+// f_{l+1} = P^T (f - A u), u = (omega / D) f; 
 template <int V, int WK>
-__global__ void __launch_bounds__(kMgThreads) mg_restrict_kernel(const MgStep a, unsigned nblk, int kper) {
+__global__ void __launch_bounds__(kMgThreads, mg_min_blocks(WK)) mg_restrict_kernel(const MgStep a) {
     if (mg_stand_down(a.st)) return;
-    const int K0 = blockIdx.y * kper, K1 = min(a.L.nz / 2, K0 + kper);
-    for (unsigned blk = blockIdx.x; blk < nblk; blk += gridDim.x)
-        mg_restrict_warp<V, WK>(a, blk * (kMgThreads / 32) + (threadIdx.x >> 5), K0, K1);
+    mg_runs(a.L, V, a.L.nz / 2, [&](unsigned wseg, int K0, int K1) { mg_restrict_warp<V, WK>(a, wseg, K0, K1); });
 }
 
 // The scalars a V-cycle inside a solve ends with: r.z -> beta (the first time
@@ -556,18 +613,77 @@ __device__ __forceinline__ void mg_rz_finish(const MgDot &d, double rz) {
 // result.  DOT (level 0 inside a solve): also f.out, r.z of the solver,
 // instead of a pass of its own over both vectors.
 template <int V, int WK, bool DOT>
-__global__ void __launch_bounds__(kMgThreads)
-    mg_post_kernel(const MgStep a, unsigned nblk, int kper, const MgDot d) {
+__global__ void __launch_bounds__(kMgThreads, mg_min_blocks(WK)) mg_post_kernel(const MgStep a, const MgDot d) {
     if (mg_stand_down(a.st)) return;
-    const int k0 = blockIdx.y * kper, k1 = min(a.L.nz, k0 + kper);
     float acc[1] = {0.f};
-    for (unsigned blk = blockIdx.x; blk < nblk; blk += gridDim.x)
-        acc[0] += mg_post_warp<V, WK>(a, blk * (kMgThreads / 32) + (threadIdx.x >> 5), k0, k1);
+    mg_runs(a.L, V, a.L.nz, [&](unsigned wseg, int k0, int k1) { acc[0] += mg_post_warp<V, WK>(a, wseg, k0, k1); });
     if constexpr (DOT) {
         double part[1], tot[1];
         block_sum<1, kMgThreads>(acc, part);
         if (grid_sum_last<1, kMgThreads>(part, d.partials, &d.st->ticket[1], tot) && threadIdx.x == 0)
             mg_rz_finish(d, tot[0]);
+    }
+}
+
+// The solver's passes A and R on the same march, for grids on which the
+// passes' TMA ring is a chain of planes in a few CTAs (kMgDirectPoints).
+//   A: p_k = z + beta p_{k-1} (p_out), d += alpha_{k-1} p_{k-1}, p.Ap -> alpha
+//   R: r -= alpha A p_k, r.r -> convergence test and replacement trigger
+struct MgPass {
+    float *p0, *p1, *d, *r;
+    SolveState *st;
+    double *partials;
+    cudaGraphConditionalHandle cond, cond_rep;
+    int use_cond;
+};
+template <int WK, bool A>
+__global__ void __launch_bounds__(kMgThreads, mg_min_blocks(WK)) mg_pass_kernel(const MgStep a, const MgPass d) {
+    SolveState *st = d.st;
+    if (st->done) return;
+    const int it = st->it;
+    const float alpha = (float)st->alpha, beta = (float)st->beta;  // A: alpha_{k-1}
+    const bool pending = st->pending != 0;
+    float *pk = it & 1 ? d.p1 : d.p0;
+    const float *pp = it & 1 ? d.p0 : d.p1;
+    float acc[1] = {0.f};
+    mg_runs(a.L, 4, a.L.nz, [&](unsigned wseg, int k0, int k1) {
+        const MgSeg<4> s(a.L, wseg);
+        if constexpr (A) {
+            mg_march<4, WK, I_P>(a, a.L.f, pp, beta, it == 0, s, k0, k1,
+                                 [&](int, int64_t cb, unsigned c, const float *av, const float *v, const float *, const float *o) {
+                                     if (!s.live) return;
+                                     *reinterpret_cast<float4 *>(pk + cb + c) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+                                     for (int m = 0; m < 4; ++m) acc[0] = fmaf(v[m], av[m], acc[0]);
+                                     if (!pending) return;
+                                     float4 *dp = reinterpret_cast<float4 *>(d.d + cb + c);
+                                     const float4 t = *dp;
+                                     *dp = make_float4(fmaf(alpha, o[0], t.x), fmaf(alpha, o[1], t.y),
+                                                       fmaf(alpha, o[2], t.z), fmaf(alpha, o[3], t.w));
+                                 });
+        } else {
+            mg_march<4, WK, I_V>(a, pk, nullptr, 0.f, false, s, k0, k1,
+                                 [&](int, int64_t cb, unsigned c, const float *av, const float *, const float *, const float *) {
+                                     if (!s.live) return;
+                                     float4 *rp = reinterpret_cast<float4 *>(d.r + cb + c);
+                                     const float4 t = *rp;
+                                     const float r[4] = {fmaf(-alpha, av[0], t.x), fmaf(-alpha, av[1], t.y),
+                                                         fmaf(-alpha, av[2], t.z), fmaf(-alpha, av[3], t.w)};
+                                     *rp = make_float4(r[0], r[1], r[2], r[3]);
+#pragma unroll
+                                     for (int m = 0; m < 4; ++m) acc[0] = fmaf(r[m], r[m], acc[0]);
+                                 });
+        }
+    });
+    double part[1], tot[1];
+    block_sum<1, kMgThreads>(acc, part);
+    if (!grid_sum_last<1, kMgThreads>(part, d.partials, &st->ticket[A ? K_PASSA : K_PASSR], tot) || threadIdx.x != 0)
+        return;
+    if constexpr (A) passa_finish(st, tot[0], false);
+    else passr_finish(st, it, tot[0], false);
+    if (d.use_cond) {
+        cudaGraphSetConditional(d.cond, st->done ? 0u : 1u);
+        cudaGraphSetConditional(d.cond_rep, st->replace ? 1u : 0u);
     }
 }
 
@@ -583,8 +699,8 @@ __global__ void __launch_bounds__(kMgThreads)
 // the transfers between levels decode, one coarse cell a thread.  The launch's
 // parameters are kept to a line or two of the constant cache, which is cold:
 // as an array of levels they took 11000 cycles to read, a miss after another.
-// 16^3 and below: 35 us with the levels in global memory -> 8 us (15700
-// cycles: copies 4000, 16^3 8300, 8^3 and transfers 2800, 24 sweeps 2970).
+// 16^3 and below: 36 us with the levels in global memory -> 11.5 us (ncu;
+// 15700 cycles: copies 4000, 16^3 7800, 8^3 900, 24 sweeps 2970).
 
 struct MgTail {
     const SolveState *st;
@@ -598,8 +714,8 @@ struct MgTail {
 
 // What sweeps a coarsest level that is the whole tail: one CTA, or above
 // kMgTailCells cells a cluster, its halo planes exchanged through distributed
-// shared memory (31^3 cells, the coarsest level of 248^3: about 700 us in one
-// CTA with the vectors in global memory -> about 30 us).
+// shared memory (31^3 cells, the coarsest level of 248^3: 700 us in one CTA with
+// the vectors in global memory -> 35 us).
 struct MgSweep {
     int ppc, na;  // planes per CTA, sweeping CTAs
     unsigned ctas;
@@ -1134,49 +1250,48 @@ cudaError_t mg_setup(const MgArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// The level kernels' grid: blocks of 128 segments of row pairs times runs of
-// planes (`planes` of them, fine or coarse), kMgBlocks blocks per SM in all.
-constexpr int kMgBlocks = 3;
-struct MgGrid {
-    dim3 grid;
-    unsigned nblk;
-    int kper;
-};
-MgGrid mg_level_grid(const MgLevel &L, int V, int planes) {
+// CTAs of a level kernel: what the device holds at once, and no more than its
+// units of work (mg_runs).
+template <int V, int WK, int KIND = 0, typename K>
+unsigned mg_level_grid(K kernel, const MgLevel &L, int planes) {  // an instance, and so a static, per kernel
+    static const int per_sm = [kernel] {
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kMgThreads, 0);
+        return std::max(1, n);
+    }();
     const int64_t np = (int64_t)(L.nx / V) * (L.ny / 2);
-    const int64_t nblk = (np + kMgThreads / 2 - 1) / (kMgThreads / 2);
-    const int64_t want = std::max<int64_t>(1, (int64_t)device_sm_count() * kMgBlocks / nblk);
-    const int kper = (int)((planes + std::min<int64_t>(want, planes) - 1) / std::min<int64_t>(want, planes));
-    // at most kMaxPassBlocks blocks leave a partial sum
-    const unsigned gz = (unsigned)((planes + kper - 1) / kper);
-    const unsigned gx = (unsigned)std::min<int64_t>(nblk, std::max<unsigned>(1u, kMaxPassBlocks / gz));
-    return MgGrid{dim3(gx, gz), (unsigned)nblk, kper};
+    const int64_t units = (np + kMgThreads / 2 - 1) / (kMgThreads / 2) * planes;
+    return (unsigned)std::min<int64_t>(std::min<int64_t>(units, kMaxPassBlocks), (int64_t)device_sm_count() * per_sm);
+}
+
+// f(V, WK) for a level's row length and kind of weights
+template <typename F>
+void mg_dispatch(const MgArgs &a, int l, F f) {
+    using V4 = std::integral_constant<int, 4>;
+    using V2 = std::integral_constant<int, 2>;
+    if (l > 0) {
+        using Stored = std::integral_constant<int, W_STORED>;
+        if (a.lv[l].nx % 4 == 0) f(V4{}, Stored{});
+        else f(V2{}, Stored{});
+    } else if (!a.block) {
+        f(V4{}, std::integral_constant<int, W_CONST0>{});
+    } else if (a.ob.kbx % 4 == 0) {
+        f(V4{}, std::integral_constant<int, W_TABV>{});
+    } else {
+        f(V4{}, std::integral_constant<int, W_TAB0>{});
+    }
+}
+MgStep mg_step(const MgArgs &a, int l, float *c) {
+    return MgStep{a.st, a.lv[l], c, a.ob, a.tab, a.rkbx, a.rkby, a.rkbz};
 }
 
 // z = M f0 (a.lv[0].f -> a.lv[0].w); dot: also r.z and what follows from it
 cudaError_t mg_vcycle(const MgArgs &a, cudaStream_t s, const MgDot *dot) {
     const int l0 = mg_l0(a), lc = a.L - 1;
-    auto step = [&](int l, float *c) { return MgStep{a.st, a.lv[l], c, a.ob, a.tab, a.rkbx, a.rkby, a.rkbz}; };
-    // f(V, WK) for the level's row length and kind of weights
-    auto dispatch = [&](int l, auto f) {
-        using V4 = std::integral_constant<int, 4>;
-        using V2 = std::integral_constant<int, 2>;
-        if (l > 0) {
-            using Stored = std::integral_constant<int, W_STORED>;
-            if (a.lv[l].nx % 4 == 0) f(V4{}, Stored{});
-            else f(V2{}, Stored{});
-        } else if (!a.block) {
-            f(V4{}, std::integral_constant<int, W_CONST0>{});
-        } else if (a.ob.kbx % 4 == 0) {
-            f(V4{}, std::integral_constant<int, W_TABV>{});
-        } else {
-            f(V4{}, std::integral_constant<int, W_TAB0>{});
-        }
-    };
     for (int l = 0; l < l0; ++l)
-        dispatch(l, [&](auto v, auto wk) {
-            const MgGrid g = mg_level_grid(a.lv[l], v(), a.lv[l + 1].nz);
-            mg_restrict_kernel<v(), wk()><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].f), g.nblk, g.kper);
+        mg_dispatch(a, l, [&](auto v, auto wk) {
+            const unsigned g = mg_level_grid<v(), wk()>(mg_restrict_kernel<v(), wk()>, a.lv[l], a.lv[l + 1].nz);
+            mg_restrict_kernel<v(), wk()><<<g, kMgThreads, 0, s>>>(mg_step(a, l, a.lv[l + 1].f));
         });
     if (l0 < lc) {
         const MgLevel &L = a.lv[l0];
@@ -1219,15 +1334,16 @@ cudaError_t mg_vcycle(const MgArgs &a, cudaStream_t s, const MgDot *dot) {
     MgDot none;
     memset(&none, 0, sizeof(none));
     for (int l = l0 - 1; l >= 0; --l)
-        dispatch(l, [&](auto v, auto wk) {
-            const MgGrid g = mg_level_grid(a.lv[l], v(), a.lv[l].nz);
+        mg_dispatch(a, l, [&](auto v, auto wk) {
             if constexpr (wk() != W_STORED) {
                 if (dot) {
-                    mg_post_kernel<v(), wk(), true><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].w), g.nblk, g.kper, *dot);
+                    const unsigned g = mg_level_grid<v(), wk(), 1>(mg_post_kernel<v(), wk(), true>, a.lv[l], a.lv[l].nz);
+                    mg_post_kernel<v(), wk(), true><<<g, kMgThreads, 0, s>>>(mg_step(a, l, a.lv[l + 1].w), *dot);
                     return;
                 }
             }
-            mg_post_kernel<v(), wk(), false><<<g.grid, kMgThreads, 0, s>>>(step(l, a.lv[l + 1].w), g.nblk, g.kper, none);
+            const unsigned g = mg_level_grid<v(), wk(), 2>(mg_post_kernel<v(), wk(), false>, a.lv[l], a.lv[l].nz);
+            mg_post_kernel<v(), wk(), false><<<g, kMgThreads, 0, s>>>(mg_step(a, l, a.lv[l + 1].w), none);
         });
     if (dot && l0 == 0) mg_rz_kernel<<<mg_grid(a.lv[0].m), kMgThreads, 0, s>>>(a.lv[0].m, a.lv[0].f, a.lv[0].w, *dot);
     return cudaGetLastError();
@@ -1254,9 +1370,25 @@ struct MgSolve {
     PassArgs ar;
     MgArgs mg;
     float *r, *z;
+    bool direct;  // passes A and R on the march
 
     cudaError_t launch_r(cudaStream_t s) {
         return GB_CFG_DISPATCH(sp.cfg_b, float, K_PASSR, true, Op, K::launch(mr, ar, sp.op, sp.gb.grid(), s));
+    }
+    // pass A (or R) on the march
+    template <bool A>
+    cudaError_t launch_direct(cudaStream_t s) {
+        const MgLevel &L = mg.lv[0];
+        MgStep t = mg_step(mg, 0, nullptr);
+        t.L.f = z;
+        const MgPass d{sp.p0, sp.p1, sp.d, r, sp.st, sp.partials, sp.cond_loop, sp.cond_rep, sp.use_cond};
+        mg_dispatch(mg, 0, [&](auto, auto wk) {
+            if constexpr (wk() != W_STORED) {
+                const unsigned g = mg_level_grid<4, wk(), A ? 3 : 4>(mg_pass_kernel<wk(), A>, L, L.nz);
+                mg_pass_kernel<wk(), A><<<g, kMgThreads, 0, s>>>(t, d);
+            }
+        });
+        return cudaGetLastError();
     }
     // the V-cycle and r.z
     cudaError_t launch_m(cudaStream_t s, int init) {
@@ -1321,9 +1453,9 @@ struct MgSolve {
             e = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
             if (e) break;
             cap_b = true;
-            e = sp.launch_a(bs);
+            e = direct ? launch_direct<true>(bs) : sp.launch_a(bs);
             if (e) break;
-            e = launch_r(bs);
+            e = direct ? launch_direct<false>(bs) : launch_r(bs);
             if (e) break;
             cudaGraph_t rbody = nullptr;
             e = add_cond(bs, rep, cudaGraphCondTypeIf, &rbody);
@@ -1392,6 +1524,7 @@ int mg_solve_op(const gbpcg_grid &g, const Op &op, const double *b, double *x, c
     P.ar.o1 = P.r;
     (void)GB_CFG_DISPATCH(cb, float, K_PASSR, true, Op, K::prepare());
     P.mg = mg_args(g, ws, M, P.r, P.z, P.sp.st);
+    P.direct = g.ny % 2 == 0 && P.mg.lv[0].m <= kMgDirectPoints;
     cudaGraph_t graph = nullptr;
     if (int rc = P.capture(&graph)) return rc;
     cudaGraphExec_t exec = nullptr;
