@@ -365,10 +365,10 @@ int gbpcg_sell_workspace_size(const gbpcg_sell *matrix, size_t *bytes);
  * symmetric positive definite.  b (read), x (initial guess in, solution
  * out): DEVICE FP64 arrays of n elements; opts: io_dtype F64, storage F32,
  * Jacobi, no flags, tol and maxit as for gbpcg_pcg_solve, workspace of
- * gbpcg_sell_workspace_size bytes (256-byte aligned).  Per iteration three
- * kernels (q = A p with p.q; x += alpha p in FP64, r -= alpha q with r.r and
- * r.z; p = D^-1 r + beta p), the scalars on the device, the loop one CUDA
- * graph.  The residual is replaced by b - A x computed in FP64 when it has
+ * gbpcg_sell_workspace_size bytes (256-byte aligned).  Per iteration two
+ * kernels (p = z + beta p, q = A p with p.q, and the last iteration's x +=
+ * alpha p in FP64; r -= alpha q, z = D^-1 r with r.r and r.z), the scalars on
+ * the device, the loop one CUDA graph.  The residual is replaced by b - A x computed in FP64 when it has
  * dropped two decades since the last replacement and when it meets the
  * tolerance, so convergence is decided on a true residual.  Fills *result
  * (rel_res_true: FP64 ||b - A x|| / ||b||); synchronises `stream`.

@@ -10,18 +10,22 @@
 // 128-byte line.  Short rows are padded with value 0 and their own row as
 // the column (an in-bounds gather that adds nothing).
 //
-// The solver is the textbook iteration split into three kernels per
+// The solver is the textbook iteration split into two kernels per
 // iteration, each with its reductions fused in and the scalars kept on the
 // device, the whole loop one CUDA graph (as the stencil solver):
-//   spmv:    q = A p, p.q               -> alpha (last CTA)
-//   update:  x += alpha p (FP64 x), r -= alpha q, z = D^-1 r, r.r, r.z
+//   spmv:    p = z + beta p formed at every entry from pairs (z, p) of the
+//            last iteration (one 8-byte gather), q = A p, p.q -> alpha (last
+//            CTA); x += alpha p of the last iteration (FP64 x)
+//   update:  r -= alpha q, z = D^-1 r, r.r, r.z, the new pairs (z, p)
 //                                       -> beta, convergence, replacement
-//   p:       p = z + beta p  (z recomputed from r)
 // plus an FP64 residual b - A x (gathering the FP64 x) at the start, when
 // the recursive residual meets the tolerance or has dropped two decades
-// since the last replacement, and at the end.  Per iteration 108 bytes per
-// row for a seven-point matrix (values and columns 56, gathers and vectors
-// 52), against the matrix-free passes' 32.
+// since the last replacement, and at the end; x is brought up to date (flush)
+// before the last two.  Per iteration 116 bytes per row for a seven-point
+// matrix (values and columns 56, gathers and vectors 60), against the
+// matrix-free passes' 32.  As three kernels (p a pass of its own) an iteration
+// of 8000 rows took 21 us and of 1.1 million rows 38.0; two kernels 17.5 and
+// 37.8 (the matrix and the vectors stream from L2).
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -69,21 +73,48 @@ __global__ void __launch_bounds__(kSellThreads)
     }
 }
 
-// q = A p and the partial p.q; last CTA: alpha.
+// Entries of a row taken together: their columns and values are loaded before
+// the first gather, so a row costs two memory latencies and not two per entry.
+constexpr int kSellBatch = 8;
+
+// q = A p with p = z + beta p_{k-1} (pn), the partial p.q, and the pending
+// x += alpha_{k-1} p_{k-1}; last CTA: alpha.
 __global__ void __launch_bounds__(kSellThreads)
-    sell_spmv_dot_kernel(const SellDev A, const float *__restrict__ p, float *__restrict__ q, SolveState *st,
-                         double *partials) {
+    sell_spmv_dot_kernel(const SellDev A, const float2 *__restrict__ zp, float *__restrict__ pn, float *__restrict__ q,
+                         double *__restrict__ x, SolveState *st, double *partials) {
     if (st->done) return;
+    const float beta = (float)st->beta;
+    const double alpha = st->alpha;
+    const bool pending = st->pending != 0;
     float acc[1] = {0.f};
     for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < A.n;
          i += (int64_t)gridDim.x * kSellThreads) {
         int64_t e;
         int w;
         sell_row(A, i, e, w);
+        const float2 own = __ldg(zp + i);
+        const double xi = pending ? x[i] : 0.0;
         float s = 0.f;
-        for (int j = 0; j < w; ++j, e += kSell) s = fmaf(__ldg(A.val + e), __ldg(p + __ldg(A.col + e)), s);
+        for (int j = 0; j < w; j += kSellBatch, e += kSellBatch * kSell) {
+            int c[kSellBatch];
+            float v[kSellBatch];
+            float2 g[kSellBatch];
+#pragma unroll
+            for (int m = 0; m < kSellBatch; ++m) {
+                const bool in = j + m < w;
+                c[m] = in ? __ldg(A.col + e + m * kSell) : (int)i;
+                v[m] = in ? __ldg(A.val + e + m * kSell) : 0.f;
+            }
+#pragma unroll
+            for (int m = 0; m < kSellBatch; ++m) g[m] = j + m < w ? __ldg(zp + c[m]) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int m = 0; m < kSellBatch; ++m) s = fmaf(v[m], fmaf(beta, g[m].y, g[m].x), s);
+        }
+        const float pi = fmaf(beta, own.y, own.x);
+        pn[i] = pi;
         q[i] = s;
-        acc[0] = fmaf(p[i], s, acc[0]);
+        acc[0] = fmaf(pi, s, acc[0]);
+        if (pending) x[i] = fma(alpha, (double)own.y, xi);
     }
     double part[1], tot[1];
     block_sum<1, kSellThreads>(acc, part);
@@ -91,26 +122,41 @@ __global__ void __launch_bounds__(kSellThreads)
         passa_finish(st, tot[0], false);
 }
 
-// x += alpha p (FP64), r -= alpha q, z = D^-1 r; partials r.r, r.z; last CTA:
-// beta, the convergence test and the replacement trigger.
+// r -= alpha q, z = D^-1 r, the pairs (z, p); partials r.r, r.z; last CTA:
+// beta, the convergence test and the replacement trigger.  Four rows a thread
+// in flight.
 __global__ void __launch_bounds__(kSellThreads)
-    sell_update_kernel(const SellDev A, double *__restrict__ x, const float *__restrict__ p,
-                       const float *__restrict__ q, float *__restrict__ r, SolveState *st, double *partials,
+    sell_update_kernel(const SellDev A, const float *__restrict__ pn, const float *__restrict__ q,
+                       float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
                        cudaGraphConditionalHandle cond, cudaGraphConditionalHandle cond_rep, int use_cond) {
     if (st->done) return;
+    constexpr int R = 4;
     const int it = st->it;
-    const double alpha = st->alpha;
-    const float af = (float)alpha;
+    const float af = (float)st->alpha;
+    const int64_t step = (int64_t)gridDim.x * kSellThreads;
     float acc[2] = {0.f, 0.f};
-    for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < A.n;
-         i += (int64_t)gridDim.x * kSellThreads) {
-        const float pi = p[i];
-        x[i] = fma(alpha, (double)pi, x[i]);
-        const float ri = fmaf(-af, q[i], r[i]);
-        r[i] = ri;
-        const float zi = __ldg(A.inv_diag + i) * ri;
-        acc[0] = fmaf(ri, ri, acc[0]);
-        acc[1] = fmaf(ri, zi, acc[1]);
+    for (int64_t i0 = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i0 < A.n; i0 += R * step) {
+        float qi[R], ri[R], di[R], pi[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+            const int64_t i = i0 + m * step;
+            const bool in = i < A.n;
+            qi[m] = in ? q[i] : 0.f;
+            ri[m] = in ? r[i] : 0.f;
+            di[m] = in ? __ldg(A.inv_diag + i) : 0.f;
+            pi[m] = in ? pn[i] : 0.f;
+        }
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+            const int64_t i = i0 + m * step;
+            if (i >= A.n) break;
+            const float rn = fmaf(-af, qi[m], ri[m]);
+            r[i] = rn;
+            const float zi = di[m] * rn;
+            zp[i] = make_float2(zi, pi[m]);
+            acc[0] = fmaf(rn, rn, acc[0]);
+            acc[1] = fmaf(rn, zi, acc[1]);
+        }
     }
     double part[2], tot[2];
     block_sum<2, kSellThreads>(acc, part);
@@ -123,14 +169,13 @@ __global__ void __launch_bounds__(kSellThreads)
     }
 }
 
-// p = D^-1 r + beta p (p = D^-1 r when beta = 0 and p was zeroed).
+// the pending x += alpha p, before x is used (p in the pairs)
 __global__ void __launch_bounds__(kSellThreads)
-    sell_p_kernel(const SellDev A, const float *__restrict__ r, float *__restrict__ p, const SolveState *st) {
-    if (st->done) return;
-    const float beta = (float)st->beta;
-    for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < A.n;
-         i += (int64_t)gridDim.x * kSellThreads)
-        p[i] = fmaf(beta, p[i], __ldg(A.inv_diag + i) * r[i]);
+    sell_flush_kernel(int64_t n, double *__restrict__ x, const float2 *__restrict__ zp, const SolveState *st) {
+    if (!st->pending) return;
+    const double alpha = st->alpha;
+    for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSellThreads)
+        x[i] = fma(alpha, (double)zp[i].y, x[i]);
 }
 
 // r = b - A x with FP64 products and sums (x gathered in FP64); r stored as
@@ -140,8 +185,8 @@ __global__ void __launch_bounds__(kSellThreads)
 template <int MODE>
 __global__ void __launch_bounds__(kSellThreads)
     sell_residual_kernel(const SellDev A, const double *__restrict__ b, const double *__restrict__ x,
-                         float *__restrict__ r, SolveState *st, double *partials, cudaGraphConditionalHandle cond,
-                         int use_cond) {
+                         float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
+                         cudaGraphConditionalHandle cond, int use_cond) {
     if (MODE == RES_REPLACE && (!st->replace || st->done)) return;
     if (MODE == RES_TRUE && st->true_known) return;
     constexpr int NV = res64_nv<MODE>();
@@ -160,7 +205,9 @@ __global__ void __launch_bounds__(kSellThreads)
         } else {
             const float rf = (float)ri;
             r[i] = rf;
-            const double zi = (double)(__ldg(A.inv_diag + i) * rf);
+            const float zf = __ldg(A.inv_diag + i) * rf;
+            zp[i] = make_float2(zf, MODE == RES_INIT ? 0.f : zp[i].y);
+            const double zi = (double)zf;
             s[0] = fma(ri, ri, s[0]);
             s[1] = fma(ri, zi, s[1]);
             s[2] = fma(bi, bi, s[2]);
@@ -290,7 +337,7 @@ std::vector<int64_t> slice_layout(int64_t n, LenFn len) {
 }
 
 struct SellWs {
-    size_t state, partials, r, p, q, total;
+    size_t state, partials, r, p, q, zp, total;
 };
 SellWs sell_ws(int64_t n) {
     SellWs w;
@@ -300,6 +347,7 @@ SellWs sell_ws(int64_t n) {
     w.r = o; o += round256((size_t)n * 4);
     w.p = o; o += round256((size_t)n * 4);
     w.q = o; o += round256((size_t)n * 4);
+    w.zp = o; o += round256((size_t)n * 8);
     w.total = o;
     return w;
 }
@@ -320,33 +368,38 @@ struct SellPlan {
     SolveState *st;
     double *partials;
     float *r, *p, *q;
+    float2 *zp;  // (z, p) of the last iteration
     double tol;
     int maxit;
     unsigned grid;
     cudaGraphConditionalHandle cond = 0, cond_rep = 0;
     int use_cond = 0;
 
+    template <int MODE>
+    void residual(cudaStream_t s) {
+        sell_residual_kernel<MODE><<<grid, kSellThreads, 0, s>>>(A, b, x, r, zp, st, partials, cond, use_cond);
+    }
+    void flush(cudaStream_t s) { sell_flush_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, zp, st); }
     void setup(cudaStream_t s) {
         sell_reset_kernel<<<1, 1, 0, s>>>(st, tol, maxit);
-        cudaMemsetAsync(p, 0, (size_t)A.n * 4, s);
-        sell_residual_kernel<RES_INIT><<<grid, kSellThreads, 0, s>>>(A, b, x, r, st, partials, cond, use_cond);
+        residual<RES_INIT>(s);
         sell_zero_x_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, st);
-        sell_p_kernel<<<grid, kSellThreads, 0, s>>>(A, r, p, st);
     }
     void body(cudaStream_t s) {
-        sell_spmv_dot_kernel<<<grid, kSellThreads, 0, s>>>(A, p, q, st, partials);
-        sell_update_kernel<<<grid, kSellThreads, 0, s>>>(A, x, p, q, r, st, partials, cond, cond_rep, use_cond);
+        sell_spmv_dot_kernel<<<grid, kSellThreads, 0, s>>>(A, zp, p, q, x, st, partials);
+        sell_update_kernel<<<grid, kSellThreads, 0, s>>>(A, p, q, r, zp, st, partials, cond, cond_rep, use_cond);
     }
     void replace(cudaStream_t s) {
-        sell_residual_kernel<RES_REPLACE><<<grid, kSellThreads, 0, s>>>(A, b, x, r, st, partials, cond, use_cond);
+        flush(s);
+        residual<RES_REPLACE>(s);
     }
-    void tail(cudaStream_t s) { sell_p_kernel<<<grid, kSellThreads, 0, s>>>(A, r, p, st); }
     void finish(cudaStream_t s) {
-        sell_residual_kernel<RES_TRUE><<<grid, kSellThreads, 0, s>>>(A, b, x, r, st, partials, cond, use_cond);
+        flush(s);
+        residual<RES_TRUE>(s);
     }
 };
 
-// reset -> r0, p0 -> while(cond){spmv; update; if(replace){residual}; p} -> true residual
+// reset -> r0, z0 -> while(cond){spmv; update; if(replace){flush; residual}} -> flush, true residual
 int sell_capture(SellPlan &P, cudaGraph_t *out) {
     cudaStream_t cs = nullptr, bs = nullptr, rs = nullptr;
     GB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -405,7 +458,6 @@ int sell_capture(SellPlan &P, cudaGraph_t *out) {
         e = cudaStreamEndCapture(rs, &tmp);
         cap_r = false;
         if (e) break;
-        P.tail(bs);
         e = cudaStreamEndCapture(bs, &tmp);
         cap_b = false;
         if (e) break;
@@ -552,6 +604,7 @@ int gbpcg_sell_pcg_solve(const gbpcg_sell *m, const double *b, double *x, const 
     P.r = reinterpret_cast<float *>(ws + W.r);
     P.p = reinterpret_cast<float *>(ws + W.p);
     P.q = reinterpret_cast<float *>(ws + W.q);
+    P.zp = reinterpret_cast<float2 *>(ws + W.zp);
     P.tol = opts->tol;
     P.maxit = opts->maxit;
     P.grid = sell_grid(m->n);
