@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(TX / (16 / sizeof(T)) * TY)
 
     SolveState *st = a.st;
     if constexpr (KIND == K_PASSA || KIND == K_PASSB || KIND == K_PASSR) {
-        if (st->done) return;  // uniform across the grid
+        if (st->done || st->replace) return;  // uniform across the grid (replace: see kLoopUnroll)
     }
     MarchScalars sc = read_scalars<KIND>(st);
     if constexpr (KIND == K_STENCIL) sc.alpha = a.scale;

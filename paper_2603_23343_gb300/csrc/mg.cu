@@ -53,6 +53,7 @@ constexpr int64_t kMgMaxCoarsest = 32768;
 // 92 -> 91 / 102 -> 98; 160^3 132 -> 132 / 165 -> 153; 192^3 179 -> 187 / 219 -> 224; 256^3 308 ->
 // 334 / 410 -> 433.
 constexpr int64_t kMgDirectPoints = 5000000;
+constexpr int kMgUnroll = 3;  // iterations per turn of the loop (kLoopUnroll)
 constexpr int kMgThreads = 256;
 constexpr int64_t kMgRunPoints = 1 << 27;  // a run of planes: its offsets fit 32 bits
 constexpr int kMgTailThreads = 1024;
@@ -82,7 +83,7 @@ struct MgArgs {
     OpBlock ob;
     const float4 *tab;  // block coefficients: the solver's per-block face table (the same weights, no divisions)
     float rkbx, rkby, rkbz;  // 1 / the block edges (mg_div)
-    const SolveState *st;  // inside a solve: every kernel stands down once st->done (NULL outside)
+    const SolveState *st;  // inside a solve: kernels stand down by its flags (NULL outside)
 };
 
 // n / d for 0 <= n < 2^22 and d >= 1, with rd = 1/d rounded to FP32:
@@ -139,7 +140,7 @@ __device__ __forceinline__ void mg_weights(const MgArgs &a, int l, int i, int j,
     mg_weights_stored(L, i, j, k, w, D);
 }
 
-__device__ __forceinline__ bool mg_stand_down(const SolveState *st) { return st && st->done; }
+__device__ __forceinline__ bool mg_stand_down(const SolveState *st) { return st && (st->done || st->replace); }
 
 // Launch geometry of the Galerkin kernel: a block is bx threads along x times
 // by rows along y and marches through zper planes.
@@ -639,7 +640,7 @@ struct MgPass {
 template <int WK, bool A>
 __global__ void __launch_bounds__(kMgThreads, mg_min_blocks(WK)) mg_pass_kernel(const MgStep a, const MgPass d) {
     SolveState *st = d.st;
-    if (st->done) return;
+    if (mg_stand_down(st)) return;
     const int it = st->it;
     const float alpha = (float)st->alpha, beta = (float)st->beta;  // A: alpha_{k-1}
     const bool pending = st->pending != 0;
@@ -1120,7 +1121,7 @@ __global__ void __launch_bounds__(kMgThreads) mg_galerkin_kernel(const MgArgs a,
 // r.z in a pass of its own, where the tail holds the whole hierarchy
 __global__ void __launch_bounds__(kMgThreads)
     mg_rz_kernel(int64_t n, const float *__restrict__ r, const float *__restrict__ z, const MgDot d) {
-    if (d.st->done) return;
+    if (mg_stand_down(d.st)) return;
     float acc[1] = {0.f};
     for (int64_t i = (int64_t)blockIdx.x * kMgThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kMgThreads)
         acc[0] = fmaf(r[i], z[i], acc[0]);
@@ -1453,9 +1454,11 @@ struct MgSolve {
             e = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
             if (e) break;
             cap_b = true;
-            e = direct ? launch_direct<true>(bs) : sp.launch_a(bs);
-            if (e) break;
-            e = direct ? launch_direct<false>(bs) : launch_r(bs);
+            for (int u = 0; u < kMgUnroll && !e; ++u) {
+                e = direct ? launch_direct<true>(bs) : sp.launch_a(bs);
+                if (!e) e = direct ? launch_direct<false>(bs) : launch_r(bs);
+                if (!e) e = launch_m(bs, 0);
+            }
             if (e) break;
             cudaGraph_t rbody = nullptr;
             e = add_cond(bs, rep, cudaGraphCondTypeIf, &rbody);
@@ -1464,12 +1467,11 @@ struct MgSolve {
             if (e) break;
             cap_r = true;
             e = sp.launch_replace(rs);  // flush, r = b - A x (FP64) stored as r
+            if (!e) e = launch_m(rs, 0);
             if (e) break;
             cudaGraph_t tmp = nullptr;
             e = cudaStreamEndCapture(rs, &tmp);
             cap_r = false;
-            if (e) break;
-            e = launch_m(bs, 0);
             if (e) break;
             e = cudaStreamEndCapture(bs, &tmp);
             cap_b = false;

@@ -25,7 +25,8 @@
 // matrix (values and columns 56, gathers and vectors 60), against the
 // matrix-free passes' 32.  As three kernels (p a pass of its own) an iteration
 // of 8000 rows took 21 us and of 1.1 million rows 38.0; two kernels 17.5 and
-// 37.8 (the matrix and the vectors stream from L2).
+// 37.8 (the matrix and the vectors stream from L2), several iterations a turn
+// of the loop 14.9 and 34.2.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -82,7 +83,7 @@ constexpr int kSellBatch = 8;
 __global__ void __launch_bounds__(kSellThreads)
     sell_spmv_dot_kernel(const SellDev A, const float2 *__restrict__ zp, float *__restrict__ pn, float *__restrict__ q,
                          double *__restrict__ x, SolveState *st, double *partials) {
-    if (st->done) return;
+    if (st->done || st->replace) return;
     const float beta = (float)st->beta;
     const double alpha = st->alpha;
     const bool pending = st->pending != 0;
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(kSellThreads)
     sell_update_kernel(const SellDev A, const float *__restrict__ pn, const float *__restrict__ q,
                        float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
                        cudaGraphConditionalHandle cond, cudaGraphConditionalHandle cond_rep, int use_cond) {
-    if (st->done) return;
+    if (st->done || st->replace) return;
     constexpr int R = 4;
     const int it = st->it;
     const float af = (float)st->alpha;
@@ -446,7 +447,7 @@ int sell_capture(SellPlan &P, cudaGraph_t *out) {
         e = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e) break;
         cap_b = true;
-        P.body(bs);
+        for (int u = 0; u < kLoopUnroll; ++u) P.body(bs);
         cudaGraph_t rbody = nullptr;
         e = add_cond(bs, P.cond_rep, cudaGraphCondTypeIf, &rbody);
         if (e) break;
