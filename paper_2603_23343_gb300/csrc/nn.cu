@@ -725,6 +725,136 @@ __global__ void __launch_bounds__(kWgThreads)
     }
 }
 
+// Weight gradient of the network's ends, where one side has 16 channels and
+// the other NC = 1 or 2 (c9: 16 -> 1, c1: 2 -> 16): a contraction over voxels
+// with M = the 16 channels of the wide side and N = 27 NC columns, one per tap
+// and narrow channel.  On the CUDA cores it was bound by shared-memory reads
+// of both sides per product (500 us and 386 us at 128^3); its bytes take
+// 10 us, and N is too small to fill a tcgen05 tile, so warps use m16n8k16 on
+// 16 voxels of a row:
+//   A  ldmatrix.trans of the wide rows (32-byte voxels, 16-byte halves swapped
+//      every four voxels: no bank conflicts)
+//   B  the narrow side shifted by each column's tap, two voxels at a time from
+//      rows kept with 16 zero or neighbouring voxels on either side
+// A stage is kWgnRows rows of up to 128 voxels, the next one on its way by
+// cp.async; a stage's products gather in the tensor core's accumulators and are
+// then added in FP32 (its additions truncate: one accumulator for a CTA's whole
+// run was 5 to 14 % further from the FP64 sums at 128^3 than the CUDA-core
+// kernel), a CTA's warps in order.
+// out[m, (t, c)] = sum_u wide[u, m] narrow[u + SGN off(t), c].
+constexpr int kWgnRows = 8;
+struct WgnArgs {
+    int X, Y, Z, XB, nxb, nyb, stages, per_cta;
+    int wide_bytes, buf_bytes;
+    const __nv_bfloat16 *wide, *narrow;
+    float *partials;
+};
+template <int NC, int SGN>
+__global__ void __launch_bounds__(256) wgrad_narrow_kernel(const WgnArgs a) {
+    extern __shared__ __align__(16) unsigned char wgn_sm[];
+    constexpr int NJ = (27 * NC + 7) / 8, NR = kWgnRows + 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int XB = a.XB, RS = (XB + 32) * NC, cpr = XB / 16;  // narrow row stride (elements), chunks per row
+    const uint32_t sm = smem_u32(wgn_sm);
+    auto cp16 = [](uint32_t d, const void *src, int bytes) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+    };
+    auto issue = [&](int st, int b) {
+        const int x0 = st % a.nxb * XB, t = st / a.nxb, y0 = t % a.nyb * kWgnRows, z = t / a.nyb;
+        const int rows = min(kWgnRows, a.Y - y0);
+        const uint32_t w = sm + b * a.buf_bytes, n = w + a.wide_bytes;
+        for (int e = tid; e < rows * XB * 2; e += 256) {
+            const int r = e / (XB * 2), q = e - r * (XB * 2), v = q >> 1;
+            cp16(w + (r * XB + v) * 32 + (((q & 1) ^ ((v >> 2) & 1)) << 4),
+                 a.wide + (((int64_t)z * a.Y + y0 + r) * a.X + x0) * 16 + q * 8, 16);
+        }
+        const int np = RS / 8;
+        for (int e = tid; e < 3 * NR * np; e += 256) {
+            const int r = e / np, q = e - r * np, zz = z + r / NR - 1, yy = y0 + r % NR - 1;
+            const int xx = x0 - 16 + q * 8 / NC;
+            const bool in = zz >= 0 && zz < a.Z && yy >= 0 && yy < a.Y && xx >= 0 && xx < a.X;
+            cp16(n + e * 16, in ? a.narrow + (((int64_t)zz * a.Y + yy) * a.X + xx) * NC : a.narrow, in ? 16 : 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // the columns' offsets in the narrow rows
+    int off[NJ];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int n = min(j * 8 + (lane >> 2), 27 * NC - 1), t = n / NC;
+        const int dz = t / 9 - 1, dy = t / 3 % 3 - 1, dx = t % 3 - 1;
+        off[j] = ((1 + SGN * dz) * NR + 1 + SGN * dy) * RS + (16 + SGN * dx + 2 * (lane & 3)) * NC + n % NC;
+    }
+    float sum[NJ][4];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[j][i] = 0.f;
+    const int s0 = blockIdx.x * a.per_cta, s1 = min(a.stages, s0 + a.per_cta);
+    if (s0 < s1) issue(s0, 0);
+    for (int st = s0; st < s1; ++st) {
+        const int b = (st - s0) & 1;
+        if (st + 1 < s1) {
+            issue(st + 1, b ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int rows = min(kWgnRows, a.Y - st / a.nxb % a.nyb * kWgnRows);
+        const uint32_t w = sm + b * a.buf_bytes;
+        const unsigned short *nr = reinterpret_cast<const unsigned short *>(wgn_sm + b * a.buf_bytes + a.wide_bytes);
+        float acc[NJ][4];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
+        for (int c = warp; c < rows * cpr; c += 8) {
+            const int yl = c / cpr, xc = (c - yl * cpr) * 16;
+            uint32_t A[4];
+            {
+                const int v = xc + (lane & 7) + (lane >> 4) * 8, h = (lane >> 3) & 1;
+                const uint32_t p = w + (yl * XB + v) * 32 + ((h ^ ((v >> 2) & 1)) << 4);
+                asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                             : "=r"(A[0]), "=r"(A[1]), "=r"(A[2]), "=r"(A[3])
+                             : "r"(p));
+            }
+            const unsigned short *q = nr + yl * RS + xc * NC;
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const unsigned short *o = q + off[j];
+                const uint32_t b0 = o[0] | (uint32_t)o[NC] << 16, b1 = o[8 * NC] | (uint32_t)o[9 * NC] << 16;
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+                             "{%8,%9}, {%0,%1,%2,%3};"
+                             : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
+                             : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(b0), "r"(b1));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[j][i] += acc[j][i];
+        __syncthreads();
+    }
+    // the warps' sums: red[warp][m][n]
+    float *red = reinterpret_cast<float *>(wgn_sm);
+    constexpr int N8 = NJ * 8;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            red[(warp * 16 + (lane >> 2) + (i >> 1) * 8) * N8 + j * 8 + 2 * (lane & 3) + (i & 1)] = sum[j][i];
+    __syncthreads();
+    float *dst = a.partials + (int64_t)blockIdx.x * (27 * 16 * NC);
+    for (int e = tid; e < 16 * 27 * NC; e += 256) {
+        const int m = e / (27 * NC), n = e - m * (27 * NC);
+        float t = 0.f;
+        for (int k = 0; k < 8; ++k) t += red[(k * 16 + m) * N8 + n];
+        // gw[o][t][i]: the wide side is the input (SGN < 0: one output channel) or the output
+        dst[SGN < 0 ? n * 16 + m : m * (27 * NC) + n] = t;
+    }
+}
+
 // out[e] = sum of the slots' partials[k][e], in a fixed order: eight threads per element, each over every
 // eighth slot, then their sums in turn (one thread per element left the GPU waiting on 80 blocks' serial
 // loads: 35 us for 152 slots of 20,736 elements).
@@ -936,6 +1066,47 @@ static int wgrad_tc(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x,
     return sum_slots((int64_t)27 * ci * co, p.S, partials, gw, s);
 }
 
+// The ends' weight gradient (wgrad_narrow_kernel): 16 -> 1 and 2 -> 16 channels, rows of whole chunks of
+// 16 voxels.  At 128^3 523 -> 43 us (16 -> 1) and 415 -> 55 us (2 -> 16), at
+// 32^3 41 -> 25 and 46 -> 24.
+inline bool wgrad_narrow_ok(int X, int ci, int co) {
+    return ((ci == 16 && co == 1) || (ci == 2 && co == 16)) && X % 16 == 0;
+}
+
+static int wgrad_narrow(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, const __nv_bfloat16 *gy, float *gw,
+                        float *partials, cudaStream_t s) {
+    const int NC = co == 1 ? 1 : 2;
+    WgnArgs a;
+    a.X = X;
+    a.Y = Y;
+    a.Z = Z;
+    a.XB = std::min(X, 128);
+    while (X % a.XB) a.XB -= 16;
+    a.nxb = X / a.XB;
+    a.nyb = (Y + kWgnRows - 1) / kWgnRows;
+    a.stages = a.nxb * a.nyb * Z;
+    a.wide_bytes = kWgnRows * a.XB * 32;
+    a.buf_bytes = a.wide_bytes + 3 * (kWgnRows + 2) * (a.XB + 32) * NC * 2;
+    a.wide = co == 1 ? x : gy;
+    a.narrow = co == 1 ? gy : x;
+    a.partials = partials;
+    // two CTAs per SM of a 152-SM part, and no more slots than the workspace was sized for
+    const int most = std::min(kWgTargetBlocks / 2, wgrad_plan(X, Y, Z, ci, co).S);
+    a.per_cta = (a.stages + most - 1) / most;
+    const int S = (a.stages + a.per_cta - 1) / a.per_cta;
+    const size_t smem = std::max<size_t>(2 * (size_t)a.buf_bytes, 8 * 16 * 56 * sizeof(float));
+    constexpr int kMaxSmem = 2 * (kWgnRows * 128 * 32 + 3 * (kWgnRows + 2) * 160 * 4);
+    if (co == 1) {
+        GB_CUDA(cudaFuncSetAttribute(wgrad_narrow_kernel<1, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+        wgrad_narrow_kernel<1, -1><<<S, 256, smem, s>>>(a);
+    } else {
+        GB_CUDA(cudaFuncSetAttribute(wgrad_narrow_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+        wgrad_narrow_kernel<2, 1><<<S, 256, smem, s>>>(a);
+    }
+    GB_CUDA(cudaGetLastError());
+    return sum_slots((int64_t)27 * ci * co, S, partials, gw, s);
+}
+
 template <int BO, int BI>
 static cudaError_t wgrad_launch(const WgradPlan &p, int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x,
                                 const __nv_bfloat16 *gy, float *partials, cudaStream_t s) {
@@ -950,6 +1121,7 @@ static int wgrad(int X, int Y, int Z, int ci, int co, const __nv_bfloat16 *x, co
     if (err && wgrad_zmarch_ok(X, Y, Z, ci, co)) return wgrad_zmarch(X, Y, Z, ci, co, x, gy, gw, partials, err, s);
     if (err && wgrad_tc_ok(X, Y, Z, ci, co)) return wgrad_tc(X, Y, Z, ci, co, x, gy, gw, partials, err, s);
     if (!wgrad_ok(X, ci, co)) return fail_arg("weight gradient: unsupported width or channel count");
+    if (wgrad_narrow_ok(X, ci, co)) return wgrad_narrow(X, Y, Z, ci, co, x, gy, gw, partials, s);
     WgradPlan p = wgrad_plan(X, Y, Z, ci, co);
     cudaError_t e;
     if (p.bo == 4 && p.bi == 4) e = wgrad_launch<4, 4>(p, X, Y, Z, ci, co, x, gy, partials, s);

@@ -125,7 +125,7 @@ constexpr double kHuge = 1e300;
 // iteration ends the solve or asks for a residual replacement, the rest of the
 // turn's kernels stand down and the replacement follows at its end.  A turn of
 // the WHILE node with its IF node costs about 5 us beside the kernels: one
-// iteration a turn took 66.1 ms for the Poisson solve at 256^3 (710
+// iteration a turn took 65.1 ms for the Poisson solve at 256^3 (678
 // iterations) and 37.8 us per SELL iteration of 1.1 million rows, four a turn
 // 62.0 ms and 34.2 us.
 constexpr int kLoopUnroll = 4;
