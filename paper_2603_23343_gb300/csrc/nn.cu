@@ -563,6 +563,135 @@ __global__ void __launch_bounds__(32 * kC1Rows, 2)
     }
 }
 
+// 1 or 2 -> 16 channels, rows of whole chunks of 16 voxels: warp-level bf16
+// matrix instructions with M = 16 voxels of a row, N = the 16 channels and
+// K = 27 CI padded to whole steps.  On the CUDA cores 27 CI fused multiply-adds
+// per output bound it (106 us for 2 -> 16, 168 for 1 -> 16 with a mask at
+// 128^3) where the bytes take 10 to 20 us; N = 16 is far below a tcgen05 tile.
+// A block holds kCnRows rows of up to 128 voxels with their neighbours (16
+// voxels on either side) in shared memory; the weights stay in registers, their
+// columns ordered so that a lane ends with four neighbouring channels and
+// writes them as one vector.  K's padding reads a row of zeros.  The steps' sums
+// are added in FP32 (the accumulator's own additions truncate: 30 % more rms
+// error than the CUDA-core sums over the whole of K; steps of 16 for CI = 2 and
+// 8 for CI = 1 are below them).  128^3, FP32 output: 221 -> 44 us (2 -> 16) and
+// 186 -> 42 us (1 -> 16).
+constexpr int kCnRows = 8;
+template <int CI, typename TO>
+__global__ void __launch_bounds__(256)
+    conv3_narrow_kernel(int X, int Y, int Z, int XB, const __nv_bfloat16 *__restrict__ in,
+                        const __nv_bfloat16 *__restrict__ w, TO *__restrict__ out, int relu,
+                        const __nv_bfloat16 *__restrict__ mask, int mstride, int moff, const double *scale,
+                        const float *__restrict__ vscale) {
+    extern __shared__ __align__(16) unsigned char cn_sm[];
+    constexpr int KS = (27 * CI + 15) / 16, NR = kCnRows + 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nxb = X / XB, nyb = (Y + kCnRows - 1) / kCnRows;
+    const int x0 = (int)blockIdx.x % nxb * XB, t0 = (int)blockIdx.x / nxb, y0 = t0 % nyb * kCnRows, z = t0 / nyb;
+    const int RS = (XB + 32) * CI, np = RS / 8;
+    const uint32_t sm = smem_u32(cn_sm);
+    for (int e = tid; e < (3 * NR + 1) * np; e += 256) {  // the last row: zeros
+        const int r = e / np, q = e - r * np, zz = z + r / NR - 1, yy = y0 + r % NR - 1, xx = x0 - 16 + q * 8 / CI;
+        const bool ok = r < 3 * NR && zz >= 0 && zz < Z && yy >= 0 && yy < Y && xx >= 0 && xx < X;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm + e * 16),
+                     "l"(ok ? in + (((int64_t)zz * Y + yy) * X + xx) * CI : in), "r"(ok ? 16 : 0)
+                     : "memory");
+    }
+    // B: k = t CI + i; column n of tile j is channel 4 (n / 2) + 2 j + (n & 1)
+    const unsigned short *wu = reinterpret_cast<const unsigned short *>(w);
+    uint32_t B[KS][2][2];
+    int off[KS][2][2 / CI];  // the taps' places in the rows: halves of a K step, then taps of a pair (CI = 1)
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = ks * 16 + h * 8 + 2 * (lane & 3), n = lane >> 2;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int o = 4 * (n >> 1) + 2 * j + (n & 1);
+                const uint32_t lo = k < 27 * CI ? wu[o * 27 * CI + k] : 0u,
+                               hi = k + 1 < 27 * CI ? wu[o * 27 * CI + k + 1] : 0u;
+                B[ks][j][h] = lo | hi << 16;
+            }
+#pragma unroll
+            for (int p = 0; p < 2 / CI; ++p) {
+                const int t = (k + p) / CI;
+                off[ks][h][p] = t < 27 ? (t / 9 * NR + t / 3 % 3) * RS + (15 + t % 3) * CI : -1;
+            }
+        }
+    const float sc = scale ? (float)*scale : 1.0f;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const unsigned short *su = reinterpret_cast<const unsigned short *>(cn_sm);
+    const int rows = min(kCnRows, Y - y0), cpr = XB / 16;
+    for (int c = warp; c < rows * cpr; c += 8) {
+        const int yl = c / cpr, xc = (c - yl * cpr) * 16, m = lane >> 2;
+        float acc[2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            uint32_t A[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int x = (xc + m + (q & 1) * 8) * CI, h = q >> 1;
+                auto at = [&](int o) { return su + (o < 0 ? 3 * NR * RS : o + yl * RS) + x; };
+                if constexpr (CI == 2)
+                    A[q] = *reinterpret_cast<const uint32_t *>(at(off[ks][h][0]));
+                else
+                    A[q] = *at(off[ks][h][0]) | (uint32_t)*at(off[ks][h][2 / CI - 1]) << 16;
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float d[4];
+                if constexpr (CI == 2) {
+                    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+                                 "{%8,%9}, {%10,%10,%10,%10};"
+                                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                                 : "r"(A[0]), "r"(A[1]), "r"(A[2]), "r"(A[3]), "r"(B[ks][j][0]), "r"(B[ks][j][1]),
+                                   "f"(0.f));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
+                                     "{%7,%7,%7,%7};"
+                                     : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                                     : "r"(A[2 * h]), "r"(A[2 * h + 1]), "r"(B[ks][j][h]), "f"(0.f));
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int64_t v = ((int64_t)z * Y + y0 + yl) * X + x0 + xc + m + r * 8;
+            const int o = 4 * (lane & 3);
+            const float vs = vscale ? sc * vscale[v] : sc;
+            float f[4] = {acc[0][2 * r] * vs, acc[0][2 * r + 1] * vs, acc[1][2 * r] * vs, acc[1][2 * r + 1] * vs};
+            if (relu)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) f[i] = f[i] < 0.0f ? 0.0f : f[i];  // NaN passes
+            if (mask) {
+                const uint2 mk = __ldg(reinterpret_cast<const uint2 *>(mask + v * mstride + moff + o));
+                const __nv_bfloat162 m0 = *reinterpret_cast<const __nv_bfloat162 *>(&mk.x),
+                                     m1 = *reinterpret_cast<const __nv_bfloat162 *>(&mk.y);
+                if (!(__bfloat162float(m0.x) > 0.0f)) f[0] = 0.0f;
+                if (!(__bfloat162float(m0.y) > 0.0f)) f[1] = 0.0f;
+                if (!(__bfloat162float(m1.x) > 0.0f)) f[2] = 0.0f;
+                if (!(__bfloat162float(m1.y) > 0.0f)) f[3] = 0.0f;
+            }
+            TO *po = out + v * 16 + o;
+            if constexpr (sizeof(TO) == 4) {
+                *reinterpret_cast<float4 *>(po) = make_float4(f[0], f[1], f[2], f[3]);
+            } else {
+                __nv_bfloat162 a = __floats2bfloat162_rn(f[0], f[1]), b = __floats2bfloat162_rn(f[2], f[3]);
+                *reinterpret_cast<uint2 *>(po) =
+                    make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b));
+            }
+        }
+    }
+}
+
 template <int CI, int CO, typename TO>
 static int conv_simt_launch(int X, int Y, int Z, const __nv_bfloat16 *in, const __nv_bfloat16 *w, TO *out, int relu,
                             const __nv_bfloat16 *mask, int mstride, int moff, const double *scale,
@@ -581,6 +710,21 @@ static int conv_simt_launch(int X, int Y, int Z, const __nv_bfloat16 *in, const 
             fn<<<grid, 32 * kC1Rows, 0, s>>>(X, Y, Z, in, w, out, relu, mask, mstride, moff, scale, vscale, chunk);
             cudaError_t e = cudaGetLastError();
             return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "conv3_c1_march launch");
+        }
+    }
+    if constexpr (CO == 16 && CI <= 2) {
+        const bool vec = !mask || (mstride % 4 == 0 && moff % 4 == 0);
+        int XB = std::min(X, 128);
+        if (X % 16 == 0 && vec) {
+            while (X % XB) XB -= 16;
+            const int64_t blocks = (int64_t)(X / XB) * ((Y + kCnRows - 1) / kCnRows) * Z;
+            if (blocks <= INT32_MAX) {
+                const size_t smem = (size_t)(3 * (kCnRows + 2) + 1) * (XB + 32) * CI * 2;
+                conv3_narrow_kernel<CI, TO><<<(unsigned)blocks, 256, smem, s>>>(X, Y, Z, XB, in, w, out, relu, mask,
+                                                                                mstride, moff, scale, vscale);
+                cudaError_t e = cudaGetLastError();
+                return e == cudaSuccess ? GBPCG_OK : fail_cuda(e, "conv3_narrow launch");
+            }
         }
     }
     if (CI % 8 == 0 && X % 128 == 0) {
