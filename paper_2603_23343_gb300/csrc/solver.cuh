@@ -124,12 +124,13 @@ constexpr double kHuge = 1e300;
 // Iterations per turn of a device-driven loop (the WHILE node's body): once an
 // iteration ends the solve or asks for a residual replacement, the rest of the
 // turn's kernels stand down and the replacement follows at its end.  A turn of
-// the WHILE node with its IF node costs about 5 us beside the kernels: one
-// iteration a turn took 65.1 ms for the Poisson solve at 256^3 (678
-// iterations) and 37.8 us per SELL iteration of 1.1 million rows, four a turn
-// 62.0 ms and 34.2 us.
-constexpr int kLoopUnroll = 4;
-
+// the WHILE node with its IF node costs about 5 us beside the kernels.  One,
+// four, eight and twelve iterations a turn: the Poisson solve at 256^3 (about
+// 660 iterations) 65.1, 61.7, 61.4, 61.3 ms, block coefficients at 128^3 (426)
+// four to twelve 13.3, 12.9, 12.9 ms, a SELL iteration of 1.1 million rows
+// 37.8, 34.3, 33.8, 33.6 us, of 8000 rows (63 iterations, three replacements)
+// 17.5, 14.9, 14.9, 15.2 us.
+constexpr int kLoopUnroll = 8;
 
 // Compensated FP32 sum (Kahan): the running error of each addition is fed
 // back into the next, so the sum of a thread's terms is good to a few FP32
