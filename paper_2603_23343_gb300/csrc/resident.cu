@@ -43,7 +43,10 @@ namespace {
 
 constexpr int kMaxWarps = kResThreads / 32;
 constexpr int kSlotsPerLane = (kResMaxCtas + 31) / 32;
-constexpr uint32_t kSumPolls = 1u << 20;  // a poll is an L2 round trip, about 0.7 us: under a second
+// A poll is an L2 round trip, about 0.7 us: under a second for the waits between CTAs that are in the
+// same problem, which are never apart by more than part of an iteration.
+constexpr uint32_t kSumPolls = 1u << 20;
+constexpr int kProgressEvery = 32;  // iterations of a batch's problem between two steps of its progress word
 
 __device__ __forceinline__ void st_slot(ulonglong2 *p, unsigned long long v, unsigned long long tag) {
     asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
@@ -498,7 +501,8 @@ __device__ __noinline__ void res_finish(Shared &sh, int half, double v) {
 //   QREG  so does q = A p between the two halves of an iteration; else A p is taken twice
 //   DREG  so many planes of d do too, updated with p one iteration late; the others: add_d
 //   X     type of b and x
-template <int NT, int MAXD, bool QREG, int DREG, typename X>
+//   BATCH the launch holds other problems: their waits count from the last step of P.progress (batch_meet)
+template <int NT, int MAXD, bool QREG, int DREG, bool BATCH, typename X>
 __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsigned char *smem, Shared &sh) {
     const int tid = threadIdx.x, lane = tid & 31;
     const int bx4 = P.bx4, by = P.by, D = P.depth;
@@ -832,6 +836,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
                         res_finish(sh, half, pair_value(t));
                         sh.rr = half ? t : sh.rr;
                     }
+                    if (BATCH && half == 1 && rank == 0 && S.it % kProgressEvery == 0) atomicAdd(P.progress, 1u);
                 }
             } else if (half == 1) {
                 // Meanwhile the other warps take d += alpha p and fetch the neighbours' faces: each CTA
@@ -945,7 +950,7 @@ template <int NT, int MAXD, bool QREG, int DREG, typename X>
 __global__ void __launch_bounds__(NT, 1) resident_kernel(const __grid_constant__ ResProb one) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
-    resident_solve<NT, MAXD, QREG, DREG, X>(one, (int)blockIdx.x, smem, sh);
+    resident_solve<NT, MAXD, QREG, DREG, false, X>(one, (int)blockIdx.x, smem, sh);
 }
 
 // Many problems: CTA c works through list[first[c]] .. list[first[c + 1] - 1], each entry a problem
@@ -955,6 +960,31 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const __grid_constant__
 struct ResSchedule {
     uint32_t first[2 * kResMaxCtas + 1];
 };
+
+// Waits until every CTA of problem P has come to it; false if one never does.  A CTA that is early waits
+// here for as long as its partners' earlier problems take, so the limit is on the polls since any problem
+// of the launch last took kProgressEvery iterations (or began): two loads each, one to two seconds.
+__device__ __forceinline__ bool batch_meet(const ResProb &P, int rank, Shared &sh) {
+    if (threadIdx.x == 0) {
+        sh.timeout = 0;
+        if (P.G > 1) {
+            atomicAdd(P.arrived, 1u);
+            unsigned seen = ld_flag(P.progress);
+            for (uint32_t polls = 0; ld_flag(P.arrived) < (unsigned)P.G;) {
+                const unsigned now = ld_flag(P.progress);
+                polls = now == seen ? polls + 1 : 0;
+                seen = now;
+                if (polls > kSumPolls) {
+                    sh.timeout = 1;
+                    break;
+                }
+            }
+        }
+        if (rank == 0 && !sh.timeout) atomicAdd(P.progress, 1u);
+    }
+    __syncthreads();
+    return sh.timeout == 0;
+}
 
 template <int NT, int MAXD, bool QREG, int DREG, typename X>
 __global__ void __launch_bounds__(NT, 2)
@@ -967,8 +997,10 @@ __global__ void __launch_bounds__(NT, 2)
         const int *src = reinterpret_cast<const int *>(probs + (a & 0xffffu));
         for (int i = threadIdx.x; i < (int)(sizeof(ResProb) / 4); i += NT) reinterpret_cast<int *>(&P)[i] = src[i];
         __syncthreads();
-        resident_solve<NT, MAXD, QREG, DREG, X>(P, (int)(a >> 16), smem, sh);
-        if (sh.timeout) break;  // the problems left over keep done = 0
+        // after a wait that ran out the problems left over keep done = 0
+        if (!batch_meet(P, (int)(a >> 16), sh)) break;
+        resident_solve<NT, MAXD, QREG, DREG, true, X>(P, (int)(a >> 16), smem, sh);
+        if (sh.timeout) break;
         __syncthreads();
     }
 }
@@ -1102,6 +1134,7 @@ ResProb make_prob(const SolveCall &c, const ResPlan &p) {
     r.st = reinterpret_cast<SolveState *>(c.ws + c.L.state);
     r.slots = reinterpret_cast<ulonglong2 *>(c.ws + c.L.partials);
     r.flags = reinterpret_cast<unsigned *>(r.slots + 2 * kResMaxCtas * kResSlotVals);
+    r.arrived = r.flags + kResMaxCtas * kResFlagStride;
     if (p.G > kResInboxAbove && inbox_bytes(p.G) <= padded * 4) r.inbox = reinterpret_cast<ulonglong2 *>(r.pg);
     return r;
 }
@@ -1322,17 +1355,19 @@ int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, cha
     }
     std::vector<ResProb> probs(n);
     size_t smem = 0;
-    char *dprobs = tables, *dlist = dprobs + (size_t)n * sizeof(ResProb);
-    if ((size_t)n * sizeof(ResProb) + best_list.size() * sizeof(uint32_t) > table_bytes) return kResNoRoom;
+    char *progress = tables, *dprobs = progress + 256, *dlist = dprobs + (size_t)n * sizeof(ResProb);
+    if (256 + (size_t)n * sizeof(ResProb) + best_list.size() * sizeof(uint32_t) > table_bytes) return kResNoRoom;
     for (int i = 0; i < n; ++i) {
         const ResPlan &p = options[i][best_pick[i]].p;
         probs[i] = make_prob(calls[i], p);
         probs[i].st = states + i;
+        probs[i].progress = reinterpret_cast<unsigned *>(progress);
         smem = std::max(smem, p.smem);
         GB_CUDA(cudaMemsetAsync(probs[i].slots, 0, kResSlotBytes, s));
         if (probs[i].inbox) GB_CUDA(cudaMemsetAsync(probs[i].inbox, 0, inbox_bytes(p.G), s));
     }
     GB_CUDA(cudaMemsetAsync(states, 0, (size_t)n * sizeof(SolveState), s));
+    GB_CUDA(cudaMemsetAsync(progress, 0, 256, s));
     // copies from pageable memory have left it when the calls return
     GB_CUDA(cudaMemcpyAsync(dprobs, probs.data(), (size_t)n * sizeof(ResProb), cudaMemcpyHostToDevice, s));
     GB_CUDA(cudaMemcpyAsync(dlist, best_list.data(), best_list.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s));

@@ -11,8 +11,9 @@ constexpr int kResThreads = 512;
 constexpr int kResMaxCtas = 160;  // bricks of one problem (GB300 has 152 SMs)
 constexpr int kResSlotVals = 4;   // 16-byte slots per CTA and grid sum
 constexpr int kResFlagStride = 8;  // words between two CTAs' face flags
-// two buffers of slots, then the flags
-constexpr size_t kResSlotBytes = (size_t)2 * kResMaxCtas * kResSlotVals * 16 + (size_t)kResMaxCtas * kResFlagStride * 4;
+// two buffers of slots, then the flags, then a batch's count of CTAs that have come to the problem
+constexpr size_t kResSlotBytes =
+    (size_t)2 * kResMaxCtas * kResSlotVals * 16 + (size_t)kResMaxCtas * kResFlagStride * 4 + 32;
 
 // How a grid is cut: sx x sy x sz bricks of 4 bx4 x by x bz points, each
 // thread of a CTA holding one four-point vector in x over `depth` planes
@@ -62,6 +63,7 @@ struct ResProb {
     SolveState *st;
     ulonglong2 *slots;
     unsigned *flags;      // per CTA: number of the sum its face values belong to
+    unsigned *arrived, *progress;  // batches: CTAs that have come to this problem; steps of any problem
     ulonglong2 *inbox;    // NULL, or every CTA's own slots of the loop's sums (grid_sum_pair)
 };
 

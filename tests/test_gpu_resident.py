@@ -109,3 +109,25 @@ def test_mixed_batch_on_chip_and_streamed(gpu_lib, io):
         assert r["status"] == r1["status"] == gpu_lib.OK and abs(r["iters"] - r1["iters"]) <= 2
         assert oracle.true_relres(b.cpu().double().numpy(), x.cpu().double().numpy()) <= tol
         assert float((x - x1).double().norm()) <= 50 * tol * float(x1.double().norm())
+
+
+def test_batch_waits_for_longer_problems(gpu_lib):
+    """Problems that end at once beside problems that iterate for seconds: a problem whose CTAs come from
+    both kinds waits for as long as the longer ones take (the limit of its wait counts from the last step
+    any problem made).  Twenty flat grids, every second right-hand side zero, fill the chip; the cubes
+    after them are larger and expected to take half the time, so each shares its CTAs with several."""
+    flat, cube = (20, 30, 201), (59, 60, 61)
+    shapes = [flat] * 20 + [cube] * 6
+    zero = [i % 2 == 1 for i in range(20)] + [True] * 6
+    bs = [torch.from_numpy(inputs.uniform_rhs(s, 320 + i, dtype=np.float64)).cuda() for i, s in enumerate(shapes)]
+    for b, z in zip(bs, zero):
+        if z:
+            b.zero_()
+    maxit = 400000
+    xs, res = gpu_lib.pcg_solve_batched(bs, tol=1e-30, maxit=maxit)
+    for x, r, z in zip(xs, res, zero):
+        if z:
+            assert r["status"] == gpu_lib.OK and r["iters"] == 0 and not torch.any(x), r
+        else:
+            assert r["status"] == gpu_lib.NOT_CONVERGED and r["iters"] == maxit, r
+    assert res[0]["time_ms"] > 2000.0  # long enough for the limit to matter
