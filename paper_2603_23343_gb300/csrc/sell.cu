@@ -78,21 +78,13 @@ __global__ void __launch_bounds__(kSellThreads)
 // the first gather, so a row costs two memory latencies and not two per entry.
 constexpr int kSellBatch = 8;
 
-// Whether a loop kernel has nothing to do.  A finished solve also ends the loop from here, so that the
-// WHILE node's condition never depends on which kernel's last step finished it.
-__device__ __forceinline__ bool sell_stand_down(const SolveState *st, cudaGraphConditionalHandle cond, int use_cond) {
-    if (st->done && use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
-    return st->done || st->replace;
-}
-
 // q = A p with p = z + beta p_{k-1} (pn), the partial p.q, and the pending
 // x += alpha_{k-1} p_{k-1}; last CTA: alpha, or a breakdown (p.q <= 0: A is
-// not positive definite), which ends the loop.
+// not positive definite), on which the update kernel ends the loop.
 __global__ void __launch_bounds__(kSellThreads)
     sell_spmv_dot_kernel(const SellDev A, const float2 *__restrict__ zp, float *__restrict__ pn, float *__restrict__ q,
-                         double *__restrict__ x, SolveState *st, double *partials, cudaGraphConditionalHandle cond,
-                         cudaGraphConditionalHandle cond_rep, int use_cond) {
-    if (sell_stand_down(st, cond, use_cond)) return;
+                         double *__restrict__ x, SolveState *st, double *partials) {
+    if (st->done || st->replace) return;
     const float beta = (float)st->beta;
     const double alpha = st->alpha;
     const bool pending = st->pending != 0;
@@ -128,22 +120,24 @@ __global__ void __launch_bounds__(kSellThreads)
     }
     double part[1], tot[1];
     block_sum<1, kSellThreads>(acc, part);
-    if (!grid_sum_last<1, kSellThreads>(part, partials, &st->ticket[K_PASSA], tot) || threadIdx.x != 0) return;
-    passa_finish(st, tot[0], false);
-    if (use_cond) {
-        cudaGraphSetConditional(cond, st->done ? 0u : 1u);
-        cudaGraphSetConditional(cond_rep, st->replace ? 1u : 0u);
-    }
+    if (grid_sum_last<1, kSellThreads>(part, partials, &st->ticket[K_PASSA], tot) && threadIdx.x == 0)
+        passa_finish(st, tot[0], false);
 }
 
 // r -= alpha q, z = D^-1 r, the pairs (z, p); partials r.r, r.z; last CTA:
 // beta, the convergence test and the replacement trigger.  Four rows a thread
-// in flight.
+// in flight.  Where it has nothing to do because the solve has ended (in the
+// product before it, say) it ends the loop: a solve that is done never leaves
+// the WHILE node's condition set.  (The product setting the condition itself
+// cost 1 us per iteration of 8000 rows and 9 us at 256^3.)
 __global__ void __launch_bounds__(kSellThreads)
     sell_update_kernel(const SellDev A, const float *__restrict__ pn, const float *__restrict__ q,
                        float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
                        cudaGraphConditionalHandle cond, cudaGraphConditionalHandle cond_rep, int use_cond) {
-    if (sell_stand_down(st, cond, use_cond)) return;
+    if (st->done || st->replace) {
+        if (st->done && use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
+        return;
+    }
     constexpr int R = 4;
     const int it = st->it;
     const float af = (float)st->alpha;
@@ -400,7 +394,7 @@ struct SellPlan {
         sell_zero_x_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, st);
     }
     void body(cudaStream_t s) {
-        sell_spmv_dot_kernel<<<grid, kSellThreads, 0, s>>>(A, zp, p, q, x, st, partials, cond, cond_rep, use_cond);
+        sell_spmv_dot_kernel<<<grid, kSellThreads, 0, s>>>(A, zp, p, q, x, st, partials);
         sell_update_kernel<<<grid, kSellThreads, 0, s>>>(A, p, q, r, zp, st, partials, cond, cond_rep, use_cond);
     }
     void replace(cudaStream_t s) {
