@@ -587,11 +587,12 @@ static int persistent_batch(int nprob, const gbpcg_grid *grids, const void *cons
 // The problems of a batch that fit the chip, solved there (resident.cu): one launch for all that leave
 // room for others beside them (bitwise the same from run to run), and one launch each for the larger
 // ones and, with GBPCG_FLAG_BATCH_GRAPH, for all (bitwise the standalone solves).  `in_batch` and
-// `alone` hold their numbers; fills their results.
+// `alone` hold their numbers; fills their results.  kResNoRoom, and nothing solved, if the shared launch
+// is not to be had; `refused` gets the problems whose own launch is not.
 static int resident_batch(const std::vector<int> &in_batch, const std::vector<int> &alone, const gbpcg_grid *grids,
                           const void *const *b, void *const *x, const gbpcg_opts *opts, gbpcg_result *results, char *ws,
                           size_t region, const std::vector<WsLayout> &L, const std::vector<size_t> &off,
-                          cudaStream_t s) {
+                          cudaStream_t s, std::vector<int> *refused) {
     const int nb = (int)in_batch.size(), n = nb + (int)alone.size();
     auto which = [&](int i) { return i < nb ? in_batch[i] : alone[i - nb]; };
     std::vector<SolveCall> calls(n);
@@ -613,10 +614,16 @@ static int resident_batch(const std::vector<int> &in_batch, const std::vector<in
                                            opts->io_dtype, s))
             return rc;
     }
+    std::vector<char> ran(n, 1);
     for (int i = nb; i < n; ++i) {
         ResPlan plan;
         resident_fits(*calls[i].g, &plan);
-        if (int rc = resident_launch(calls[i], plan, s, states + i)) return rc;
+        const int rc = resident_launch(calls[i], plan, s, states + i);
+        if (rc && rc != kResNoRoom) return rc;
+        if (rc) {
+            ran[i] = 0;
+            refused->push_back(which(i));
+        }
     }
     GB_CUDA(cudaEventRecord(e1, s));
     std::vector<SolveState> hs(n);
@@ -627,13 +634,14 @@ static int resident_batch(const std::vector<int> &in_batch, const std::vector<in
     for (int i = 0; i < n; ++i) {
         gbpcg_result &r = results[which(i)];
         memset(&r, 0, sizeof(r));
+        if (!ran[i]) continue;
         r.iters = hs[i].it;
         r.status = hs[i].done ? hs[i].status : GBPCG_TIMEOUT;
         r.rel_res_recursive = hs[i].bb > 0 ? sqrt(hs[i].rr / hs[i].bb) : 0.0;
         r.rel_res_true = hs[i].bb_true > 0 ? sqrt(hs[i].rr_true / hs[i].bb_true) : 0.0;
         r.time_ms = ms;
         r.replacements = hs[i].n_replace;
-        r.pass_launches[0] = (nb ? 1 : 0) + (n - nb);
+        r.pass_launches[0] = (nb ? 1 : 0) + (n - nb - (int)refused->size());
         r.pass_launches[1] = 2 * (hs[i].it + hs[i].n_replace);
         if (r.status == GBPCG_TIMEOUT) set_error("a bounded device wait timed out during a batched solve");
     }
@@ -653,11 +661,12 @@ static int check_batch(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts 
 }
 
 // The problems in the streaming kernels: one persistent kernel where it takes them (batch.cu), else
-// (block coefficients, unaligned rows, GBPCG_FLAG_BATCH_GRAPH) one CUDA graph with a branch per problem.
+// (block coefficients, unaligned rows, GBPCG_FLAG_BATCH_GRAPH, or not `persistent`) one CUDA graph with a
+// branch per problem.
 static int streamed_batch(int nprob, const gbpcg_grid *grids, const void *const *b, void *const *x,
                           const gbpcg_opts *opts, gbpcg_result *results, char *ws, const std::vector<WsLayout> &L,
-                          const std::vector<size_t> &off, cudaStream_t s) {
-    if (!(opts->flags & GBPCG_FLAG_BATCH_GRAPH) && batch_persistent_ok(nprob, grids))
+                          const std::vector<size_t> &off, cudaStream_t s, bool persistent = true) {
+    if (persistent && !(opts->flags & GBPCG_FLAG_BATCH_GRAPH) && batch_persistent_ok(nprob, grids))
         return persistent_batch(nprob, grids, b, x, opts, results, ws, L, off, s);
 
     // tile configurations: explicit, autotuned (cached per shape), or the defaults
@@ -844,11 +853,12 @@ int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_
     ResPlan plan;
     const bool resident = !opts->tile_cfg && !(opts->flags & GBPCG_FLAG_PROFILE) && resident_fits(g, &plan);
     const bool host_loop = opts->flags & GBPCG_FLAG_HOST_LOOP;
-    const int rc = (opts->flags & GBPCG_FLAG_PROFILE) ? solve_profiled<float>(call, tma, result, s)
-                   : resident && host_loop            ? resident_host_loop(call, plan, s)
-                   : resident                         ? resident_launch(call, plan, s)
-                   : host_loop                        ? solve_host_loop<float>(call, tma, s)
-                                                      : solve_launch<float>(call, tma, s);
+    int rc = kResNoRoom;
+    if (resident) rc = host_loop ? resident_host_loop(call, plan, s) : resident_launch(call, plan, s);
+    if (rc == kResNoRoom)
+        rc = (opts->flags & GBPCG_FLAG_PROFILE) ? solve_profiled<float>(call, tma, result, s)
+             : host_loop                        ? solve_host_loop<float>(call, tma, s)
+                                                : solve_launch<float>(call, tma, s);
     if (rc) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
@@ -947,15 +957,21 @@ int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *
     } else if (!graph && !opts->tile_cfg) {
         choice = resident_choice(nprob, grids);
     }
-    const std::vector<int> &in_batch = choice.in_batch, &alone = choice.alone, &rest = choice.rest;
+    std::vector<int> &in_batch = choice.in_batch, &alone = choice.alone, &rest = choice.rest;
     if (!in_batch.empty() || !alone.empty()) {
-        int rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s);
-        if (rc == kResNoRoom) {  // (the tables outgrew the batch's region: one launch each)
-            std::vector<int> each = in_batch;
-            each.insert(each.end(), alone.begin(), alone.end());
-            rc = resident_batch({}, each, grids, b, x, opts, results, ws, region, L, off, s);
+        std::vector<int> refused;
+        int rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, &refused);
+        if (rc == kResNoRoom) {  // the tables outgrew the batch's region, or too few SMs: one launch each
+            alone.insert(alone.begin(), in_batch.begin(), in_batch.end());
+            in_batch.clear();
+            rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, &refused);
         }
         if (rc) return rc;
+        for (int i : refused) alone.erase(std::find(alone.begin(), alone.end(), i));
+        rest.insert(rest.end(), refused.begin(), refused.end());
+        const bool whole = refused.empty();  // else the persistent kernel would not be resident either
+        if (in_batch.empty() && alone.empty())
+            return streamed_batch(nprob, grids, b, x, opts, results, ws, L, off, s, whole);
         if (!rest.empty()) {
             const int m = (int)rest.size();
             std::vector<gbpcg_grid> g2(m);
@@ -971,7 +987,7 @@ int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *
                 L2[i] = L[rest[i]];
                 off2[i] = off[rest[i]];
             }
-            rc = streamed_batch(m, g2.data(), b2.data(), x2.data(), opts, r2.data(), ws, L2, off2, s);
+            rc = streamed_batch(m, g2.data(), b2.data(), x2.data(), opts, r2.data(), ws, L2, off2, s, whole);
             if (rc == GBPCG_ERR_ARG || rc == GBPCG_ERR_CUDA) return rc;
             for (int i = 0; i < m; ++i) results[rest[i]] = r2[i];
         }

@@ -1139,6 +1139,18 @@ ResProb make_prob(const SolveCall &c, const ResPlan &p) {
     return r;
 }
 
+// A cooperative launch, or kResNoRoom where this context may not use the SMs it asks for (a context
+// limited to part of the GPU): nothing has run then, and the caller streams the problem instead.
+int cooperative(const cudaLaunchConfig_t &lc, void *fn, void **kargs) {
+    const cudaError_t e = cudaLaunchKernelExC(&lc, fn, kargs);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return kResNoRoom;
+    }
+    GB_CUDA(e);
+    return GBPCG_OK;
+}
+
 int launch_one(const ResProb &r, const ResPlan &p, int io, cudaStream_t s) {
     void *fn = io == GBPCG_F64 ? resident_fn<double>(p.build) : resident_fn<float>(p.build);
     GB_CUDA(allow_smem(fn, kResMaxSmem));
@@ -1154,8 +1166,7 @@ int launch_one(const ResProb &r, const ResPlan &p, int io, cudaStream_t s) {
     attr[0].val.cooperative = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    GB_CUDA(cudaLaunchKernelExC(&lc, fn, kargs));
-    return GBPCG_OK;
+    return cooperative(lc, fn, kargs);
 }
 
 // Plan of a shape, from the kept ones if it is there; false if it does not fit.
@@ -1390,8 +1401,7 @@ int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, cha
     attr[0].val.cooperative = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    GB_CUDA(cudaLaunchKernelExC(&lc, fn, kargs));
-    return GBPCG_OK;
+    return cooperative(lc, fn, kargs);
 }
 
 }  // namespace gb

@@ -29,10 +29,15 @@ struct ResPlan {
 // Whether one solve of this grid runs on chip (constant coefficients), and its plan.
 bool resident_fits(const gbpcg_grid &g, ResPlan *plan);
 
+// Instead of a status: nothing has been solved, and the problem is to be streamed (or launched alone).
+constexpr int kResNoRoom = -1;
+
 // The whole solve, enqueued on s; its scalars go to *st (DEVICE), or to the workspace's state block.
+// kResNoRoom where the context may not use the SMs of the plan.
 int resident_launch(const SolveCall &c, const ResPlan &plan, cudaStream_t s, SolveState *st = nullptr);
 
-// The same solve driven from the host, which reads the device's stop flag after every iteration.
+// The same solve driven from the host, which reads the device's stop flag after every iteration (kResNoRoom
+// as above).
 int resident_host_loop(const SolveCall &c, const ResPlan &plan, cudaStream_t s);
 
 // Which problems of a batch run here, all in one launch or one by one, and which in the streaming
@@ -43,8 +48,7 @@ struct ResidentChoice {
 ResidentChoice resident_choice(int n, const gbpcg_grid *grids);
 
 // One launch of calls[0 .. n) (ResidentChoice::in_batch) on s.  states: DEVICE, one per problem; tables:
-// DEVICE scratch (kResNoRoom, and nothing enqueued, if it is too small).
-constexpr int kResNoRoom = -1;
+// DEVICE scratch (kResNoRoom if it is too small, or the context may not use every SM).
 int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes, int io,
                           cudaStream_t s);
 
