@@ -411,8 +411,8 @@ int gbpcg_autotune_record(const gbpcg_grid *grid, const gbpcg_opts *opts, int32_
 int gbpcg_mg_workspace_size(const gbpcg_grid *grid, size_t *bytes);
 
 /* z = M r, one V-cycle (the hierarchy is built in the call): r, z DEVICE
- * FP32 (nz, ny, nx), distinct; *levels (may be NULL) receives the number of
- * levels.  Workspace: DEVICE, gbpcg_mg_workspace_size bytes, 256-byte
+ * FP32 (nz, ny, nx), distinct, of any alignment (16 bytes saves a copy of
+ * each); *levels (may be NULL) receives the number of levels.  Workspace: DEVICE, gbpcg_mg_workspace_size bytes, 256-byte
  * aligned. */
 int gbpcg_mg_vcycle(const gbpcg_grid *grid, const float *r, float *z, void *workspace, size_t workspace_bytes,
                     int32_t *levels, gbpcg_stream stream);

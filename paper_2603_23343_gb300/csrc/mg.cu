@@ -1583,9 +1583,18 @@ int gbpcg_mg_vcycle(const gbpcg_grid *grid, const float *r, float *z, void *work
     const MgLayout M = mg_layout(*grid, GBPCG_F64);
     if (!workspace || workspace_bytes < M.total || (reinterpret_cast<uintptr_t>(workspace) & 255u))
         return fail_arg("workspace: gbpcg_mg_workspace_size() bytes, 256-byte aligned");
+    if ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(z)) & (sizeof(float) - 1))
+        return fail_arg("r and z must be aligned to their element size");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(workspace);
-    const MgArgs a = mg_args(*grid, ws, M, const_cast<float *>(r), z, nullptr);
+    MgArgs a = mg_args(*grid, ws, M, const_cast<float *>(r), z, nullptr);
+    // the level kernels take 16-byte vectors of r and z: others go through the solver's r and z in the workspace
+    const size_t bytes = (size_t)a.lv[0].m * sizeof(float);
+    if (mg_l0(a) > 0 && (reinterpret_cast<uintptr_t>(r) & 15u)) {
+        a.lv[0].f = reinterpret_cast<float *>(ws + M.r);
+        GB_CUDA(cudaMemcpyAsync(a.lv[0].f, r, bytes, cudaMemcpyDeviceToDevice, s));
+    }
+    if (mg_l0(a) > 0 && (reinterpret_cast<uintptr_t>(z) & 15u)) a.lv[0].w = reinterpret_cast<float *>(ws + M.base.z);
     if (grid->k_block) {  // the per-block face table the level-0 weights come from
         const int nbx = (grid->nx + grid->kbx - 1) / grid->kbx, nby = (grid->ny + grid->kby - 1) / grid->kby,
                   nbz = (grid->nz + grid->kbz - 1) / grid->kbz;
@@ -1595,6 +1604,7 @@ int gbpcg_mg_vcycle(const gbpcg_grid *grid, const float *r, float *z, void *work
     }
     GB_CUDA(mg_setup(a, s));
     GB_CUDA(mg_vcycle(a, s, nullptr));
+    if (a.lv[0].w != z) GB_CUDA(cudaMemcpyAsync(z, a.lv[0].w, bytes, cudaMemcpyDeviceToDevice, s));
     if (levels) *levels = a.L;
     return GBPCG_OK;
 }
