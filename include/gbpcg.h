@@ -370,7 +370,9 @@ int gbpcg_sell_workspace_size(const gbpcg_sell *matrix, size_t *bytes);
  * alpha p in FP64; r -= alpha q, z = D^-1 r with r.r and r.z), the scalars on
  * the device, the loop one CUDA graph.  The residual is replaced by b - A x computed in FP64 when it has
  * dropped two decades since the last replacement and when it meets the
- * tolerance, so convergence is decided on a true residual.  Fills *result
+ * tolerance, so convergence is decided on a true residual.  b and x are scaled
+ * by a power of two inside the solve as in gbpcg_pcg_solve, so any scale of b
+ * converges alike.  Fills *result
  * (rel_res_true: FP64 ||b - A x|| / ||b||); synchronises `stream`.
  */
 int gbpcg_sell_pcg_solve(const gbpcg_sell *matrix, const double *b, double *x, const gbpcg_opts *opts,

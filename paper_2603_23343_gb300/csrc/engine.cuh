@@ -66,6 +66,7 @@ struct __align__(16) SolveState {
     int true_known; // 1: rr_true, bb_true already hold b - A x of the final x
     unsigned long long rhs_bits;  // max |b| as the bit pattern of a non-negative double
     double rzm;     // r.M r of the last residual (preconditioners other than Jacobi)
+    double scale;   // rhs_scale (Sliced-ELL solves)
     unsigned int ticket[8];
 };
 

@@ -21,7 +21,10 @@
 // plus an FP64 residual b - A x (gathering the FP64 x) at the start, when
 // the recursive residual meets the tolerance or has dropped two decades
 // since the last replacement, and at the end; x is brought up to date (flush)
-// before the last two.  Per iteration 116 bytes per row for a seven-point
+// before the last two.  The solver works on s b and s x, s a power of two
+// that brings max |b| near 1 when it is far from 1 (rhs_scale), so that the
+// FP32 vectors and products neither under- nor overflow (x is multiplied at
+// the start and the end: exact).  Per iteration 116 bytes per row for a seven-point
 // matrix (values and columns 56, gathers and vectors 60), against the
 // matrix-free passes' 32.  As three kernels (p a pass of its own) an iteration
 // of 8000 rows took 21 us and of 1.1 million rows 38.0; two kernels 17.5 and
@@ -177,28 +180,37 @@ __global__ void __launch_bounds__(kSellThreads)
     }
 }
 
-// the pending x += alpha p, before x is used (p in the pairs)
+// the pending x += alpha p, before x is used (p in the pairs); FINAL: and x back in the caller's units
+template <bool FINAL>
 __global__ void __launch_bounds__(kSellThreads)
     sell_flush_kernel(int64_t n, double *__restrict__ x, const float2 *__restrict__ zp, const SolveState *st) {
-    if (!st->pending) return;
+    const double unit = FINAL ? 1.0 / st->scale : 1.0;
+    const bool pending = st->pending != 0;
+    if (!pending && unit == 1.0) return;
     const double alpha = st->alpha;
-    for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSellThreads)
-        x[i] = fma(alpha, (double)zp[i].y, x[i]);
+    for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSellThreads) {
+        const double v = pending ? fma(alpha, (double)zp[i].y, x[i]) : x[i];
+        x[i] = FINAL ? v * unit : v;
+    }
 }
 
-// r = b - A x with FP64 products and sums (x gathered in FP64); r stored as
-// FP32.  INIT: sums r.r, r.z, b.b -> start state; REPLACE: r.r, r.z -> the
-// replacement's decisions (only when one was requested); TRUE: r.r -> the
-// reported true residual.
-template <int MODE>
+// r = s (b - A x) with FP64 products and sums (x gathered in FP64), s the power of two of rhs_scale (in the
+// loop, REPLACE, x holds s x); r stored as FP32.  INIT: sums r.r, r.z, b.b -> start state; REPLACE: r.r, r.z -> the replacement's
+// decisions (only when one was requested); TRUE: r.r -> the reported true residual.  INIT runs twice:
+// the first takes s = 1 and the largest |b|, the second (AGAIN) runs only if that asks for another s.
+template <int MODE, bool AGAIN>
 __global__ void __launch_bounds__(kSellThreads)
     sell_residual_kernel(const SellDev A, const double *__restrict__ b, const double *__restrict__ x,
                          float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
                          cudaGraphConditionalHandle cond, int use_cond) {
     if (MODE == RES_REPLACE && (!st->replace || st->done)) return;
     if (MODE == RES_TRUE && st->true_known) return;
+    constexpr bool FIRST = MODE == RES_INIT && !AGAIN;
+    const double sc = FIRST ? 1.0 : st->scale;
+    if (AGAIN && sc == 1.0) return;
     constexpr int NV = res64_nv<MODE>();
     double s[3] = {0.0, 0.0, 0.0};
+    unsigned long long mb = 0;
     for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < A.n;
          i += (int64_t)gridDim.x * kSellThreads) {
         int64_t e;
@@ -206,8 +218,13 @@ __global__ void __launch_bounds__(kSellThreads)
         sell_row(A, i, e, w);
         double ax = 0.0;
         for (int j = 0; j < w; ++j, e += kSell) ax = fma((double)__ldg(A.val + e), __ldg(x + __ldg(A.col + e)), ax);
-        const double bi = __ldg(b + i);
-        const double ri = bi - ax;
+        const double bl = __ldg(b + i);
+        if (FIRST) {
+            const unsigned long long u = (unsigned long long)__double_as_longlong(bl) & ~(1ull << 63);
+            mb = u > mb ? u : mb;
+        }
+        const double bi = sc * bl;
+        const double ri = bi - (MODE == RES_REPLACE ? ax : sc * ax);
         if (MODE == RES_TRUE) {
             s[0] = fma(ri, ri, s[0]);
         } else {
@@ -220,6 +237,19 @@ __global__ void __launch_bounds__(kSellThreads)
             s[1] = fma(ri, zi, s[1]);
             s[2] = fma(bi, bi, s[2]);
         }
+    }
+    if (FIRST) {
+        __shared__ unsigned long long smax;
+        if (threadIdx.x == 0) smax = 0;
+        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o);
+            mb = t > mb ? t : mb;
+        }
+        if ((threadIdx.x & 31) == 0) atomicMax(&smax, mb);
+        __syncthreads();
+        if (threadIdx.x == 0) atomicMax(&st->rhs_bits, smax);  // before this block's partial sums count
     }
     __shared__ double red[kSellThreads / 32][3];
 #pragma unroll
@@ -237,6 +267,7 @@ __global__ void __launch_bounds__(kSellThreads)
     }
     if (!grid_sum_last<NV, kSellThreads>(part, partials, &st->ticket[4 + MODE], tot) || threadIdx.x != 0) return;
     res64_finish<MODE>(st, tot, 1.0);
+    if (FIRST) st->scale = rhs_scale(__ldcg(&st->rhs_bits));
     if (MODE != RES_TRUE && use_cond) cudaGraphSetConditional(cond, st->done ? 0u : 1u);
 }
 
@@ -247,11 +278,12 @@ __global__ void sell_reset_kernel(SolveState *st, double tol, int maxit) {
     st->status = GBPCG_NOT_CONVERGED;
 }
 
-// x = 0 when b = 0 (the start state marks it)
-__global__ void __launch_bounds__(kSellThreads) sell_zero_x_kernel(int64_t n, double *x, const SolveState *st) {
-    if (!st->zero_x) return;
+// x = 0 when b = 0 (the start state marks it), else x in the solve's units
+__global__ void __launch_bounds__(kSellThreads) sell_start_x_kernel(int64_t n, double *x, const SolveState *st) {
+    const double sc = st->zero_x ? 0.0 : st->scale;
+    if (sc == 1.0) return;
     for (int64_t i = (int64_t)blockIdx.x * kSellThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSellThreads)
-        x[i] = 0.0;
+        x[i] = sc == 0.0 ? 0.0 : sc * x[i];
 }
 
 // ------------------------------------------------------------- assembly --
@@ -383,15 +415,19 @@ struct SellPlan {
     cudaGraphConditionalHandle cond = 0, cond_rep = 0;
     int use_cond = 0;
 
-    template <int MODE>
+    template <int MODE, bool AGAIN = false>
     void residual(cudaStream_t s) {
-        sell_residual_kernel<MODE><<<grid, kSellThreads, 0, s>>>(A, b, x, r, zp, st, partials, cond, use_cond);
+        sell_residual_kernel<MODE, AGAIN><<<grid, kSellThreads, 0, s>>>(A, b, x, r, zp, st, partials, cond, use_cond);
     }
-    void flush(cudaStream_t s) { sell_flush_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, zp, st); }
+    template <bool FINAL = false>
+    void flush(cudaStream_t s) {
+        sell_flush_kernel<FINAL><<<grid, kSellThreads, 0, s>>>(A.n, x, zp, st);
+    }
     void setup(cudaStream_t s) {
         sell_reset_kernel<<<1, 1, 0, s>>>(st, tol, maxit);
         residual<RES_INIT>(s);
-        sell_zero_x_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, st);
+        residual<RES_INIT, true>(s);
+        sell_start_x_kernel<<<grid, kSellThreads, 0, s>>>(A.n, x, st);
     }
     void body(cudaStream_t s) {
         sell_spmv_dot_kernel<<<grid, kSellThreads, 0, s>>>(A, zp, p, q, x, st, partials);
@@ -402,7 +438,7 @@ struct SellPlan {
         residual<RES_REPLACE>(s);
     }
     void finish(cudaStream_t s) {
-        flush(s);
+        flush<true>(s);
         residual<RES_TRUE>(s);
     }
 };
