@@ -557,13 +557,13 @@ __device__ __forceinline__ void mg_restrict_warp(const MgStep &a, unsigned wseg,
                                  });
 }
 
-// One warp's post-smoothing of the planes [k0, k1) of its segments; returns
-// its points' sum of f.out.
-template <int V, int WK>
-__device__ __forceinline__ float mg_post_warp(const MgStep &a, unsigned wseg, int k0, int k1) {
+// One warp's post-smoothing of the planes [k0, k1) of its segments; DOT: its
+// points' f.out go into acc, compensated, for a thread may hold hundreds of
+// terms (215 at 256^3, more on larger grids).
+template <int V, int WK, bool DOT>
+__device__ __forceinline__ void mg_post_warp(const MgStep &a, unsigned wseg, int k0, int k1, KahanF &acc) {
     const MgSeg<V> s(a.L, wseg);
     float *out = a.L.w;
-    float acc = 0.f;
     mg_march<V, WK, I_POST>(a, a.L.f, a.L.od, 0.f, false, s, k0, k1,
                                 [&](int, int64_t cb, unsigned c, const float *av, const float *v, const float *f, const float *o) {
                                     float r[V];
@@ -575,10 +575,13 @@ __device__ __forceinline__ float mg_post_warp(const MgStep &a, unsigned wseg, in
                                     } else {
                                         *reinterpret_cast<float2 *>(out + cb + c) = make_float2(r[0], r[1]);
                                     }
+                                    if constexpr (DOT) {
+                                        float t = f[0] * r[0];
 #pragma unroll
-                                    for (int m = 0; m < V; ++m) acc = fmaf(f[m], r[m], acc);
+                                        for (int m = 1; m < V; ++m) t = fmaf(f[m], r[m], t);
+                                        acc.add(t);
+                                    }
                                 });
-    return acc;
 }
 
 // f_{l+1} = P^T (f - A u), u = (omega / D) f; 
@@ -616,9 +619,10 @@ __device__ __forceinline__ void mg_rz_finish(const MgDot &d, double rz) {
 template <int V, int WK, bool DOT>
 __global__ void __launch_bounds__(kMgThreads, mg_min_blocks(WK)) mg_post_kernel(const MgStep a, const MgDot d) {
     if (mg_stand_down(a.st)) return;
-    float acc[1] = {0.f};
-    mg_runs(a.L, V, a.L.nz, [&](unsigned wseg, int k0, int k1) { acc[0] += mg_post_warp<V, WK>(a, wseg, k0, k1); });
+    KahanF sum;
+    mg_runs(a.L, V, a.L.nz, [&](unsigned wseg, int k0, int k1) { mg_post_warp<V, WK, DOT>(a, wseg, k0, k1, sum); });
     if constexpr (DOT) {
+        const float acc[1] = {(float)sum.value()};
         double part[1], tot[1];
         block_sum<1, kMgThreads>(acc, part);
         if (grid_sum_last<1, kMgThreads>(part, d.partials, &d.st->ticket[1], tot) && threadIdx.x == 0)
