@@ -8,8 +8,8 @@
 // brick faces:
 //
 //   p = r + beta p           own points; halo points from the neighbours' r
-//   q = A p, sum p.q         -> grid sum -> alpha
-//   d += alpha p, r -= alpha q, sum r.r; face values of r to L2
+//   q = u A p, sum p.q       -> grid sum -> alpha      (u: a power of two, ResProb::unit)
+//   d += u alpha p, r -= alpha q, sum r.r; face values of r to L2
 //                            -> grid sum -> beta, convergence, replacement
 //
 // A grid sum is one hop: every CTA publishes its partial sum together with
@@ -140,7 +140,9 @@ struct Shared {
     float redf[kMaxWarps];
     Pair rr;            // r.r of the current residual
     float alpha, beta;
-    float slow_below;   // ||r||^2 at or below this: the FP64 tests of passb_finish decide
+    float dalpha;       // alpha of d: times ResProb::unit
+    float slow_below;   // ||r||^2 at or below this: the FP64 tests of passb_finish decide (fast_range)
+    float slow_base;    // the same while r.r is a plain pair
     int timeout;
 };
 
@@ -469,27 +471,69 @@ __device__ __forceinline__ bool grid_sum_pair(const Shared &sh, const ResProb &P
     return ok;
 }
 
-// The loop's scalars after an FP64 finish: FP32 pairs, and the bound above which no FP64 test of
-// passb_finish can trigger.  Thread 0.
+// The same sum in FP64, where the pairs' total is beyond their range: one thread of each CTA, for the
+// same seq, through the slots behind those the pairs use.
+__device__ __forceinline__ bool grid_sum_wide(const Shared &sh, const ResProb &P, int rank, unsigned seq, double &v) {
+    v = 0.0;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) v += (double)sh.redf[w];
+    if (P.G == 1) return true;
+    ulonglong2 *slots = P.slots + (size_t)(seq & 1u) * (kResMaxCtas * kResSlotVals) + (kResSlotVals - 1) * kResMaxCtas;
+    st_slot(slots + rank, (unsigned long long)__double_as_longlong(v), seq);
+    v = 0.0;
+    for (int j = 0; j < P.G; ++j) {
+        unsigned long long bits, tag;
+        uint32_t polls = 0;
+        do ld_slot(slots + j, bits, tag);
+        while (tag != seq && ++polls <= kSumPolls);
+        if (tag != seq) return false;
+        v += __longlong_as_double((long long)bits);
+    }
+    return true;
+}
+
+// Where r.r is no plain pair (it is then {0, 0}, and S.rz holds it), no half iteration is fast.
+__device__ __forceinline__ void fast_range(Shared &sh) {
+    sh.slow_below = pair_plain(sh.rr) ? sh.slow_base : INFINITY;
+    if (!pair_plain(sh.rr)) sh.rr = Pair{0.0f, 0.0f};
+}
+
+// The loop's scalars after an FP64 finish: FP32 pairs (r.r is S.rz where it is no plain pair), and the
+// bound above which no FP64 test of passb_finish can trigger.  Thread 0.
 __device__ __forceinline__ void loop_scalars(Shared &sh, bool saved_pair) {
     SolveState &S = sh.st;
     sh.rr = saved_pair ? pair_from((unsigned long long)__double_as_longlong(S.rzm)) : pair_of(S.rr);
     sh.beta = S.it == 0 ? 0.0f : (float)S.beta;
     const float t = __double2float_ru(fmax(S.tol2 * S.bb, kReplaceDrop2 * S.rr_rep));
-    sh.slow_below = fmaxf(t * 1.00001f, 1e-36f);
+    sh.slow_base = fmaxf(t * 1.00001f, 1e-36f);
+    fast_range(sh);
 }
 
 // The FP64 finish of a half iteration (thread 0), where the fast tests do not settle it.
-__device__ __noinline__ void res_finish(Shared &sh, int half, double v) {
+__device__ __noinline__ void res_finish(Shared &sh, const ResProb &P, int half, double v) {
     SolveState &S = sh.st;
-    S.rz = pair_value(sh.rr);
+    if (pair_plain(sh.rr)) S.rz = pair_value(sh.rr);
     if (half == 0) {
         passa_finish(&S, v, false);
         sh.alpha = (float)S.alpha;
+        sh.dalpha = sh.alpha * P.unit;
     } else {
         passb_finish(&S, S.it, v, v, false);
         S.pending = 0;            // (d is up to date already)
         sh.beta = (float)S.beta;  // (a replacement sets its own)
+    }
+}
+
+// The same where the sum is beyond the pairs' range.
+__device__ __noinline__ void res_finish_wide(Shared &sh, const ResProb &P, int rank, unsigned seq, int half) {
+    double v;
+    if (!grid_sum_wide(sh, P, rank, seq, v)) {
+        sh.timeout = 1;
+        return;
+    }
+    res_finish(sh, P, half, v);
+    if (half) {
+        sh.rr = Pair{0.0f, 0.0f};
+        fast_range(sh);
     }
 }
 
@@ -607,7 +651,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
     auto flush = [&]() {
         if (fresh) return;
         fresh = true;
-        const float a = pending ? sh.alpha : 0.0f;
+        const float a = pending ? sh.dalpha : 0.0f;
         pending = false;
         const double inv_s = 1.0 / rhs_scale(S.rhs_bits);
         const X is = (X)inv_s;
@@ -724,7 +768,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
     while (alive && !S.done && left-- > 0) {
         // ---- p_k = r_k + beta p_{k-1}: own points, then the halo from the neighbours' r ----
         {
-            const float beta = sh.beta, dalpha = pending ? sh.alpha : 0.0f;
+            const float beta = sh.beta, dalpha = pending ? sh.dalpha : 0.0f;
             pending = false;
             int pl = plane;
             asm volatile("" : "+r"(pl));
@@ -824,17 +868,25 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
                 Pair t;
                 const bool ok = grid_sum_pair(sh, P, rank, seq, t);
                 if (lane == 0) {
+                    const Pair rr = sh.rr;
                     if (!ok) {
                         sh.timeout = 1;
-                    } else if (half == 0 && pair_plain(t)) {
-                        sh.alpha = pair_div(sh.rr, t);
+                    } else if (half == 0 && pair_plain(t) && rr.s != 0.0f) {
+                        const float a = pair_div(rr, t);
+                        sh.alpha = a;
+                        sh.dalpha = a * P.unit;
                     } else if (half == 1 && t.s > sh.slow_below && pair_plain(t) && S.it + 1 < S.maxit) {
                         sh.beta = pair_div(t, sh.rr);
                         sh.rr = t;
                         S.it += 1;
+                    } else if (!pair_plain(t)) {
+                        res_finish_wide(sh, P, rank, seq, half);
                     } else {
-                        res_finish(sh, half, pair_value(t));
-                        sh.rr = half ? t : sh.rr;
+                        res_finish(sh, P, half, pair_value(t));
+                        if (half) {
+                            sh.rr = t;
+                            sh.slow_below = sh.slow_base;
+                        }
                     }
                     if (BATCH && half == 1 && rank == 0 && S.it % kProgressEvery == 0) atomicAdd(P.progress, 1u);
                 }
@@ -842,11 +894,12 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
                 // Meanwhile the other warps take d += alpha p and fetch the neighbours' faces: each CTA
                 // raises its flag once its own face values (stored before the barrier above) are visible.
                 if (DREG < MAXD && D > DREG && tid >= 64) {
-                    if (act) add_d(tid, p0, DREG, 1, alpha);
+                    const float dalpha = sh.dalpha;
+                    if (act) add_d(tid, p0, DREG, 1, dalpha);
                     const int nd = D - DREG;
                     for (int k = (tid >> 5) - 2; k < 2 * nd; k += NT / 32 - 2) {
                         const int t = k < nd ? lane : lane + 32;
-                        if (t < nact) add_d(t, ps + (k < nd ? ow0 : ow1), DREG + (k < nd ? k : k - nd), D, alpha);
+                        if (t < nact) add_d(t, ps + (k < nd ? ow0 : ow1), DREG + (k < nd ? k : k - nd), D, dalpha);
                     }
                 }
                 if (tid < 64 && P.G > 1) {
@@ -903,7 +956,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
         }
         // what the fast steps kept as pairs (a finish that ended the loop has set its own values)
         if (!S.done) {
-            S.rr = S.rz = pair_value(sh.rr);
+            if (pair_plain(sh.rr)) S.rr = S.rz = pair_value(sh.rr);
             S.beta = (double)sh.beta;
         }
         S.rzm = __longlong_as_double((long long)pair_bits(sh.rr));
@@ -913,7 +966,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
     __syncthreads();
 
     if (P.save && alive) {
-        const float a = pending ? sh.alpha : 0.0f;
+        const float a = pending ? sh.dalpha : 0.0f;
 #pragma unroll
         for (int i = 0; i < DREG; ++i)
             if (i < D && act) {
@@ -1118,7 +1171,13 @@ ResProb make_prob(const SolveCall &c, const ResPlan &p) {
     r.nx = g.nx; r.ny = g.ny; r.nz = g.nz; r.nxp = (g.nx + 3) & ~3;
     r.sx = p.sx; r.sy = p.sy; r.sz = p.sz; r.bx4 = p.bx4; r.by = p.by; r.bz = p.bz;
     r.zseg = p.zseg; r.depth = p.depth; r.dplanes = p.dplanes; r.cols = p.cols; r.G = p.G;
+    // the operator times a power of two (exact) that brings its diagonal below 1: p.q then has r.r's
+    // magnitude, and the FP32 sums the range they have in the passes
     r.op = make_op_const(g.nx, g.ny, g.nz);
+    int e = 0;
+    (void)std::frexp(r.op.d, &e);
+    r.unit = std::ldexp(1.0f, -e);
+    for (float *c : {&r.op.cx, &r.op.cy, &r.op.cz, &r.op.d}) *c *= r.unit;
     r.maxit = c.maxit; r.iters = 0x7fffffff;
     r.final_x = 1;
     auto cc = [](int m) { double h = 1.0 / (m + 1); return 1.0 / (h * h); };

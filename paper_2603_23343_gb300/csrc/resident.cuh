@@ -55,7 +55,8 @@ int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, cha
 struct ResProb {
     int nx, ny, nz, nxp;  // nxp: row pitch of zg and pg, nx rounded up to a multiple of 4
     int sx, sy, sz, bx4, by, bz, zseg, depth, cols, G, dplanes;
-    OpConst op;
+    OpConst op;  // times unit
+    float unit;  // a power of two
     int maxit, iters;           // iters: iterations this launch may take
     int resume, save, final_x;  // host-driven loop: state from / to the workspace; final x update
     double cx, cy, cz, tol;

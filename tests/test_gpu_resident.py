@@ -131,3 +131,20 @@ def test_batch_waits_for_longer_problems(gpu_lib):
         else:
             assert r["status"] == gpu_lib.NOT_CONVERGED and r["iters"] == maxit, r
     assert res[0]["time_ms"] > 2000.0  # long enough for the limit to matter
+
+
+@pytest.mark.parametrize("shape", [(32, 32, 32), (64, 64, 64), (3, 5, 9)])
+def test_sums_beyond_single_precision_range(gpu_lib, shape):
+    """An initial guess so far off that r.r exceeds FP32's largest number, though no thread's part does:
+    the grid sums are taken in FP64 there, and the iterations are those of the passes."""
+    cfgs = gpu_lib.tile_configs()
+    code = gpu_lib.tile_cfg_code(cfgs.index((32, 16, 4)), cfgs.index((32, 16, 4)))
+    b = torch.from_numpy(inputs.uniform_rhs(shape, 330, dtype=np.float64)).cuda()
+    x0 = torch.from_numpy(inputs.uniform_rhs(shape, 331, dtype=np.float64)).cuda()
+    r0 = float(gpu_lib.stencil_apply(x0).norm())
+    x0 *= np.sqrt(2e39 if min(shape) > 8 else 1e37) / r0
+    its = 12 if min(shape) > 8 else 4
+    (xr, r), (xp, p) = [gpu_lib.pcg_solve(b, x0.clone(), tol=1e-6, maxit=its, tile_cfg=c) for c in (0, code)]
+    assert r["status"] == p["status"] == gpu_lib.NOT_CONVERGED and r["iters"] == p["iters"] == its, (r, p)
+    assert abs(r["rel_res_recursive"] - p["rel_res_recursive"]) <= 1e-3 * p["rel_res_recursive"]
+    assert float((xr - xp).norm()) <= 1e-4 * float(xp.norm())
