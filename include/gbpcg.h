@@ -306,8 +306,9 @@ int gbpcg_pcg_solve(const gbpcg_grid *grid, const void *b, void *x, const gbpcg_
  * shapes, else 64x16.  Otherwise (block coefficients, or GBPCG_FLAG_BATCH_GRAPH) each
  * problem's whole solve is a branch of one CUDA graph with its own
  * device-driven loop, tiles per shape from the autotuner (with
- * GBPCG_FLAG_BATCH_GRAPH, grids that fit the chip are solved one after
- * another as gbpcg_pcg_solve would, bit for bit).
+ * GBPCG_FLAG_BATCH_GRAPH, grids that fit the chip are solved as
+ * gbpcg_pcg_solve would, bit for bit, side by side where they leave each
+ * other room).
  */
 int gbpcg_workspace_size_batched(int32_t nprob, const gbpcg_grid *grids, const gbpcg_opts *opts,
                                  size_t *bytes);

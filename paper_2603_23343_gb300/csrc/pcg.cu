@@ -586,13 +586,13 @@ static int persistent_batch(int nprob, const gbpcg_grid *grids, const void *cons
 
 // The problems of a batch that fit the chip, solved there (resident.cu): one launch for all that leave
 // room for others beside them (bitwise the same from run to run), and one launch each for the larger
-// ones and, with GBPCG_FLAG_BATCH_GRAPH, for all (bitwise the standalone solves).  `in_batch` and
+// ones.  `standalone` (GBPCG_FLAG_BATCH_GRAPH): all bitwise the standalone solves.  `in_batch` and
 // `alone` hold their numbers; fills their results.  kResNoRoom, and nothing solved, if the shared launch
 // is not to be had; `refused` gets the problems whose own launch is not.
 static int resident_batch(const std::vector<int> &in_batch, const std::vector<int> &alone, const gbpcg_grid *grids,
                           const void *const *b, void *const *x, const gbpcg_opts *opts, gbpcg_result *results, char *ws,
                           size_t region, const std::vector<WsLayout> &L, const std::vector<size_t> &off,
-                          cudaStream_t s, std::vector<int> *refused) {
+                          cudaStream_t s, bool standalone, std::vector<int> *refused) {
     const int nb = (int)in_batch.size(), n = nb + (int)alone.size();
     auto which = [&](int i) { return i < nb ? in_batch[i] : alone[i - nb]; };
     std::vector<SolveCall> calls(n);
@@ -610,9 +610,11 @@ static int resident_batch(const std::vector<int> &in_batch, const std::vector<in
     struct Ev { cudaEvent_t a, b; ~Ev() { cudaEventDestroy(a); cudaEventDestroy(b); } } guard{e0, e1};
     GB_CUDA(cudaEventRecord(e0, s));
     if (nb) {
-        if (int rc = resident_batch_launch(nb, calls.data(), states, ws + state_bytes, region - state_bytes,
-                                           opts->io_dtype, s))
-            return rc;
+        const int rc = standalone ? resident_standalone_launch(nb, calls.data(), states, ws + state_bytes,
+                                                               region - state_bytes, opts->io_dtype, s)
+                                  : resident_batch_launch(nb, calls.data(), states, ws + state_bytes,
+                                                          region - state_bytes, opts->io_dtype, s);
+        if (rc) return rc;
     }
     std::vector<char> ran(n, 1);
     for (int i = nb; i < n; ++i) {
@@ -952,19 +954,23 @@ int gbpcg_pcg_solve_batched(int32_t nprob, const gbpcg_grid *grids, const void *
     const bool graph = opts->flags & GBPCG_FLAG_BATCH_GRAPH;
     ResidentChoice choice;
     if (graph && !opts->tile_cfg && !(opts->flags & GBPCG_FLAG_AUTOTUNE)) {
-        ResPlan plan;  // bit for bit the standalone solves
-        for (int i = 0; i < nprob; ++i) (resident_fits(grids[i], &plan) ? choice.alone : choice.rest).push_back(i);
+        // bit for bit the standalone solves; side by side where two have room
+        for (int i = 0; i < nprob; ++i) {
+            ResPlan plan;
+            const bool fits = resident_fits(grids[i], &plan);
+            (!fits ? choice.rest : 2 * plan.G <= device_sm_count() ? choice.in_batch : choice.alone).push_back(i);
+        }
     } else if (!graph && !opts->tile_cfg) {
         choice = resident_choice(nprob, grids);
     }
     std::vector<int> &in_batch = choice.in_batch, &alone = choice.alone, &rest = choice.rest;
     if (!in_batch.empty() || !alone.empty()) {
         std::vector<int> refused;
-        int rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, &refused);
+        int rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, graph, &refused);
         if (rc == kResNoRoom) {  // the tables outgrew the batch's region, or too few SMs: one launch each
             alone.insert(alone.begin(), in_batch.begin(), in_batch.end());
             in_batch.clear();
-            rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, &refused);
+            rc = resident_batch(in_batch, alone, grids, b, x, opts, results, ws, region, L, off, s, false, &refused);
         }
         if (rc) return rc;
         for (int i : refused) alone.erase(std::find(alone.begin(), alone.end(), i));

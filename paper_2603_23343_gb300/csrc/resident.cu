@@ -1009,7 +1009,8 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const __grid_constant__
 // Many problems: CTA c works through list[first[c]] .. list[first[c + 1] - 1], each entry a problem
 // (low half) and a brick of it (high half).  Every CTA takes its problems in the same common order,
 // so the CTAs of the first unfinished problem all reach it and no two problems wait for one another.
-// Two CTAs of half the threads share an SM: one computes while the other waits for its grid sums.
+// Two CTAs of half the threads share an SM: one computes while the other waits for its grid sums.  (With
+// GBPCG_FLAG_BATCH_GRAPH, one CTA with the threads and bricks of a standalone solve.)
 struct ResSchedule {
     uint32_t first[2 * kResMaxCtas + 1];
 };
@@ -1040,7 +1041,7 @@ __device__ __forceinline__ bool batch_meet(const ResProb &P, int rank, Shared &s
 }
 
 template <int NT, int MAXD, bool QREG, int DREG, typename X>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NT, NT == kResThreads ? 1 : 2)
     resident_batch_kernel(const ResProb *probs, const uint32_t *list, const __grid_constant__ ResSchedule sched) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
@@ -1353,106 +1354,79 @@ ResidentChoice resident_choice(int n, const gbpcg_grid *grids) {
     return r;
 }
 
-int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes, int io,
-                          cudaStream_t s) {
-    const int sms = device_sm_count(), group = std::min(sms, kResMaxCtas), ctas = std::min(2 * sms, 2 * kResMaxCtas);
-    // Plans of each problem for a falling number of CTAs.  Fewer CTAs per problem waste less on the grid
-    // sums, more finish the longest ones sooner: of a few trade-offs (the most CTA time a problem may
-    // take over its cheapest plan) the one whose schedule ends first is taken.
-    struct Option { ResPlan p; double cycles; };
-    std::vector<std::vector<Option>> options(n);
-    for (int i = 0; i < n; ++i) {
-        const gbpcg_grid &g = *calls[i].g;
-        const double it = expected_iters(g);
-        for (int m = group;;) {
-            ResPlan p;
-            if (!find_plan(g.nx, g.ny, g.nz, batch_limits(m), &p)) break;
-            options[i].push_back({p, p.cycles * it});
-            if (p.G <= 1) break;
-            m = std::min(p.G - 1, p.G * 3 / 4);
-        }
-        if (options[i].empty()) return fail_arg("a problem of the batch does not fit the on-chip solver");
-    }
-    std::vector<int> order(n), pick(n), best_pick(n);
-    for (int i = 0; i < n; ++i) order[i] = i;
-    std::vector<uint32_t> best_list;
-    ResSchedule sched;
-    double best_end = 1e300;
-    for (double slack : {1.0, 1.1, 1.25, 1.5, 2.0, 3.0}) {
-        for (int i = 0; i < n; ++i) {
-            double least = 1e300;
-            for (const Option &o : options[i]) least = std::min(least, o.cycles * o.p.G);
-            pick[i] = -1;
-            for (int k = 0; k < (int)options[i].size(); ++k) {
-                const Option &o = options[i][k];
-                if (o.cycles * o.p.G <= slack * least &&
-                    (pick[i] < 0 || o.cycles < options[i][pick[i]].cycles)) pick[i] = k;
-            }
-        }
-        std::sort(order.begin(), order.end(), [&](int a, int b) {
-            const double ca = options[a][pick[a]].cycles, cb = options[b][pick[b]].cycles;
-            return ca != cb ? ca > cb : a < b;
+namespace {
+
+// A problem of a shared launch, by its number among the calls.
+struct Placed {
+    int i;
+    ResPlan p;
+    double cycles;  // estimated, of the whole solve
+};
+
+// Each problem in turn, the longest first, on the CTAs that are free first; the end of the last one.
+double place(std::vector<Placed> &probs, int ctas, std::vector<uint32_t> *list, ResSchedule *sched) {
+    std::sort(probs.begin(), probs.end(), [](const Placed &a, const Placed &b) {
+        return a.cycles != b.cycles ? a.cycles > b.cycles : a.i < b.i;
+    });
+    std::vector<std::vector<uint32_t>> lists(ctas);
+    std::vector<double> free_at(ctas, 0.0);
+    std::vector<int> by(ctas);
+    double end = 0.0;
+    for (const Placed &o : probs) {
+        for (int c = 0; c < ctas; ++c) by[c] = c;
+        std::partial_sort(by.begin(), by.begin() + o.p.G, by.end(), [&](int a, int b) {
+            return free_at[a] != free_at[b] ? free_at[a] < free_at[b] : a < b;
         });
-        // each problem in turn on the CTAs that are free first
-        std::vector<std::vector<uint32_t>> lists(ctas);
-        std::vector<double> free_at(ctas, 0.0);
-        std::vector<int> by(ctas);
-        double end = 0.0;
-        for (int i : order) {
-            const Option &o = options[i][pick[i]];
-            for (int c = 0; c < ctas; ++c) by[c] = c;
-            std::partial_sort(by.begin(), by.begin() + o.p.G, by.end(), [&](int a, int b) {
-                return free_at[a] != free_at[b] ? free_at[a] < free_at[b] : a < b;
-            });
-            const double t = free_at[by[o.p.G - 1]] + o.cycles;
-            for (int r = 0; r < o.p.G; ++r) {
-                free_at[by[r]] = t;
-                lists[by[r]].push_back((uint32_t)i | (uint32_t)r << 16);
-            }
-            end = std::max(end, t);
+        const double t = free_at[by[o.p.G - 1]] + o.cycles;
+        for (int r = 0; r < o.p.G; ++r) {
+            free_at[by[r]] = t;
+            lists[by[r]].push_back((uint32_t)o.i | (uint32_t)r << 16);
         }
-        if (end < best_end) {
-            best_end = end;
-            best_pick = pick;
-            best_list.clear();
-            for (int c = 0; c < ctas; ++c) {
-                sched.first[c] = (uint32_t)best_list.size();
-                best_list.insert(best_list.end(), lists[c].begin(), lists[c].end());
-            }
-            sched.first[ctas] = (uint32_t)best_list.size();
-        }
-        if (n > 8 * ctas) break;  // many problems: the schedule is even whatever the trade-off
+        end = std::max(end, t);
     }
+    list->clear();
+    for (int c = 0; c < ctas; ++c) {
+        sched->first[c] = (uint32_t)list->size();
+        list->insert(list->end(), lists[c].begin(), lists[c].end());
+    }
+    sched->first[ctas] = (uint32_t)list->size();
+    return end;
+}
+
+size_t tables_bytes(size_t n, size_t entries) {
+    return round256(256 + n * sizeof(ResProb) + entries * sizeof(uint32_t));
+}
+
+// One launch of `fn` over `ctas` CTAs of `threads`, working through `list`.  The tables (tables_bytes):
+// the progress word, the problems by their numbers (n of them), the list.
+int launch_placed(void *fn, int threads, int ctas, size_t smem_limit, const std::vector<Placed> &placed, int n,
+                  const std::vector<uint32_t> &list, const ResSchedule &sched, const SolveCall *calls,
+                  SolveState *states, char *tables, cudaStream_t s) {
     std::vector<ResProb> probs(n);
+    memset(static_cast<void *>(probs.data()), 0, (size_t)n * sizeof(ResProb));
     size_t smem = 0;
     char *progress = tables, *dprobs = progress + 256, *dlist = dprobs + (size_t)n * sizeof(ResProb);
-    if (256 + (size_t)n * sizeof(ResProb) + best_list.size() * sizeof(uint32_t) > table_bytes) return kResNoRoom;
-    for (int i = 0; i < n; ++i) {
-        const ResPlan &p = options[i][best_pick[i]].p;
-        probs[i] = make_prob(calls[i], p);
-        probs[i].st = states + i;
-        probs[i].progress = reinterpret_cast<unsigned *>(progress);
-        smem = std::max(smem, p.smem);
-        GB_CUDA(cudaMemsetAsync(probs[i].slots, 0, kResSlotBytes, s));
-        if (probs[i].inbox) GB_CUDA(cudaMemsetAsync(probs[i].inbox, 0, inbox_bytes(p.G), s));
+    for (const Placed &o : placed) {
+        ResProb &r = probs[o.i];
+        r = make_prob(calls[o.i], o.p);
+        r.st = states + o.i;
+        r.progress = reinterpret_cast<unsigned *>(progress);
+        smem = std::max(smem, o.p.smem);
+        GB_CUDA(cudaMemsetAsync(r.slots, 0, kResSlotBytes, s));
+        if (r.inbox) GB_CUDA(cudaMemsetAsync(r.inbox, 0, inbox_bytes(o.p.G), s));
     }
-    GB_CUDA(cudaMemsetAsync(states, 0, (size_t)n * sizeof(SolveState), s));
     GB_CUDA(cudaMemsetAsync(progress, 0, 256, s));
     // copies from pageable memory have left it when the calls return
     GB_CUDA(cudaMemcpyAsync(dprobs, probs.data(), (size_t)n * sizeof(ResProb), cudaMemcpyHostToDevice, s));
-    GB_CUDA(cudaMemcpyAsync(dlist, best_list.data(), best_list.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-    void *fn = io == GBPCG_F64
-                   ? reinterpret_cast<void *>(
-                         &resident_batch_kernel<kBatchThreads, kBuildDepth[kBatchBuild], true, kBuildDregs[kBatchBuild], double>)
-                   : reinterpret_cast<void *>(
-                         &resident_batch_kernel<kBatchThreads, kBuildDepth[kBatchBuild], true, kBuildDregs[kBatchBuild], float>);
-    GB_CUDA(allow_smem(fn, kBatchMaxSmem));
+    GB_CUDA(cudaMemcpyAsync(dlist, list.data(), list.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+    GB_CUDA(allow_smem(fn, smem_limit));
     const ResProb *ap = reinterpret_cast<const ResProb *>(dprobs);
     const uint32_t *al = reinterpret_cast<const uint32_t *>(dlist);
-    void *kargs[] = {&ap, &al, &sched};
+    ResSchedule arg = sched;
+    void *kargs[] = {&ap, &al, &arg};
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)ctas);
-    lc.blockDim = dim3(kBatchThreads);
+    lc.blockDim = dim3((unsigned)threads);
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1461,6 +1435,101 @@ int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, cha
     lc.attrs = attr;
     lc.numAttrs = 1;
     return cooperative(lc, fn, kargs);
+}
+
+template <typename X>
+void *batch_fn(int build) {
+    switch (build) {
+        case 0: return reinterpret_cast<void *>(&resident_batch_kernel<kResThreads, kBuildDepth[0], true, kBuildDregs[0], X>);
+        case 1: return reinterpret_cast<void *>(&resident_batch_kernel<kResThreads, kBuildDepth[1], true, kBuildDregs[1], X>);
+        default: return reinterpret_cast<void *>(&resident_batch_kernel<kResThreads, kBuildDepth[2], false, kBuildDregs[2], X>);
+    }
+}
+
+}  // namespace
+
+int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes, int io,
+                          cudaStream_t s) {
+    const int sms = device_sm_count(), group = std::min(sms, kResMaxCtas), ctas = std::min(2 * sms, 2 * kResMaxCtas);
+    // Plans of each problem for a falling number of CTAs.  Fewer CTAs per problem waste less on the grid
+    // sums, more finish the longest ones sooner: of a few trade-offs (the most CTA time a problem may
+    // take over its cheapest plan) the one whose schedule ends first is taken.
+    std::vector<std::vector<Placed>> options(n);
+    for (int i = 0; i < n; ++i) {
+        const gbpcg_grid &g = *calls[i].g;
+        const double it = expected_iters(g);
+        for (int m = group;;) {
+            ResPlan p;
+            if (!find_plan(g.nx, g.ny, g.nz, batch_limits(m), &p)) break;
+            options[i].push_back({i, p, p.cycles * it});
+            if (p.G <= 1) break;
+            m = std::min(p.G - 1, p.G * 3 / 4);
+        }
+        if (options[i].empty()) return fail_arg("a problem of the batch does not fit the on-chip solver");
+    }
+    std::vector<Placed> best;
+    std::vector<uint32_t> best_list, list;
+    ResSchedule best_sched, sched;
+    double best_end = 1e300;
+    for (double slack : {1.0, 1.1, 1.25, 1.5, 2.0, 3.0}) {
+        std::vector<Placed> pick(n);
+        for (int i = 0; i < n; ++i) {
+            double least = 1e300;
+            for (const Placed &o : options[i]) least = std::min(least, o.cycles * o.p.G);
+            const Placed *b = nullptr;
+            for (const Placed &o : options[i])
+                if (o.cycles * o.p.G <= slack * least && (!b || o.cycles < b->cycles)) b = &o;
+            pick[i] = *b;
+        }
+        const double end = place(pick, ctas, &list, &sched);
+        if (end < best_end) {
+            best_end = end;
+            best = pick;
+            best_list = list;
+            best_sched = sched;
+        }
+        if (n > 8 * ctas) break;  // many problems: the schedule is even whatever the trade-off
+    }
+    if (tables_bytes(n, best_list.size()) > table_bytes) return kResNoRoom;
+    GB_CUDA(cudaMemsetAsync(states, 0, (size_t)n * sizeof(SolveState), s));
+    void *fn = io == GBPCG_F64
+                   ? reinterpret_cast<void *>(
+                         &resident_batch_kernel<kBatchThreads, kBuildDepth[kBatchBuild], true, kBuildDregs[kBatchBuild], double>)
+                   : reinterpret_cast<void *>(
+                         &resident_batch_kernel<kBatchThreads, kBuildDepth[kBatchBuild], true, kBuildDregs[kBatchBuild], float>);
+    return launch_placed(fn, kBatchThreads, ctas, kBatchMaxSmem, best, n, best_list, best_sched, calls, states, tables, s);
+}
+
+int resident_standalone_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes,
+                               int io, cudaStream_t s) {
+    const int ctas = std::min(device_sm_count(), kResMaxCtas);
+    std::vector<Placed> placed[kBuilds];
+    std::vector<uint32_t> list[kBuilds];
+    ResSchedule sched[kBuilds];
+    for (int i = 0; i < n; ++i) {
+        ResPlan p;
+        if (!resident_fits(*calls[i].g, &p)) return fail_arg("a problem of the batch does not fit the on-chip solver");
+        placed[p.build].push_back({i, p, p.cycles * expected_iters(*calls[i].g)});
+    }
+    size_t need = 0;
+    for (int b = 0; b < kBuilds; ++b) {
+        if (placed[b].empty()) continue;
+        place(placed[b], ctas, &list[b], &sched[b]);
+        need += tables_bytes(n, list[b].size());
+    }
+    if (need > table_bytes) return kResNoRoom;
+    GB_CUDA(cudaMemsetAsync(states, 0, (size_t)n * sizeof(SolveState), s));
+    for (int b = 0, launched = 0; b < kBuilds; ++b) {
+        if (placed[b].empty()) continue;
+        void *fn = io == GBPCG_F64 ? batch_fn<double>(b) : batch_fn<float>(b);
+        const int rc = launch_placed(fn, kResThreads, ctas, kResMaxSmem, placed[b], n, list[b], sched[b], calls, states,
+                                     tables, s);
+        if (rc == kResNoRoom && launched) return fail_cuda(cudaErrorCooperativeLaunchTooLarge, "batch launch");
+        if (rc) return rc;
+        launched = 1;
+        tables += tables_bytes(n, list[b].size());
+    }
+    return GBPCG_OK;
 }
 
 }  // namespace gb

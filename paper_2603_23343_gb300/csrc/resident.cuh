@@ -52,6 +52,11 @@ ResidentChoice resident_choice(int n, const gbpcg_grid *grids);
 int resident_batch_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes, int io,
                           cudaStream_t s);
 
+// The same with the bricks and threads of the standalone solves, whose bits the results have; one launch
+// per build of the kernel, problems side by side where they leave each other room.
+int resident_standalone_launch(int n, const SolveCall *calls, SolveState *states, char *tables, size_t table_bytes,
+                               int io, cudaStream_t s);
+
 struct ResProb {
     int nx, ny, nz, nxp;  // nxp: row pitch of zg and pg, nx rounded up to a multiple of 4
     int sx, sy, sz, bx4, by, bz, zseg, depth, cols, G, dplanes;
