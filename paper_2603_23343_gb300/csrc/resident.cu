@@ -46,6 +46,7 @@ constexpr int kSlotsPerLane = (kResMaxCtas + 31) / 32;
 // A poll is an L2 round trip, about 0.7 us: under a second for the waits between CTAs that are in the
 // same problem, which are never apart by more than part of an iteration.
 constexpr uint32_t kSumPolls = 1u << 20;
+constexpr unsigned kResLaunchSums = 16;  // of a host-driven launch: at most two at the start, two per iteration, four after
 constexpr int kProgressEvery = 32;  // iterations of a batch's problem between two steps of its progress word
 
 __device__ __forceinline__ void st_slot(ulonglong2 *p, unsigned long long v, unsigned long long tag) {
@@ -590,7 +591,7 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
     res_setup(P, rank, ps, psize, tab);
 
     SolveState &S = sh.st;
-    unsigned seq = 0;
+    unsigned seq = P.seq0;
     float rr_[MAXD][4], qr[QREG ? MAXD : 1][4], dr[DREG ? DREG : 1][4];
     bool pending = false;  // the planes of d in registers lack the last alpha p
     auto clear_d = [&]() {
@@ -744,8 +745,8 @@ __device__ __forceinline__ void resident_solve(const ResProb &P, int rank, unsig
         for (int e = tid; e < nhalo; e += NT) {
             const int2 t = tab[e];
             if (t.x < 0) continue;
-            const int n = e < nvec ? 4 : 1;
-            for (int j = 0; j < n; ++j) ps[t.x + j] = __ldcg(P.pg + t.y + j);
+            if (e < nvec) *reinterpret_cast<float4 *>(ps + t.x) = __ldcg(reinterpret_cast<const float4 *>(P.pg + t.y));
+            else ps[t.x] = __ldcg(P.pg + t.y);
         }
     } else {
         if (tid == 0) {
@@ -1211,9 +1212,13 @@ int cooperative(const cudaLaunchConfig_t &lc, void *fn, void **kargs) {
     return GBPCG_OK;
 }
 
+void *single_fn(const ResPlan &p, int io) {
+    return io == GBPCG_F64 ? resident_fn<double>(p.build) : resident_fn<float>(p.build);
+}
+
+// One launch (after allow_smem).
 int launch_one(const ResProb &r, const ResPlan &p, int io, cudaStream_t s) {
-    void *fn = io == GBPCG_F64 ? resident_fn<double>(p.build) : resident_fn<float>(p.build);
-    GB_CUDA(allow_smem(fn, kResMaxSmem));
+    void *fn = single_fn(p, io);
     ResProb arg = r;
     void *kargs[] = {&arg};
     cudaLaunchConfig_t lc = {};
@@ -1263,6 +1268,7 @@ int resident_launch(const SolveCall &c, const ResPlan &plan, cudaStream_t s, Sol
     GB_CUDA(cudaMemsetAsync(c.ws + c.L.state, 0, c.L.partials + kResSlotBytes - c.L.state, s));
     if (st) r.st = st;
     if (r.inbox) GB_CUDA(cudaMemsetAsync(r.inbox, 0, inbox_bytes(r.G), s));
+    GB_CUDA(allow_smem(single_fn(plan, c.io), kResMaxSmem));
     return launch_one(r, plan, c.io, s);
 }
 
@@ -1273,8 +1279,11 @@ int resident_host_loop(const SolveCall &c, const ResPlan &plan, cudaStream_t s) 
     r.save = 1;
     r.iters = 0;
     int done = 0;
-    for (int i = 0;; ++i) {
-        GB_CUDA(cudaMemsetAsync(r.slots, 0, kResSlotBytes, s));
+    // what a launch does besides its iteration is most of the loop: the slots are cleared once, and each
+    // launch numbers its sums from where the one before cannot have come to
+    GB_CUDA(allow_smem(single_fn(plan, c.io), kResMaxSmem));
+    GB_CUDA(cudaMemsetAsync(r.slots, 0, kResSlotBytes, s));
+    for (int i = 0;; ++i, r.seq0 += kResLaunchSums) {
         if (int rc = launch_one(r, plan, c.io, s)) return rc;
         GB_CUDA(cudaMemcpyAsync(&done, &r.st->done, sizeof(int), cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaStreamSynchronize(s));
@@ -1286,7 +1295,7 @@ int resident_host_loop(const SolveCall &c, const ResPlan &plan, cudaStream_t s) 
     r.iters = 0;
     r.save = 0;
     r.final_x = 1;
-    GB_CUDA(cudaMemsetAsync(r.slots, 0, kResSlotBytes, s));
+    r.seq0 += kResLaunchSums;
     return launch_one(r, plan, c.io, s);
 }
 

@@ -64,6 +64,7 @@ struct ResProb {
     float unit;  // a power of two
     int maxit, iters;           // iters: iterations this launch may take
     int resume, save, final_x;  // host-driven loop: state from / to the workspace; final x update
+    unsigned seq0;              // number of the last grid sum before this launch's
     double cx, cy, cz, tol;
     const void *b;
     void *x;
