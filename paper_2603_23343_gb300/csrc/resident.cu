@@ -1319,29 +1319,37 @@ double expected_iters(const gbpcg_grid &g) {
 // Which way a batch goes is decided by estimates of the two, measured with grids of 32 to 160 points per
 // axis on GB300.  On chip: a problem alone takes its plan's cycles; in the shared launch an iteration of
 // any takes about 14 us and G of the 2 x 152 CTAs.  Streaming kernel: 175 G points per second once the
-// GPU is full, a quarter of a microsecond per iteration for its scalar steps, and no problem's iteration
-// in less than 34 us.  So many large grids stream (24 of 48 to 160 points per axis: 65.6 against 78.8 ms
+// GPU is full, a quarter of a microsecond per iteration for its scalar steps, and a problem's own
+// iterations follow one another at 32 us and its points (one problem of 64^3: 31 us, 128^3 42, 192^3 73,
+// 256^3 126).  So many large grids stream (24 of 48 to 160 points per axis: 65.6 against 78.8 ms
 // on chip), a few large or many small ones do not (3: 14.2 against 7.0 ms; 200 of 32^3: 8.2 against 5.4;
-// 64 of 64^3: 22.6 against 19.9; 16 of 128^3: 63.3 against 57.0).
+// 64 of 64^3: 22.6 against 19.9; 16 of 128^3: 63.3 against 57.0).  Problems that do not fit stream either
+// way, and others beside them fill the gaps a long one leaves (160^3, 32^3, 64^3, 192^3 and 48^3: 42.0 ms
+// all streamed, 48.0 with the four on chip; 200^3 and 32 of 32^3: 48.9 against 46.6).
 constexpr int64_t kBatchPoints = 400000;  // larger ones leave too little of the chip to others
-constexpr double kSmMhz = 1900.0, kSharedUs = 14.0, kStreamedPerUs = 175e3, kStreamedStepUs = 0.25, kStreamedUs = 34.0;
+constexpr double kSmMhz = 1900.0, kSharedUs = 14.0, kStreamedPerUs = 175e3, kStreamedStepUs = 0.25, kStreamedUs = 32.0;
+constexpr double kMixMargin = 0.95;  // of the estimates, where part of the batch streams in any case
 
 ResidentChoice resident_choice(int n, const gbpcg_grid *grids) {
     ResidentChoice r;
     const double ctas = 2.0 * std::min(device_sm_count(), kResMaxCtas);
     bool aligned = true;  // the streaming kernel's condition on every grid
-    double alone = 0.0, shared = 0.0, shared_one = 0.0, streamed = 0.0, streamed_one = 0.0;
+    double alone = 0.0, shared = 0.0, shared_one = 0.0;
+    double streamed = 0.0, streamed_one = 0.0, rest = 0.0, rest_one = 0.0;  // of all problems, of those that do not fit
     for (int i = 0; i < n; ++i) {
         const gbpcg_grid &g = grids[i];
         const int64_t pts = (int64_t)g.nx * g.ny * g.nz;
         const double it = expected_iters(g);
         aligned = aligned && !g.k_block && g.nx % 4 == 0;
+        const double sum = it * (pts / kStreamedPerUs + kStreamedStepUs), one = it * (kStreamedUs + pts / kStreamedPerUs);
+        streamed += sum;
+        streamed_one = std::max(streamed_one, one);
         ResPlan p, q;
         if (!resident_fits(g, &p)) {
             r.rest.push_back(i);
-            continue;
-        }
-        if (pts <= kBatchPoints && find_plan(g.nx, g.ny, g.nz, batch_limits((int)(ctas / 2)), &q)) {
+            rest += sum;
+            rest_one = std::max(rest_one, one);
+        } else if (pts <= kBatchPoints && find_plan(g.nx, g.ny, g.nz, batch_limits((int)(ctas / 2)), &q)) {
             r.in_batch.push_back(i);
             shared += kSharedUs * it * std::ceil((double)pts / (4 * kBatchThreads * kBuildDepth[kBatchBuild])) / ctas;
             shared_one = std::max(shared_one, kSharedUs * it);
@@ -1349,14 +1357,13 @@ ResidentChoice resident_choice(int n, const gbpcg_grid *grids) {
             r.alone.push_back(i);
             alone += it * p.cycles / kSmMhz;
         }
-        streamed += it * (pts / kStreamedPerUs + kStreamedStepUs);
-        streamed_one = std::max(streamed_one, it * kStreamedUs);
     }
     if (r.in_batch.size() == 1) {  // nothing to share the chip with
         r.alone.push_back(r.in_batch[0]);
         r.in_batch.clear();
     }
-    if (aligned && alone + std::max(shared, shared_one) > std::max(streamed, streamed_one)) {
+    const double on_chip = alone + std::max(shared, shared_one) + std::max(rest, rest_one);
+    if (aligned && (r.rest.empty() ? 1.0 : kMixMargin) * on_chip > std::max(streamed, streamed_one)) {
         r = ResidentChoice{};
         for (int i = 0; i < n; ++i) r.rest.push_back(i);
     }

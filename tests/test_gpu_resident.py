@@ -148,3 +148,12 @@ def test_sums_beyond_single_precision_range(gpu_lib, shape):
     assert r["status"] == p["status"] == gpu_lib.NOT_CONVERGED and r["iters"] == p["iters"] == its, (r, p)
     assert abs(r["rel_res_recursive"] - p["rel_res_recursive"]) <= 1e-3 * p["rel_res_recursive"]
     assert float((xr - xp).norm()) <= 1e-4 * float(xp.norm())
+
+
+def test_batch_with_a_grid_that_does_not_fit_streams_as_one(gpu_lib):
+    """One grid must stream; the others fill the gaps it leaves, in the same launch, rather than going
+    before it on chip."""
+    shapes = [(160, 160, 160), (32, 32, 32), (64, 64, 64), (192, 192, 192), (48, 48, 48)]
+    bs = [torch.from_numpy(inputs.uniform_rhs(sh, 340 + i)).cuda() for i, sh in enumerate(shapes)]
+    _, res = gpu_lib.pcg_solve_batched(bs, tol=1e-3, maxit=3000)
+    assert all(r["status"] == gpu_lib.OK for r in res) and res[0]["pass_launches"][0] == 1
