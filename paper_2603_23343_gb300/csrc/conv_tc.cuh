@@ -1064,10 +1064,10 @@ __global__ void __launch_bounds__(128) wgrad_tc_kernel(const __grid_constant__ W
 // core's operand reads are next: 9 MMAs of 28 (M = 64, N = 48) shared-memory
 // wavefronts per 16 voxels.
 //
-// The steps (a plane of a column of rows) of the whole grid are split evenly
-// over the CTAs, to one step; each writes its sums to its own slot, added in a
-// fixed order.  The tensor core's accumulator truncates, so the error grows
-// with the length of a CTA's run (wgrad_zmarch_plan).
+// The steps (a plane of a column of rows) of the whole grid are split over the
+// CTAs; each writes its sums to its own slot, added in a fixed order.  The
+// tensor core's accumulator truncates, so the error grows with the length of a
+// CTA's run (wgrad_zmarch_plan).
 
 struct __align__(128) WgzMaps {
     CUtensorMap gy;  // (8, X, Co / 8, Y, Z) BF16, box (8, XB + 2, Co / 8, R + 2, 1)
@@ -1094,7 +1094,8 @@ __global__ void __launch_bounds__(128) wgrad_zmarch_kernel(const __grid_constant
     __shared__ int s_err;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c = (int)blockIdx.x, s0 = c * a.per_cta + min(c, a.extra), s1 = s0 + a.per_cta + (c < a.extra ? 1 : 0);
+    const int c = (int)blockIdx.x;
+    const int s0 = c * a.per_cta + min(c, a.extra), s1 = min(a.steps, s0 + a.per_cta + (c < a.extra ? 1 : 0));
     const uint32_t idesc = idesc_bf16_mn(a.co == 16 ? 64 : 128, a.ni);
     const uint32_t ncol = tmem_cols(9 * a.ni);
 

@@ -1124,12 +1124,21 @@ inline WgzPlan wgrad_zmarch_plan(int X, int Y, int Z, int ci, int co) {
     a.steps = a.nxb * a.nyb * Z;
     // about two CTAs per SM of a 152-SM part, one after the other (a sum of half the length in the tensor
     // core's accumulator, whose rounding grows with it), fixed so that workspace sizes do not depend on
-    // the device that asks.  Their steps differ by one at most: equal counts with what is left over in a
-    // last CTA made the runs up to 14 % longer and their error up to 10 % larger, for the same time.
+    // the device that asks.  Equal counts of steps, with what is left over in a last CTA, unless they make
+    // longer runs than equal counts of 128-voxel tiles would: then the steps are split over all CTAs, to one
+    // (equal counts made the runs up to 14 % longer than the tiles' and their error up to 10 % larger: for
+    // the same time at 64^3 and 128^3; 64 x 64 x 32, 16 -> 16 channels, equal counts 27.2 us, split 29.1).
     const int most = std::max(1, kWgTargetBlocks / 2 / (ci / a.ni));
-    p.S = std::min(a.steps, most);
-    a.per_cta = a.steps / p.S;
-    a.extra = a.steps % p.S;
+    const int64_t tiles = ((int64_t)X * Y * Z + 127) / 128;
+    a.per_cta = (a.steps + most - 1) / most;
+    if ((int64_t)a.per_cta * a.R * a.XB <= (tiles + most - 1) / most * 128) {
+        p.S = (a.steps + a.per_cta - 1) / a.per_cta;
+        a.extra = 0;
+    } else {
+        p.S = std::min(a.steps, most);
+        a.per_cta = a.steps / p.S;
+        a.extra = a.steps % p.S;
+    }
     p.smem = (size_t)a.ngy * a.gy_slot + (size_t)a.nx * a.x_slot + 2048;
     a.partials = nullptr;
     a.err = nullptr;
