@@ -194,12 +194,24 @@ __global__ void __launch_bounds__(kSellThreads)
     }
 }
 
-// r = s (b - A x) with FP64 products and sums (x gathered in FP64), s the power of two of rhs_scale (in the
+// The scale of a solve from max |b| and the norm of the first residual: a small b is not scaled up past
+// s ||r0|| = 2^40, so that the residual of an initial guess far off stays within FP32.
+__device__ __forceinline__ double sell_scale(unsigned long long rhs_bits, double r0) {
+    const double s = rhs_scale(rhs_bits);
+    if (s <= 1.0 || r0 == 0.0) return s;
+    int e = 0;
+    frexp(r0, &e);
+    return isfinite(r0) ? fmax(1.0, fmin(s, ldexp(1.0, 40 - e))) : 1.0;
+}
+
+// r = s (b - A x) with FP64 products and sums (x gathered in FP64), s the power of two of sell_scale (in the
 // loop, REPLACE, x holds s x); r stored as FP32.  INIT: sums r.r, r.z, b.b -> start state; REPLACE: r.r, r.z -> the replacement's
 // decisions (only when one was requested); TRUE: r.r -> the reported true residual.  INIT runs twice:
 // the first takes s = 1 and the largest |b|, the second (AGAIN) runs only if that asks for another s.
+// (Six CTAs per SM: left to itself the compiler takes 32 registers for REPLACE and spills, 1.5 % of a
+// solve with rows of 65 and 129 entries.)
 template <int MODE, bool AGAIN>
-__global__ void __launch_bounds__(kSellThreads)
+__global__ void __launch_bounds__(kSellThreads, 6)
     sell_residual_kernel(const SellDev A, const double *__restrict__ b, const double *__restrict__ x,
                          float *__restrict__ r, float2 *__restrict__ zp, SolveState *st, double *partials,
                          cudaGraphConditionalHandle cond, int use_cond) {
@@ -267,7 +279,7 @@ __global__ void __launch_bounds__(kSellThreads)
     }
     if (!grid_sum_last<NV, kSellThreads>(part, partials, &st->ticket[4 + MODE], tot) || threadIdx.x != 0) return;
     res64_finish<MODE>(st, tot, 1.0);
-    if (FIRST) st->scale = rhs_scale(__ldcg(&st->rhs_bits));
+    if (FIRST) st->scale = sell_scale(__ldcg(&st->rhs_bits), sqrt(tot[0]));
     if (MODE != RES_TRUE && use_cond) cudaGraphSetConditional(cond, st->done ? 0u : 1u);
 }
 

@@ -33,3 +33,19 @@ def test_any_scale_of_b(gpu_lib, guess):
         assert torch.equal(x, ref), k
     z, r = gpu_lib.sell_pcg_solve(m, torch.zeros_like(b), x0.clone() + 1.0, tol=tol)
     assert r["status"] == gpu_lib.OK and r["iters"] == 0 and not torch.any(z)
+
+
+def test_a_small_b_and_a_guess_far_off(gpu_lib):
+    """The residual of the guess, not b, bounds the scale: the iterations are those of the same guess with b
+    within range (whose share of the residual is 1e-14 and less either way)."""
+    shape = (13, 20, 31)
+    m = gpu_lib.sell_from_stencil(shape)
+    b = torch.from_numpy(inputs.uniform_rhs(shape, 93, dtype=np.float64)).cuda().ravel()
+    x0 = torch.from_numpy(inputs.uniform_rhs(shape, 94, dtype=np.float64)).cuda().ravel() * 1e13
+    xs = []
+    for s in (1.0, 2.0 ** -100, 2.0 ** -300):
+        x, r = gpu_lib.sell_pcg_solve(m, b * s, x0.clone(), tol=1e-6, maxit=20)
+        assert r["status"] == gpu_lib.NOT_CONVERGED and r["iters"] == 20, (s, r)
+        xs.append(x)
+    for x in xs[1:]:
+        assert float((x - xs[0]).norm()) <= 1e-4 * float(xs[0].norm())
