@@ -252,8 +252,9 @@ int gbpcg_workspace_size(const gbpcg_grid *grid, const gbpcg_opts *opts, size_t 
  * A constant-coefficient problem with nx >= 8 whose residual fits the GPU's
  * registers and whose search direction fits its shared memory (up to about
  * four million points) is solved in one cooperative launch that keeps both
- * there; others, and calls with tile_cfg or GBPCG_FLAG_PROFILE, run the data
- * passes from a device-driven CUDA graph.
+ * there; others, calls with tile_cfg or GBPCG_FLAG_PROFILE, and calls in a
+ * context that may not use enough SMs for that launch run the data passes
+ * from a device-driven CUDA graph.
  *
  * Mixed precision (opts->storage BF16 or F16, FP64 b and x): iterative
  * refinement.  Each outer step computes r = b - A x in FP64 and stops when

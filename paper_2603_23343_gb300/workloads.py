@@ -11,8 +11,8 @@ run through the C ABI on cuda:0:
       (seed 2): one cooperative kernel launch each
   python -m paper_2603_23343_gb300.workloads sell    --n N --reps R
       R Sliced-ELL products y = A x with the N^3 seven-point operator
-  python -m paper_2603_23343_gb300.workloads vcycle  --n N --reps R
-      R multigrid V-cycles (with the Galerkin set-up) on the N^3 Poisson operator
+  python -m paper_2603_23343_gb300.workloads vcycle  --n N --reps R [--coef poisson|lognormal]
+      R multigrid V-cycles (with the Galerkin set-up) on the N^3 operator
   python -m paper_2603_23343_gb300.workloads forward --n N --reps R
       R applications of the learned preconditioner (seeded initial weights) on the seeded
       lognormal problem at N^3
@@ -70,14 +70,15 @@ def sell(n, reps):
     print(f"sell spmv {n}^3 x{reps}: {m.nnz_stored} stored entries")
 
 
-def vcycle(n, reps):
+def vcycle(n, reps, coef):
     r = torch.from_numpy(inputs.uniform_rhs((n, n, n), 3)).cuda()
-    ws = binding.mg_workspace(r.shape)
+    k = learned.problem((n, n, n), 100)[0] if coef == "lognormal" else None
+    ws = binding.mg_workspace(r.shape, k)
     z = torch.empty_like(r)
     for _ in range(reps):
-        _, levels = binding.mg_vcycle(r, z, workspace=ws)
+        _, levels = binding.mg_vcycle(r, z, k_block=k, workspace=ws)
     torch.cuda.synchronize()
-    print(f"vcycle {n}^3 x{reps}: {levels} levels")
+    print(f"vcycle {n}^3 {coef} x{reps}: {levels} levels")
 
 
 def forward(n, reps):
@@ -112,12 +113,14 @@ def main(argv=None):
     ap.add_argument("--n", type=int, default=128)
     ap.add_argument("--reps", type=int, default=2)
     ap.add_argument("--storage", choices=["fp32", "fp16", "bf16"], default="fp32", help="passes only")
-    ap.add_argument("--coef", choices=["poisson", "lognormal"], default="poisson", help="passes only")
+    ap.add_argument("--coef", choices=["poisson", "lognormal"], default="poisson", help="passes and vcycle")
     a = ap.parse_args(argv)
     if not torch.cuda.is_available():
         raise SystemExit("the workloads need a CUDA GPU")
     if a.workload == "passes":
         passes(a.n, a.reps, a.storage, a.coef)
+    elif a.workload == "vcycle":
+        vcycle(a.n, a.reps, a.coef)
     else:
         globals()[a.workload](a.n, a.reps)
 
