@@ -18,13 +18,15 @@
 // item of any unfinished problem (an atomic counter in the problem's claim
 // word, whose upper half holds the phase's item count), preferring the problem it
 // worked on last; the CTA that completes a phase's last item adds the
-// problem's partial sums in item order (bitwise reproducible), takes the
+// problem's partial sums in item order, takes the
 // scalar step (alpha; beta, convergence, the replacement trigger) and opens
 // the problem's next phase.  So one problem's pass B runs while another's
 // pass A does, a finished problem drops out, and no CTA waits for work
 // while any is available.  The z depth of a pass item is chosen when its
 // phase opens: about two items per CTA over the unfinished problems, 4 to 32
-// planes.
+// planes.  (A batch whose problems finish together is bitwise reproducible; in
+// an uneven one the moment a problem drops out moves the depth of the others'
+// next phases, and with it the last bits of their sums from run to run.)
 //
 // Every wait is bounded: the grid barrier (a counter and a generation word)
 // after kBarrierPolls polls, a CTA finding no work after kIdlePolls tries;
